@@ -16,7 +16,6 @@ using qsd::cplx;
 using qsd::Targets;
 using qsd::group_base;
 using qsd::member_offset;
-using qsd::rotate8;
 
 int g_sms = 0;
 int sm_count()
@@ -77,43 +76,147 @@ __global__ void k_diag(typename cplx<R>::t *__restrict__ psi, uint64_t N, int k,
 
 // Product of T-type phases and CZ signs (Sec. 2, Sec. 3.5): amplitude i gets
 // e^{i pi m(i)/4}, m(i) = sum_q c_q i_q + 4 sum_a i_a popc(i & P_a) mod 8, with
-// P_a the CZ partners b > a of qubit a.  The index splits into low bits l
-// (below L) and high bits h.  The low part m_lo(l) (the c_q and partner pairs
-// inside the low bits) is a table built once per CTA in shared memory; every
-// chunk of 2^L amplitudes shares h, so m_hi(h) and the mask M_h of low qubits
-// whose partner set meets h an odd number of times are computed once per
-// chunk:  m(i) = m_lo(l) + m_hi(h) + 4 popc(l & M_h).  CZ-only ops cost no
-// floating-point work.
-constexpr int kPhaseLowBits = 14;
+// P_a the CZ partners b > a of qubit a.  The index splits into a column e (the
+// kPhaseRowBits lowest bits, one or two amplitudes per thread), a row r of the
+// chunk and the bits h above the chunk:
+//   m(i) = m0(e) + m1(r) + m_hi(h) + 4 popc(r & Mr_h) + 4 popc(e & (X_r ^ Me_h)),
+// m0 in a register for the whole launch, (m1, X_r) a table of at most 32 rows
+// in shared memory, m_hi(h) and the mask M_h (bits below the chunk's top whose
+// partner set meets h an odd number of times) formed once per chunk by each
+// warp, its lanes taking one term each.
+// Bound by HBM (amplitudes with m = 0 are not touched): four rows are in flight
+// per thread.  complex128: the factor e^{i pi/4} costs four FP64 operations and
+// the FP64 pipe gives two results a clock per SM, so a warp whose lanes are half
+// odd and half even pays for all of them.  m is odd exactly where the odd
+// coefficients' bits have odd parity; two rows are therefore paired so that
+// exactly one of a thread's two amplitudes is odd (the second row's column with
+// its lowest odd bit flipped when the rows' parities agree), and one rotation
+// serves both: 2 FP64 operations per amplitude, below the HBM time.
+// 27 qubits complex128, T-type and CZ terms: 1139 -> 680 us (94% of the HBM copy
+// rate); 28 qubits complex64: 996 -> 680 us; a phase op on 14 qubits: 53 -> 4 us
+// (chunks used to be 2^14 amplitudes with a table entry each, built by every
+// CTA; 83 gates on 16 qubits, half of them CZs: 1.79 -> 0.40 ms).
+constexpr int kPhaseThreads = 256;
+constexpr int kPhaseChunkRows = 32;          // most rows of a chunk
+template <typename R> constexpr int kPhaseVec = sizeof(R) == 4 ? 2 : 1;        // amplitudes per thread and row
+template <typename R> constexpr int kPhaseRowBits = sizeof(R) == 4 ? 9 : 8;    // log2(kPhaseThreads * kPhaseVec)
 
 template <typename R>
-__global__ void __launch_bounds__(256)
-k_phase(typename cplx<R>::t *__restrict__ psi, int n, const qs_phase_dev *__restrict__ ph, int n_act)
+__global__ void __launch_bounds__(kPhaseThreads, 4)
+k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev *__restrict__ ph, int n_act)
 {
     using C = typename cplx<R>::t;
-    __shared__ uint8_t tab[1 << kPhaseLowBits];
+    constexpr int VEC = kPhaseVec<R>, RB = kPhaseRowBits<R>;
     __shared__ uint64_t part[64];
     __shared__ int act[64];
-    const int L = n < kPhaseLowBits ? n : kPhaseLowBits;
-    const uint64_t c0 = ph->cmask[0], c1 = ph->cmask[1], c2 = ph->cmask[2];
+    __shared__ uint32_t row_x[kPhaseChunkRows];
+    __shared__ uint8_t row_m[kPhaseChunkRows];
+    const uint64_t cm[3] = {ph->cmask[0], ph->cmask[1], ph->cmask[2]};
     const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
-    for (int i = threadIdx.x; i < n_act; i += blockDim.x) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int i = tid; i < n_act; i += kPhaseThreads) {
         part[i] = terms[i].partners;
         act[i] = terms[i].a;
     }
     __syncthreads();
-    const uint64_t cm[3] = {c0, c1, c2};
-    for (int l = threadIdx.x; l < (1 << L); l += blockDim.x) tab[l] = qsd::phase_low((uint64_t)l, cm, act, part, n_act, L);
+    const int rb = min(n, RB);                       // a state below a row: its own bits
+    const int rows = 1 << (L - rb);
+    if (tid < rows) {
+        const uint64_t r = (uint64_t)tid << rb;
+        uint32_t x = 0;
+        for (int t = 0; t < n_act && act[t] < rb; t++) x |= ((uint32_t)__popcll(r & part[t]) & 1u) << act[t];
+        row_x[tid] = x;
+        row_m[tid] = qsd::phase_low(r, cm, act, part, n_act, L);
+    }
+    const uint32_t e = (uint32_t)(VEC * tid);
+    int m0[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; v++) m0[v] = qsd::phase_low(e + v, cm, act, part, n_act, rb);
+    // complex128: the lowest odd coefficient among the lanes' bits, and the
+    // column with that bit flipped
+    const uint32_t odd = VEC == 1 ? (uint32_t)cm[0] & 31u : 0u;
+    const uint32_t e2 = e ^ (odd & (0u - odd));
+    const int m02 = odd ? qsd::phase_low(e2, cm, act, part, n_act, rb) : 0;
+    const bool in = e < (1u << rb);
+    const bool any_odd = cm[0] != 0;
+    const bool pairs = odd != 0 && rows > 1 && rb == RB;
     __syncthreads();
     const uint64_t n_chunks = 1ULL << (n - L);
+    constexpr int kAhead = 4;
     for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
         const uint64_t h = ch << L;
-        uint64_t Mh;
-        const int mh = qsd::phase_high(h, cm, act, part, n_act, L, Mh);
-        C *base = psi + h;
-        for (int l = threadIdx.x; l < (1 << L); l += blockDim.x) {
-            const int m = (tab[l] + mh + 4 * __popcll((uint64_t)l & Mh)) & 7;
-            if (m) base[l] = rotate8<C, R>(base[l], m);
+        uint32_t Mh = 0, parh = 0;
+        for (int t = lane; t < n_act; t += 32) {
+            const int a = act[t];
+            const uint32_t o = (uint32_t)__popcll(h & part[t]) & 1u;
+            if (a >= L) parh ^= (uint32_t)(h >> a) & o;
+            else Mh |= o << a;
+        }
+        Mh = __reduce_or_sync(0xffffffffu, Mh);
+        parh = __reduce_xor_sync(0xffffffffu, parh & 1u);
+        const int mh = __popcll(h & cm[0]) + 2 * __popcll(h & cm[1]) + 4 * (__popcll(h & cm[2]) + (int)parh);
+        const uint32_t Me = Mh & ((1u << rb) - 1u), Mr = Mh >> rb;
+        if (!in) continue;
+        for (int r = 0; r < rows; r += kAhead) {
+            int m[kAhead][VEC];
+            C v[kAhead][VEC];
+            C *p[kAhead];
+#pragma unroll
+            for (int j = 0; j < kAhead; j++) {
+                const int rj = r + j;
+                const bool ok = rj < rows;
+                const int mr = ok ? row_m[rj] + mh + 4 * __popc((uint32_t)rj & Mr) : 0;
+                const uint32_t X = ok ? row_x[rj] ^ Me : 0u;
+                // the second row of a pair: the column that makes exactly one of the two odd
+                bool other = false;
+                if (pairs && (j & 1)) other = ok && !((mr ^ m[j - 1][0] ^ m0[0]) & 1);
+                const uint32_t ej = other ? e2 : e;
+                p[j] = psi + h + ((uint64_t)rj << rb) + ej;
+#pragma unroll
+                for (int k = 0; k < VEC; k++)
+                    m[j][k] = ok ? ((other ? m02 : m0[k]) + mr + 4 * __popc((ej + k) & X)) & 7 : 0;
+            }
+#pragma unroll
+            for (int j = 0; j < kAhead; j++) {
+                if constexpr (VEC == 2) {
+                    if (m[j][0] | m[j][1]) {
+                        const float4 w = *reinterpret_cast<const float4 *>(p[j]);
+                        v[j][0] = make_float2(w.x, w.y);
+                        v[j][1] = make_float2(w.z, w.w);
+                    }
+                } else {
+                    v[j][0] = C{};
+                    if (m[j][0]) v[j][0] = *p[j];
+                }
+            }
+            if (pairs) {
+#pragma unroll
+                for (int j = 0; j < kAhead; j += 2) {
+                    const bool first = m[j][0] & 1;
+                    const C t = qsd::eighth_turn(first ? v[j][0] : v[j + 1][0]);
+                    if (first) v[j][0] = t;
+                    else v[j + 1][0] = t;
+                }
+            } else if (any_odd) {
+#pragma unroll
+                for (int j = 0; j < kAhead; j++)
+#pragma unroll
+                    for (int k = 0; k < VEC; k++)
+                        if (m[j][k] & 1) v[j][k] = qsd::eighth_turn(v[j][k]);
+            }
+#pragma unroll
+            for (int j = 0; j < kAhead; j++) {
+#pragma unroll
+                for (int k = 0; k < VEC; k++) {
+                    v[j][k] = qsd::quarter_turns<C>(v[j][k], m[j][k] >> 1);
+                }
+                if constexpr (VEC == 2) {
+                    if (m[j][0] | m[j][1])
+                        *reinterpret_cast<float4 *>(p[j]) = make_float4(v[j][0].x, v[j][0].y, v[j][1].x, v[j][1].y);
+                } else {
+                    if (m[j][0]) *p[j] = v[j][0];
+                }
+            }
         }
     }
 }
@@ -194,20 +297,26 @@ int qs_launch_diag(qs_state *s, const int *dev_qubits, int k, const void *dev_ta
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_diag launch: %s", cudaGetErrorString(e));
 }
 
+template <typename R>
+static void launch_phase_r(qs_state *s, const void *dev_phase, int n_act)
+{
+    // chunks of up to 32 rows, fewer rows where the chunks would not fill the GPU
+    const int rb = std::min(s->n, kPhaseRowBits<R>);
+    const uint64_t cap = (uint64_t)sm_count() * 4;
+    int L = std::min(s->n, rb + 5);
+    while (L > rb && (1ULL << (s->n - L)) < cap) L--;
+    const int grid = (int)std::min<uint64_t>(1ULL << (s->n - L), cap);
+    k_phase<R><<<grid, kPhaseThreads, 0, (cudaStream_t)s->stream>>>(
+        reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, (const qs_phase_dev *)dev_phase, n_act);
+}
+
 int qs_launch_phase(qs_state *s, const void *dev_phase, int n_act)
 {
     s->perm_invariant = false;
     int rc = qs_materialize(s);
     if (rc) return rc;
-    const int L = s->n < kPhaseLowBits ? s->n : kPhaseLowBits;
-    const uint64_t chunks = 1ULL << (s->n - L);
-    const int block = 256;
-    int grid = (int)std::min<uint64_t>(chunks, (uint64_t)sm_count() * 8);
-    cudaStream_t st = (cudaStream_t)s->stream;
-    if (s->dtype == QS_C128)
-        k_phase<double><<<grid, block, 0, st>>>((double2 *)s->amp, s->n, (const qs_phase_dev *)dev_phase, n_act);
-    else
-        k_phase<float><<<grid, block, 0, st>>>((float2 *)s->amp, s->n, (const qs_phase_dev *)dev_phase, n_act);
+    if (s->dtype == QS_C128) launch_phase_r<double>(s, dev_phase, n_act);
+    else launch_phase_r<float>(s, dev_phase, n_act);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_phase launch: %s", cudaGetErrorString(e));
 }

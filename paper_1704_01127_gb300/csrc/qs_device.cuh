@@ -92,22 +92,37 @@ __device__ __forceinline__ double flip(double x, bool f)
     return __longlong_as_double(__double_as_longlong(x) ^ (f ? (long long)0x8000000000000000ULL : 0LL));
 }
 
-template <typename C, typename R>
-__device__ __forceinline__ C rotate8(C a, int m)
+__device__ __forceinline__ float2 eighth_turn(float2 a)   // times e^{i pi / 4}
 {
-    if (m & 1) {
-        const R r = (R)0.70710678118654752440;
-        C b;
-        b.x = (a.x - a.y) * r;
-        b.y = (a.x + a.y) * r;
-        a = b;
-    }
-    const int q = (m >> 1) & 3;                  // i^q: 0 (x, y), 1 (-y, x), 2 (-x, -y), 3 (y, -x)
+    const float r = 0.70710678118654752440f;
+    return make_float2((a.x - a.y) * r, (a.x + a.y) * r);
+}
+// the FP64 form in volatile statements: the compiler otherwise computes it for
+// every amplitude and selects, and the FP64 pipe is the narrow one
+__device__ __forceinline__ double2 eighth_turn(double2 a)
+{
+    double2 b;
+    asm volatile("{\n\t.reg .f64 s, d;\n\tsub.rn.f64 d, %2, %3;\n\tadd.rn.f64 s, %2, %3;\n\t"
+                 "mul.rn.f64 %0, d, %4;\n\tmul.rn.f64 %1, s, %4;\n\t}"
+                 : "=d"(b.x), "=d"(b.y)
+                 : "d"(a.x), "d"(a.y), "d"(0.70710678118654752440));
+    return b;
+}
+template <typename C>
+__device__ __forceinline__ C quarter_turns(C a, int q)   // times i^q: 0 (x, y), 1 (-y, x), 2 (-x, -y), 3 (y, -x)
+{
+    q &= 3;
     const bool sw = q & 1;
     C o;
     o.x = flip(sw ? a.y : a.x, q == 1 || q == 2);
     o.y = flip(sw ? a.x : a.y, q >= 2);
     return o;
+}
+template <typename C, typename R>
+__device__ __forceinline__ C rotate8(C a, int m)
+{
+    if (m & 1) a = eighth_turn(a);
+    return quarter_turns<C>(a, m >> 1);
 }
 
 // Phase products (Sec. 2, Sec. 3.5): amplitude i gets e^{i pi m(i)/4},

@@ -1,0 +1,45 @@
+"""Diagonal sweeps at the edges of their tiling: states below a row, one row,
+several rows per chunk, chunks of 32 rows; odd coefficients on the lanes' bits,
+above them, on both and nowhere."""
+import numpy as np
+import pytest
+
+import paper_1704_01127_gb300.qs as qs
+from inputs import random_state, random_phase_poly
+from oracle import sim
+
+pytestmark = pytest.mark.gpu
+
+EPS = {qs.QS_C128: 2.0 ** -53, qs.QS_C64: 2.0 ** -24}
+
+
+def rounded(psi, dtype):
+    return psi.astype(np.complex64).astype(np.complex128) if dtype == qs.QS_C64 else psi
+
+
+@pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
+@pytest.mark.parametrize("odd", ["none", "lanes", "above", "both"])
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 10, 14, 19, 20, 23])
+def test_phase_rows_and_chunks(dtype, odd, n):
+    coeff, edges = random_phase_poly(n, 2 * n if n > 1 else 0, 31 * n)
+    coeff = np.asarray(coeff) // 2 * 2
+    if odd in ("lanes", "both"):
+        coeff[min(2, n - 1)] += 1
+        coeff[0] += 1
+    if odd in ("above", "both"):
+        coeff[n - 1] += 1
+        coeff[n // 2] += 1
+    psi = rounded(random_state(n, n), dtype)
+    ref = psi.copy()
+    sim.apply_phase(ref, coeff, edges)
+    h = qs.qs_alloc(n, dtype)
+    try:
+        qs.qs_set_amplitudes(h, psi)
+        qs.qs_apply_phase(h, coeff, edges)
+        out = qs.qs_get_amplitudes(h)
+    finally:
+        qs.qs_free(h)
+    # an odd factor: one rounded sum and one rounded product per component, and
+    # the rounding of sqrt(1/2); even ones are exact
+    bound = 8 * EPS[dtype] if odd != "none" else 4 * EPS[qs.QS_C128]
+    assert np.all(np.abs(out - ref) <= bound * np.abs(psi))
