@@ -52,32 +52,91 @@ k_dense(typename cplx<R>::t *__restrict__ psi, uint64_t n_groups, Targets t,
         qsd::dense_group<R, K, false>(psi + group_base<K>(g, t), t, Us);
 }
 
-// Table diagonal on up to QS_MAX_DIAG_K qubits: psi_i *= d[x(i)].
+// The diagonal sweeps split an index into a column (the kDiagRowBits lowest
+// bits, one amplitude of complex128 or two of complex64 per thread), a row of
+// its chunk and the bits above the chunk; a thread keeps four rows in flight.
+constexpr int kDiagThreads = 256;
+constexpr int kDiagAhead = 4;
+constexpr int kDiagChunkRows = 32;                                           // most rows of a chunk
+template <typename R> constexpr int kDiagVec = sizeof(R) == 4 ? 2 : 1;       // amplitudes per thread and row
+template <typename R> constexpr int kDiagRowBits = sizeof(R) == 4 ? 9 : 8;   // log2(kDiagThreads * kDiagVec)
+
+// Table diagonal on up to QS_MAX_DIAG_K qubits: psi_i *= d[x(i)], x(i) the
+// column's, the row's and the chunk's target bits OR-ed together, each formed
+// once per launch, per launch (shared memory) and per chunk.  complex64 is
+// bound by HBM (28 qubits: 837 -> 666 us, 95% of the copy rate, with four rows in
+// flight instead of one amplitude and its table look-up); complex128 by the
+// FP64 pipe (four operations an amplitude, 883 us at 27 qubits: 1022 -> 983 us).
 template <typename R>
-__global__ void k_diag(typename cplx<R>::t *__restrict__ psi, uint64_t N, int k, const int *__restrict__ qg,
-                       const R *__restrict__ dg)
+__global__ void __launch_bounds__(kDiagThreads, 4)
+k_diag(typename cplx<R>::t *__restrict__ psi, int n, int L, int k, const int *__restrict__ qg, const R *__restrict__ dg)
 {
     using C = typename cplx<R>::t;
+    constexpr int VEC = kDiagVec<R>, RB = kDiagRowBits<R>;
     __shared__ int q[QS_MAX_DIAG_K];
-    if (threadIdx.x < k) q[threadIdx.x] = qg[threadIdx.x];
-    __syncthreads();
+    __shared__ int row_x[kDiagChunkRows];
     const C *d = reinterpret_cast<const C *>(dg);
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
+    const int tid = threadIdx.x;
+    if (tid < k) q[tid] = qg[tid];
+    __syncthreads();
+    auto bits = [&](uint64_t i) {
         int x = 0;
         for (int j = 0; j < k; j++) x |= (int)((i >> q[j]) & 1) << j;
-        C m = __ldg(&d[x]);
-        C a = psi[i], o;
-        o.x = a.x * m.x - a.y * m.y;
-        o.y = a.x * m.y + a.y * m.x;
-        psi[i] = o;
+        return x;
+    };
+    const int rb = min(n, RB), rows = 1 << (L - rb);
+    if (tid < rows) row_x[tid] = bits((uint64_t)tid << rb);
+    const uint32_t e = (uint32_t)(VEC * tid);
+    const bool in = e < (1u << rb);
+    int xe[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; v++) xe[v] = bits(e + v);
+    __syncthreads();
+    if (!in) return;
+    const uint64_t n_chunks = 1ULL << (n - L);
+    for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
+        const uint64_t h = ch << L;
+        const int xh = bits(h);
+        for (int r = 0; r < rows; r += kDiagAhead) {
+            C v[kDiagAhead][VEC], m[kDiagAhead][VEC];
+#pragma unroll
+            for (int j = 0; j < kDiagAhead; j++) {
+                if (r + j >= rows) break;
+                const C *p = psi + h + ((uint64_t)(r + j) << rb) + e;
+                const int x = xh | row_x[r + j];
+                if constexpr (VEC == 2) {
+                    const float4 w = *reinterpret_cast<const float4 *>(p);
+                    v[j][0] = make_float2(w.x, w.y);
+                    v[j][1] = make_float2(w.z, w.w);
+                } else {
+                    v[j][0] = *p;
+                }
+#pragma unroll
+                for (int i = 0; i < VEC; i++) m[j][i] = __ldg(&d[x | xe[i]]);
+            }
+#pragma unroll
+            for (int j = 0; j < kDiagAhead; j++) {
+                if (r + j >= rows) break;
+                C *p = psi + h + ((uint64_t)(r + j) << rb) + e;
+                C o[VEC];
+#pragma unroll
+                for (int i = 0; i < VEC; i++) {
+                    o[i].x = v[j][i].x * m[j][i].x - v[j][i].y * m[j][i].y;
+                    o[i].y = v[j][i].x * m[j][i].y + v[j][i].y * m[j][i].x;
+                }
+                if constexpr (VEC == 2)
+                    *reinterpret_cast<float4 *>(p) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+                else
+                    *p = o[0];
+            }
+        }
     }
 }
 
 // Product of T-type phases and CZ signs (Sec. 2, Sec. 3.5): amplitude i gets
 // e^{i pi m(i)/4}, m(i) = sum_q c_q i_q + 4 sum_a i_a popc(i & P_a) mod 8, with
 // P_a the CZ partners b > a of qubit a.  The index splits into a column e (the
-// kPhaseRowBits lowest bits, one or two amplitudes per thread), a row r of the
+// kDiagRowBits lowest bits, one or two amplitudes per thread), a row r of the
 // chunk and the bits h above the chunk:
 //   m(i) = m0(e) + m1(r) + m_hi(h) + 4 popc(r & Mr_h) + 4 popc(e & (X_r ^ Me_h)),
 // m0 in a register for the whole launch, (m1, X_r) a table of at most 32 rows
@@ -96,25 +155,20 @@ __global__ void k_diag(typename cplx<R>::t *__restrict__ psi, uint64_t N, int k,
 // rate); 28 qubits complex64: 996 -> 680 us; a phase op on 14 qubits: 53 -> 4 us
 // (chunks used to be 2^14 amplitudes with a table entry each, built by every
 // CTA; 83 gates on 16 qubits, half of them CZs: 1.79 -> 0.40 ms).
-constexpr int kPhaseThreads = 256;
-constexpr int kPhaseChunkRows = 32;          // most rows of a chunk
-template <typename R> constexpr int kPhaseVec = sizeof(R) == 4 ? 2 : 1;        // amplitudes per thread and row
-template <typename R> constexpr int kPhaseRowBits = sizeof(R) == 4 ? 9 : 8;    // log2(kPhaseThreads * kPhaseVec)
-
 template <typename R>
-__global__ void __launch_bounds__(kPhaseThreads, 4)
+__global__ void __launch_bounds__(kDiagThreads, 4)
 k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev *__restrict__ ph, int n_act)
 {
     using C = typename cplx<R>::t;
-    constexpr int VEC = kPhaseVec<R>, RB = kPhaseRowBits<R>;
+    constexpr int VEC = kDiagVec<R>, RB = kDiagRowBits<R>;
     __shared__ uint64_t part[64];
     __shared__ int act[64];
-    __shared__ uint32_t row_x[kPhaseChunkRows];
-    __shared__ uint8_t row_m[kPhaseChunkRows];
+    __shared__ uint32_t row_x[kDiagChunkRows];
+    __shared__ uint8_t row_m[kDiagChunkRows];
     const uint64_t cm[3] = {ph->cmask[0], ph->cmask[1], ph->cmask[2]};
     const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
     const int tid = threadIdx.x, lane = tid & 31;
-    for (int i = tid; i < n_act; i += kPhaseThreads) {
+    for (int i = tid; i < n_act; i += kDiagThreads) {
         part[i] = terms[i].partners;
         act[i] = terms[i].a;
     }
@@ -142,7 +196,7 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
     const bool pairs = odd != 0 && rows > 1 && rb == RB;
     __syncthreads();
     const uint64_t n_chunks = 1ULL << (n - L);
-    constexpr int kAhead = 4;
+    constexpr int kAhead = kDiagAhead;
     for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
         const uint64_t h = ch << L;
         uint32_t Mh = 0, parh = 0;
@@ -280,34 +334,46 @@ int qs_launch_dense(qs_state *s, const int *sorted_qubits, int k, const void *de
                                : launch_dense_r<float>(s, sorted_qubits, k, dev_matrix);
 }
 
-int qs_launch_diag(qs_state *s, const int *dev_qubits, int k, const void *dev_table)
+// Chunk bits of a diagonal sweep: up to 32 rows, fewer where the chunks would
+// not fill the GPU; *grid: its blocks.
+template <typename R>
+static int diag_chunk(int n, int *grid)
 {
-    s->perm_invariant = false;
-    int rc = qs_materialize(s);
-    if (rc) return rc;
-    uint64_t N = 1ULL << s->n;
-    const int block = 256;
-    int grid = grid_for(N, block, 8);
-    cudaStream_t st = (cudaStream_t)s->stream;
-    if (s->dtype == QS_C128)
-        k_diag<double><<<grid, block, 0, st>>>((double2 *)s->amp, N, k, dev_qubits, (const double *)dev_table);
-    else
-        k_diag<float><<<grid, block, 0, st>>>((float2 *)s->amp, N, k, dev_qubits, (const float *)dev_table);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_diag launch: %s", cudaGetErrorString(e));
+    const int rb = std::min(n, kDiagRowBits<R>);
+    const uint64_t cap = (uint64_t)sm_count() * 4;
+    int L = std::min(n, rb + 5);
+    while (L > rb && (1ULL << (n - L)) < cap) L--;
+    *grid = (int)std::min<uint64_t>(1ULL << (n - L), cap);
+    return L;
+}
+
+template <typename R>
+static void launch_diag_r(qs_state *s, const int *dev_qubits, int k, const void *dev_table)
+{
+    int grid;
+    const int L = diag_chunk<R>(s->n, &grid);
+    k_diag<R><<<grid, kDiagThreads, 0, (cudaStream_t)s->stream>>>(
+        reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, k, dev_qubits, reinterpret_cast<const R *>(dev_table));
 }
 
 template <typename R>
 static void launch_phase_r(qs_state *s, const void *dev_phase, int n_act)
 {
-    // chunks of up to 32 rows, fewer rows where the chunks would not fill the GPU
-    const int rb = std::min(s->n, kPhaseRowBits<R>);
-    const uint64_t cap = (uint64_t)sm_count() * 4;
-    int L = std::min(s->n, rb + 5);
-    while (L > rb && (1ULL << (s->n - L)) < cap) L--;
-    const int grid = (int)std::min<uint64_t>(1ULL << (s->n - L), cap);
-    k_phase<R><<<grid, kPhaseThreads, 0, (cudaStream_t)s->stream>>>(
+    int grid;
+    const int L = diag_chunk<R>(s->n, &grid);
+    k_phase<R><<<grid, kDiagThreads, 0, (cudaStream_t)s->stream>>>(
         reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, (const qs_phase_dev *)dev_phase, n_act);
+}
+
+int qs_launch_diag(qs_state *s, const int *dev_qubits, int k, const void *dev_table)
+{
+    s->perm_invariant = false;
+    int rc = qs_materialize(s);
+    if (rc) return rc;
+    if (s->dtype == QS_C128) launch_diag_r<double>(s, dev_qubits, k, dev_table);
+    else launch_diag_r<float>(s, dev_qubits, k, dev_table);
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_diag launch: %s", cudaGetErrorString(e));
 }
 
 int qs_launch_phase(qs_state *s, const void *dev_phase, int n_act)

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import paper_1704_01127_gb300.qs as qs
-from inputs import random_state, random_phase_poly
+from inputs import random_diag, random_phase_poly, random_qubits, random_state
 from oracle import sim
 
 pytestmark = pytest.mark.gpu
@@ -43,3 +43,21 @@ def test_phase_rows_and_chunks(dtype, odd, n):
     # the rounding of sqrt(1/2); even ones are exact
     bound = 8 * EPS[dtype] if odd != "none" else 4 * EPS[qs.QS_C128]
     assert np.all(np.abs(out - ref) <= bound * np.abs(psi))
+
+
+@pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
+@pytest.mark.parametrize("n,k", [(1, 1), (2, 2), (8, 3), (9, 9), (10, 1), (14, 12), (19, 6), (20, 12), (23, 5)])
+def test_table_rows_and_chunks(dtype, n, k):
+    qubits, d = random_qubits(n, k, 5 * n + k), random_diag(k, k)
+    psi = rounded(random_state(n, n + 1), dtype)
+    ref = psi.copy()
+    sim.apply_diag(ref, qubits, d)
+    h = qs.qs_alloc(n, dtype)
+    try:
+        qs.qs_set_amplitudes(h, psi)
+        qs.qs_apply_diag(h, qubits, d)
+        out = qs.qs_get_amplitudes(h)
+    finally:
+        qs.qs_free(h)
+    # the table's rounding, one rounded product and one rounded sum per component
+    assert np.all(np.abs(out - ref) <= 8 * EPS[dtype] * np.abs(psi))
