@@ -157,10 +157,39 @@ __device__ __forceinline__ int phase_high(uint64_t h, const uint64_t *cm, const 
     return (mh + 4 * parh) & 7;
 }
 
+// fl(x^2) of a double, rounded to nearest even, from integer operations: the
+// FP64 unit gives two results a clock per SM, the integer units 64, so a pass
+// that also adds in FP64 runs the squares beside it.  x = m 2^(e - 1075), m the
+// 53-bit significand; m^2 has 105 or 106 bits (s = 0 or 1) and its top 53 are
+// kept: the round bit and the bits below it sit in x (bit 0 set when a dropped
+// word is not zero), whose carry out of 2^31 - 1 + lsb is the increment.  Squares
+// outside the normal range (and zeros, infinities, NaN) take the FP64 unit.
+__device__ __forceinline__ double sq_rn(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d) & 0x7FFFFFFFu, lo = (uint32_t)__double2loint(d);
+    const uint32_t e = hi >> 20;
+    if (e - 513u > 1020u) return __dmul_rn(d, d);
+    const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
+    const uint64_t ll = (uint64_t)lo * lo, lh = (uint64_t)lo * mh, hh = (uint64_t)mh * mh;
+    uint32_t L1, H0, H1;   // m^2 = H1:H0:L1:L0
+    const uint32_t lhl = (uint32_t)lh, lhh = (uint32_t)(lh >> 32);
+    asm("add.cc.u32 %0, %3, %4;\n\taddc.cc.u32 %1, %5, %6;\n\taddc.u32 %2, %7, 0;"
+        : "=r"(L1), "=r"(H0), "=r"(H1)
+        : "r"((uint32_t)(ll >> 32)), "r"(lhl << 1), "r"((uint32_t)hh), "r"(__funnelshift_l(lhl, lhh, 1)),
+          "r"((uint32_t)(hh >> 32)));
+    const uint32_t s = H1 >> 9, sh = 20u + s;
+    const uint32_t ql = __funnelshift_r(L1, H0, sh), qh = __funnelshift_r(H0, H1, sh);
+    const uint32_t x = (L1 << (32u - sh)) | ((uint32_t)ll != 0u ? 1u : 0u);
+    uint32_t rl, rh;
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %2, %3;\n\taddc.cc.u32 %0, %4, 0;\n\taddc.u32 %1, %5, %6;\n\t}"
+        : "=r"(rl), "=r"(rh)
+        : "r"(x), "r"(0x7FFFFFFFu + (ql & 1u)), "r"(ql), "r"(qh), "r"((2u * e - 1024u + s) << 20));
+    return __hiloint2double((int)rh, (int)rl);
+}
 // p = fl(fl(re^2) + fl(im^2)) in FP64 (no contraction into an FMA).
 __device__ __forceinline__ double prob(double2 a)
 {
-    return __dadd_rn(__dmul_rn(a.x, a.x), __dmul_rn(a.y, a.y));
+    return __dadd_rn(sq_rn(a.x), sq_rn(a.y));
 }
 // x^2 of a float as a double, exact: the 24-bit significand squared fits in
 // 48 bits, so the product is assembled from integer operations (the same value

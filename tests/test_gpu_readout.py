@@ -1,5 +1,6 @@
 """Results read out: amplitudes by index (more and fewer indices than one launch
-takes, none, one out of range, qubits moved to other bits)."""
+takes, none, one out of range, qubits moved to other bits) and complex128
+probabilities over the whole range of doubles."""
 import numpy as np
 import pytest
 
@@ -40,3 +41,26 @@ def test_gather_after_remapped_circuit():
     finally:
         qs.qs_free(h)
         qs.qs_schedule_free(sched)
+
+
+@pytest.mark.parametrize("n", [1, 2, 9, 13])
+def test_c128_probabilities_over_every_exponent(n):
+    """The squares are built from integers and rounded as FP64 products: bit for
+    bit numpy's, with ties, subnormals, overflow, signed zeros and infinities."""
+    g = np.random.default_rng(11 + n)
+    bits = g.integers(0, 1 << 64, size=2 << n, dtype=np.uint64)
+    bits[1::3] &= ~np.uint64((1 << 26) - 1)          # exact ties of the 53-bit result among them
+    bits[(bits >> np.uint64(52) & np.uint64(0x7FF)) == 0x7FF] &= np.uint64(0x800FFFFFFFFFFFFF)
+    special = np.array([0.0, -0.0, 5e-324, -1.0, 1.0, np.inf, 2.0 ** -511, 2.0 ** -512, 2.0 ** 511.5,
+                        1.7976931348623157e308, 1.0 + 2.0 ** -52, 1.5 + 2.0 ** -27])[:2 << n]
+    bits[:special.size] = special.view(np.uint64)
+    f = bits.view(np.float64)
+    with np.errstate(over="ignore", under="ignore"):
+        want = f[0::2] * f[0::2] + f[1::2] * f[1::2]
+    h = qs.qs_alloc(n, qs.QS_C128)
+    try:
+        qs.qs_set_amplitudes(h, f.view(np.complex128))
+        got = qs.qs_probabilities(h)
+    finally:
+        qs.qs_free(h)
+    assert np.array_equal(got.view(np.uint64), want.view(np.uint64))
