@@ -131,39 +131,76 @@ k_batch(const BatchCirc *__restrict__ circ, const int *__restrict__ order, int n
     }
 }
 
-// Per-circuit FP64 statistics: one CTA per circuit.
+__global__ void k_log_table(qsd::LogTable *t) { qsd::log_table_init(*t); }
+
+// Per-circuit FP64 statistics: a CTA per 2^kStatsBits amplitudes (circuit
+// blk[i].x, part blk[i].y), then a warp per circuit over its CTAs' sums.  Bound
+// by the FP64 pipe (about 12 operations an amplitude; 102 M amplitudes: 2.1 ms);
+// one CTA per circuit, with its own log table, left most SMs idle: 10.2 -> 2.0 ms.
+constexpr int kStatsBits = 15;
+
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_batch_stats(const BatchCirc *__restrict__ circ, const typename cplx<R>::t *__restrict__ amp, double *__restrict__ out)
+k_batch_stats(const BatchCirc *__restrict__ circ, const int2 *__restrict__ blk, const qsd::LogTable *__restrict__ table,
+              const typename cplx<R>::t *__restrict__ amp, double *__restrict__ part)
 {
-    __shared__ qsd::LogTable lt;
-    __shared__ double red[4][8];
-    static_assert(sizeof(qsd::LogTable) + sizeof(red) < 48 * 1024, "static shared memory");
-    qsd::log_table_init(lt);
+    using C2 = typename cplx<R>::t;
+    __shared__ __align__(16) qsd::LogTable lt;
+    __shared__ double red[3][8];
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(table);
+        uint4 *dst = reinterpret_cast<uint4 *>(&lt);
+        for (int i = threadIdx.x; i < (int)(sizeof(lt) / sizeof(uint4)); i += 256) dst[i] = src[i];
+    }
     __syncthreads();
-    const BatchCirc cc = circ[blockIdx.x];
-    const uint64_t N = 1ULL << cc.n;
-    const double Nd = (double)N;
-    double a[4] = {0, 0, 0, 0};
-    for (uint64_t i = threadIdx.x; i < N; i += blockDim.x) {
-        const double p = qsd::prob(amp[cc.amp_off + i]);
-        a[0] += p;
-        if (p >= 2.2250738585072014e-308) a[1] -= p * qsd::log_tab(lt, p);
-        a[3] = fma(p, p, a[3]);
+    const int2 at = blk[blockIdx.x];
+    const BatchCirc cc = circ[at.x];
+    const uint32_t N = 1u << min(cc.n, kStatsBits);
+    const C2 *psi = amp + cc.amp_off + ((uint64_t)at.y << kStatsBits);
+    double a[3] = {0, 0, 0};   // sum p, -sum p ln p, sum p^2
+    constexpr int kAhead = 4;
+    for (uint32_t i0 = threadIdx.x; i0 < N; i0 += 256 * kAhead) {
+        C2 v[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; k++) v[k] = i0 + 256u * k < N ? psi[i0 + 256u * k] : C2{};
+#pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            const double p = qsd::prob(v[k]);
+            a[0] += p;
+            // p of 2^-1022 or more (an integer compare: FP64 ones run on the FP64 pipe)
+            if ((uint32_t)__double2hiint(p) - 0x00100000u <= 0x7FE00000u) a[1] -= p * qsd::log_tab(lt, p);
+            a[2] = fma(p, p, a[2]);
+        }
     }
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
+    for (int j = 0; j < 3; j++) {
         double v = a[j];
         for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if ((threadIdx.x & 31) == 0) red[j][threadIdx.x >> 5] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
-        // sum p, entropy, mean of N p (= sum p), mean of (N p)^2 (= N sum p^2)
-        const int src = threadIdx.x == 2 ? 0 : threadIdx.x;
+    if (threadIdx.x < 3) {
         double v = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) v += red[src][w];
-        out[4 * blockIdx.x + threadIdx.x] = threadIdx.x == 3 ? v * Nd : v;
+        for (int w = 0; w < 8; w++) v += red[threadIdx.x][w];
+        part[3 * (size_t)blockIdx.x + threadIdx.x] = v;
+    }
+}
+
+// sum p, entropy, mean of N p (= sum p), mean of (N p)^2 (= N sum p^2)
+__global__ void __launch_bounds__(32)
+k_batch_stats_final(const BatchCirc *__restrict__ circ, const int *__restrict__ first, const double *__restrict__ part,
+                    double *__restrict__ out)
+{
+    const int c = blockIdx.x, b0 = first[c], b1 = first[c + 1];
+    double a[3] = {0, 0, 0};
+    for (int b = b0 + (int)threadIdx.x; b < b1; b += 32)
+        for (int j = 0; j < 3; j++) a[j] += part[3 * (size_t)b + j];
+    for (int j = 0; j < 3; j++)
+        for (int o = 16; o; o >>= 1) a[j] += __shfl_down_sync(0xffffffffu, a[j], o);
+    if (threadIdx.x == 0) {
+        out[4 * c] = out[4 * c + 2] = a[0];
+        out[4 * c + 1] = a[1];
+        out[4 * c + 3] = a[2] * (double)(1ULL << circ[c].n);
     }
 }
 
@@ -183,6 +220,9 @@ struct qs_batch {
     void *stream = nullptr;
     void *amp = nullptr;
     void *ops = nullptr, *circ = nullptr, *order = nullptr, *pool = nullptr, *stats = nullptr;
+    // statistics: (circuit, part) of every CTA, the first CTA of every circuit, their sums, the log table
+    void *sblk = nullptr, *sfirst = nullptr, *spart = nullptr, *slog = nullptr;
+    int n_sblk = 0;
     std::vector<int> nq;
     std::vector<uint64_t> amp_off;
     int cluster = 1, block = 256;
@@ -334,8 +374,25 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
         if (!rc) rc = upload(&b->circ, circ);
         if (!rc) rc = upload(&b->order, order);
         if (!rc) rc = upload(&b->pool, pool);
-        if (!rc && (e = cudaMalloc(&b->stats, sizeof(double) * 4 * n_circ)) != cudaSuccess)
+        std::vector<int2> sblk;
+        std::vector<int> sfirst;
+        for (int c = 0; c < n_circ; c++) {
+            sfirst.push_back((int)sblk.size());
+            const int parts = 1 << std::max(0, circ[c].n - kStatsBits);
+            for (int p = 0; p < parts; p++) sblk.push_back(make_int2(c, p));
+        }
+        sfirst.push_back((int)sblk.size());
+        b->n_sblk = (int)sblk.size();
+        if (!rc) rc = upload(&b->sblk, sblk);
+        if (!rc) rc = upload(&b->sfirst, sfirst);
+        if (!rc && ((e = cudaMalloc(&b->stats, sizeof(double) * 4 * n_circ)) != cudaSuccess ||
+                    (e = cudaMalloc(&b->spart, sizeof(double) * 3 * sblk.size())) != cudaSuccess ||
+                    (e = cudaMalloc(&b->slog, sizeof(qsd::LogTable))) != cudaSuccess))
             rc = qs_fail(QS_ENOMEM, "qs_batch_create: stats: %s", cudaGetErrorString(e));
+        if (!rc) {
+            k_log_table<<<1, 256, 0, (cudaStream_t)stream>>>((qsd::LogTable *)b->slog);
+            if ((e = cudaGetLastError()) != cudaSuccess) rc = qs_fail(QS_ECUDA, "qs_batch_create: %s", cudaGetErrorString(e));
+        }
         if (rc) {
             qs_batch_free(b);
             return rc;
@@ -351,7 +408,7 @@ extern "C" void qs_batch_free(qs_batch *b)
     if (b->stream) cudaStreamSynchronize((cudaStream_t)b->stream);
     else cudaDeviceSynchronize();
     if (b->exec) cudaGraphExecDestroy(b->exec);
-    for (void *p : {b->amp, b->ops, b->circ, b->order, b->pool, b->stats})
+    for (void *p : {b->amp, b->ops, b->circ, b->order, b->pool, b->stats, b->sblk, b->sfirst, b->spart, b->slog})
         if (p) cudaFree(p);
     delete b;
 }
@@ -424,12 +481,15 @@ extern "C" int qs_batch_stats(qs_batch *b, double *out)
     return qs_guard([&]() -> int {
         if (!b || !out) return qs_fail(QS_EINVAL, "qs_batch_stats: bad arguments");
         cudaStream_t st = (cudaStream_t)b->stream;
+        const BatchCirc *circ = (const BatchCirc *)b->circ;
+        const qsd::LogTable *log = (const qsd::LogTable *)b->slog;
         if (b->dtype == QS_C128)
-            k_batch_stats<double><<<b->n_circ, 256, 0, st>>>((const BatchCirc *)b->circ, (const double2 *)b->amp,
-                                                             (double *)b->stats);
+            k_batch_stats<double><<<b->n_sblk, 256, 0, st>>>(circ, (const int2 *)b->sblk, log, (const double2 *)b->amp,
+                                                             (double *)b->spart);
         else
-            k_batch_stats<float><<<b->n_circ, 256, 0, st>>>((const BatchCirc *)b->circ, (const float2 *)b->amp,
-                                                            (double *)b->stats);
+            k_batch_stats<float><<<b->n_sblk, 256, 0, st>>>(circ, (const int2 *)b->sblk, log, (const float2 *)b->amp,
+                                                            (double *)b->spart);
+        k_batch_stats_final<<<b->n_circ, 32, 0, st>>>(circ, (const int *)b->sfirst, (const double *)b->spart, (double *)b->stats);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, b->stats, sizeof(double) * 4 * b->n_circ, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
