@@ -284,19 +284,31 @@ __global__ void k_stats_partial(const C *__restrict__ psi, uint64_t N, double *_
     acc.partials<NSTAT>(part);
 }
 
+// The blocks' partial sums added up in a fixed order by one block (2432 of them:
+// 27 us by one warp, 8 us by 512 threads).
+constexpr int kFinalThreads = 512;
+
 template <int NSTAT>
-__global__ void k_stats_final(const double *__restrict__ part, int nblocks, double *__restrict__ out)
+__global__ void __launch_bounds__(kFinalThreads) k_stats_final(const double *__restrict__ part, int nblocks, double *__restrict__ out)
 {
-    // one warp; fixed order for reproducibility
+    __shared__ double red[NSTAT][kFinalThreads / 32];
     double acc[NSTAT];
 #pragma unroll
     for (int j = 0; j < NSTAT; j++) acc[j] = 0;
-    for (int b = threadIdx.x; b < nblocks; b += 32)
+    for (int b = threadIdx.x; b < nblocks; b += kFinalThreads)
 #pragma unroll
         for (int j = 0; j < NSTAT; j++) acc[j] += part[(size_t)b * NSTAT + j];
 #pragma unroll
     for (int j = 0; j < NSTAT; j++) {
         double v = acc[j];
+        for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) red[j][threadIdx.x >> 5] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+#pragma unroll
+    for (int j = 0; j < NSTAT; j++) {
+        double v = threadIdx.x < kFinalThreads / 32 ? red[j][threadIdx.x] : 0.0;
         for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if (threadIdx.x == 0) out[j] = v;
     }
@@ -431,27 +443,130 @@ __global__ void k_segment_sums_small(const T *__restrict__ src, uint64_t nseg, i
         out[seg] = tree_sum_serial(src, seg * (uint64_t)len, len);
 }
 
-// Q_0 = 0, Q_{s+1} = Q_s + T_s (one thread); R_{s,0} = Q_s, R_{s,j+1} = R_{s,j} + S_{sG+j}.
-__global__ void k_prefix_super(const double *__restrict__ T, uint64_t ns, double *__restrict__ Q)
+// Sequential sums c <- fl(c + p), p >= 0.  The order of the additions is part of
+// the draws' definition, but they need not run one after another: while c
+// stays in one binade with unit u in the last place, fl(c + p) = c + u r(p)
+// with r(p) = p / u rounded to an integer, whatever c is, unless p / u lies
+// exactly half-way (then the parity of c decides).  So a warp rounds 32 values
+// to units of c's last place, adds integers in any order, and takes the 32
+// additions one by one only where a value ties or the sum reaches the next
+// binade.  Bit for bit the sequential sums, without the FP64 pipe and without
+// its latency 32 times over.
+constexpr uint32_t kFull = 0xffffffffu;
+
+// r(p) for a sum with exponent field E >= 1; *slow: a tie, or p as large as c.
+__device__ __forceinline__ uint64_t chain_term(double p, int E, bool &slow)
 {
-    double q = 0.0;
-    for (uint64_t s = 0; s < ns; s++) {
-        Q[s] = q;
-        q = q + T[s];
+    const uint64_t b = (uint64_t)__double_as_longlong(p);
+    const int e = (int)(b >> 52);
+    const uint64_t f = b & 0xFFFFFFFFFFFFFULL, m = e ? f | (1ULL << 52) : f;
+    const int sh = E - max(e, 1);
+    if (sh >= 54) return 0;                       // below u / 4
+    if (sh <= 0) {
+        slow = slow || m != 0;                    // c + p leaves the binade (infinities and NaN too)
+        return 0;
+    }
+    const uint64_t t = m + (1ULL << (sh - 1));
+    slow = slow || (t << (64 - sh)) == 0;         // exactly half-way
+    return t >> sh;
+}
+
+// The 32 additions in lane order; *incl: the sum up to this lane's value.
+__device__ __forceinline__ double chain_slow(double c, double p, double &incl)
+{
+    const int lane = threadIdx.x & 31;
+    incl = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < 32; k++) {
+        c = c + __shfl_sync(kFull, p, k);
+        if (lane == k) incl = c;
+    }
+    return c;
+}
+
+// sum of v < 2^54 over the warp, in every lane (two 27-bit halves, 32 of which fit 32 bits)
+__device__ __forceinline__ uint64_t warp_sum54(uint64_t v)
+{
+    const uint32_t lo = __reduce_add_sync(kFull, (uint32_t)v & 0x7FFFFFFu);
+    const uint32_t hi = __reduce_add_sync(kFull, (uint32_t)(v >> 27));
+    return (uint64_t)lo + ((uint64_t)hi << 27);
+}
+
+// c after this warp's 32 values in lane order; *half: the sum after lane 15's.
+__device__ __forceinline__ double chain_add(double c, double p, double &half)
+{
+    const uint64_t cb = (uint64_t)__double_as_longlong(c);
+    const int E = (int)(cb >> 52);
+    bool slow = E == 0;
+    const uint64_t r = chain_term(p, E, slow);
+    const uint64_t s16 = warp_sum54((threadIdx.x & 31) < 16 ? r : 0), s32 = warp_sum54(r);
+    if (__any_sync(kFull, slow) || (int)((cb + s32) >> 52) != E) {
+        double incl;
+        const double end = chain_slow(c, p, incl);
+        half = __shfl_sync(kFull, incl, 15);
+        return end;
+    }
+    half = __longlong_as_double((long long)(cb + s16));
+    return __longlong_as_double((long long)(cb + s32));
+}
+
+// The same with *excl the sum before this lane's value.
+__device__ __forceinline__ double chain_scan(double c, double p, double &excl)
+{
+    const int lane = threadIdx.x & 31;
+    const uint64_t cb = (uint64_t)__double_as_longlong(c);
+    const int E = (int)(cb >> 52);
+    bool slow = E == 0;
+    const uint64_t r = chain_term(p, E, slow);
+    uint64_t v = r;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t w = __shfl_up_sync(kFull, v, o);
+        if (lane >= o) v += w;
+    }
+    const uint64_t all = __shfl_sync(kFull, v, 31);
+    // r < 2^53 each: 32 of them stay below 2^58
+    if (__any_sync(kFull, slow) || (int)((cb + all) >> 52) != E) {
+        double incl;
+        const double end = chain_slow(c, p, incl);
+        excl = __shfl_up_sync(kFull, incl, 1);
+        if (lane == 0) excl = c;
+        return end;
+    }
+    excl = __longlong_as_double((long long)(cb + v - r));
+    return __longlong_as_double((long long)(cb + all));
+}
+
+// One warp: out[i] = the sequential sum of v[0 .. i-1] on top of c0 (out[0] = c0).
+__device__ __forceinline__ void prefix_chain(const double *__restrict__ v, uint64_t n, double c0, double *__restrict__ out)
+{
+    const int lane = threadIdx.x & 31;
+    constexpr int kAhead = 8;
+    double c = c0;
+    for (uint64_t i0 = 0; i0 < n; i0 += 32 * kAhead) {
+        double x[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; k++) x[k] = i0 + 32 * k + lane < n ? v[i0 + 32 * k + lane] : 0.0;
+#pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            if (i0 + 32 * k >= n) break;
+            double excl;
+            c = chain_scan(c, x[k], excl);
+            if (i0 + 32 * k + lane < n) out[i0 + 32 * k + lane] = excl;
+        }
     }
 }
 
-__global__ void k_prefix_blocks(const double *__restrict__ S, const double *__restrict__ Q, uint64_t ns,
-                                uint64_t G, double *__restrict__ R)
+// Q_0 = 0, Q_{s+1} = Q_s + T_s (one warp).  R_{s,0} = Q_s (0 without Q),
+// R_{s,j+1} = R_{s,j} + S_{sG+j}, a warp per super-block.  One thread per chain,
+// 29 qubits (512 chains of 1024): 37 + 154 us, now 16 + 23 us.
+__global__ void k_prefix_super(const double *__restrict__ T, uint64_t ns, double *__restrict__ Q) { prefix_chain(T, ns, 0.0, Q); }
+
+__global__ void __launch_bounds__(128)
+k_prefix_blocks(const double *__restrict__ S, const double *__restrict__ Q, uint64_t ns, uint64_t G, double *__restrict__ R)
 {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += stride) {
-        double r = Q[s];
-        for (uint64_t j = 0; j < G; j++) {
-            R[s * G + j] = r;
-            r = r + S[s * G + j];
-        }
-    }
+    const uint64_t s = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s < ns) prefix_chain(S + s * G, G, Q ? Q[s] : 0.0, R + s * G);
 }
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t seed, uint64_t j)
@@ -493,92 +608,116 @@ __global__ void k_draw(const C *__restrict__ psi, const double *__restrict__ Q, 
     }
 }
 
-// ---- draws by binary search over stored running sums (blocks of 1024)
+// ---- draws by checkpoints of the running sums (blocks of 1024)
 //
-// The per-draw scan above adds the probabilities of one block to R_b one
-// after another until the sum passes u.  The same sums, in the same order,
-// can be formed once for every block: c_{b,x} = R_b + p_{bB} + ... + p_{bB+x}
-// (sequential FP64 additions).  They do not decrease (p >= 0 and rounding is
-// monotone), so the scan's answer, the first x with c_{b,x} > u (B - 1 when
-// there is none), is found by binary search: bit for bit the same outcome.
+// The per-draw scan above adds the probabilities of one block to R_b one after
+// another until the sum passes u.  The sums c_{b,x} = R_b + p_{bB} + ... +
+// p_{bB+x}, in that order, are the same for every draw of the block and do not
+// decrease (p >= 0 and rounding is monotone), so each block that some draw
+// falls into is summed once, the sum kept after every kCkRun values, and a draw
+// then finds its run among the block's checkpoints and adds up that run alone:
+// bit for bit the scan's outcome.
+//   k_locate      block of every draw; with few draws for the number of blocks,
+//                 the list of the blocks that were hit (slot[b]: b's place in it)
+//   k_checkpoints the sums, a warp per block
+//   k_draw_run    the draws
+// 27 qubits complex64, 10^6 draws: 6.26 ms (a scan per draw) -> 0.94 ms; 29
+// qubits, 4096 draws: 441 -> 50 us.  complex128 stored every probability and
+// every running sum before (N doubles of scratch).
+constexpr int kCkRun = 16;
+constexpr int kCks = 1024 / kCkRun;
 
-// Block sums of 1024 probabilities as k_segment_sums<C, 32> forms them, and the
-// probabilities themselves stored (p[i] = prob(psi[i])).
-template <typename C>
-__global__ void k_block_sums_store(const C *__restrict__ psi, uint64_t nseg, double *__restrict__ out,
-                                   double *__restrict__ p)
+__global__ void k_locate(const double *__restrict__ Q, const double *__restrict__ R, uint64_t ns, uint64_t G, uint64_t seed,
+                         int64_t m, uint32_t *__restrict__ blk, uint32_t *__restrict__ slot, uint32_t *__restrict__ list,
+                         uint32_t *__restrict__ n_list)
 {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
-    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t seg = warp; seg < nseg; seg += nwarps) {
-        const uint64_t start = seg * 1024 + (uint64_t)lane * 32;
-        double buf[32];
-#pragma unroll
-        for (int i = 0; i < 32; i++) buf[i] = prob(psi[start + i]);
-#pragma unroll
-        for (int i = 0; i < 32; i += 2)
-            *reinterpret_cast<double2 *>(p + start + i) = make_double2(buf[i], buf[i + 1]);
-#pragma unroll
-        for (int w = 32; w > 1; w >>= 1) {
-#pragma unroll
-            for (int i = 0; i < w / 2; i++) buf[i] = buf[2 * i] + buf[2 * i + 1];
+    for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; j0 < m; j0 += stride) {
+        const int64_t j = j0 + lane;
+        uint32_t b = 0;
+        bool first = false;
+        if (j < m) {
+            const double u = (double)(splitmix64(seed, (uint64_t)j) >> 11) * 0x1.0p-53;
+            const uint64_t s = last_le(Q, ns, u);
+            b = (uint32_t)(s * G + last_le(R + s * G, G, u));
+            blk[j] = b;
+            if (slot) first = atomicExch(&slot[b], 0u) == 0xFFFFFFFFu;
         }
-        double v = buf[0];
-        for (int o = 1; o < 32; o <<= 1) {
-            double w = __shfl_down_sync(0xffffffffu, v, o);
-            if ((lane & (2 * o - 1)) == 0) v = v + w;
+        if (slot) {
+            const uint32_t hits = __ballot_sync(0xffffffffu, first);
+            uint32_t at = 0;
+            if (lane == 0 && hits) at = atomicAdd(n_list, (uint32_t)__popc(hits));
+            at = __shfl_sync(0xffffffffu, at, 0) + (uint32_t)__popc(hits & ((1u << lane) - 1u));
+            if (first) list[at] = b;
         }
-        if (lane == 0) out[seg] = v;
     }
 }
 
-// In place: p[bB + x] <- c_{b,x} = R_b + p_{bB} + ... + p_{bB+x}.  Lane l of a
-// warp owns block 32 w + l; the warp moves its 32 blocks through shared memory
-// 32 values at a time, so every global access is a 256-byte run.
-constexpr int kRunThreads = 128;
-
-__global__ void __launch_bounds__(kRunThreads) k_running_sums(double *__restrict__ p, const double *__restrict__ R,
-                                                              uint64_t nb)
+// slot[list[i]] = i (after k_locate: every block is in the list once)
+__global__ void k_slots(const uint32_t *__restrict__ list, const uint32_t *__restrict__ n_list, uint32_t *__restrict__ slot)
 {
-    __shared__ double tile[kRunThreads / 32][32][33];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g * 32 < nb; g += nwarps) {
-        const uint64_t b0 = g * 32;
-        const int nblk = nb - b0 < 32 ? (int)(nb - b0) : 32;
-        double c = lane < nblk ? R[b0 + lane] : 0.0;
-        for (int x0 = 0; x0 < 1024; x0 += 32) {
-            for (int r = 0; r < nblk; r++) tile[wl][r][lane] = p[(b0 + r) * 1024 + x0 + lane];
-            __syncwarp();
-            if (lane < nblk)
-                for (int x = 0; x < 32; x++) {
-                    c = c + tile[wl][lane][x];
-                    tile[wl][lane][x] = c;
+    const uint32_t n = *n_list;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) slot[list[i]] = i;
+}
+
+template <typename C>
+__global__ void __launch_bounds__(128)
+k_checkpoints(const C *__restrict__ psi, const double *__restrict__ R, uint32_t nb, const uint32_t *__restrict__ list,
+              const uint32_t *__restrict__ n_list, double *__restrict__ ck)
+{
+    static_assert(kCkRun == 16, "two checkpoints per 32 values");
+    const int lane = threadIdx.x & 31;
+    const uint32_t n_work = list ? *n_list : nb, nwarps = (gridDim.x * blockDim.x) >> 5;
+    constexpr int kAhead = 8;
+    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_work; w += nwarps) {
+        const uint32_t b = list ? list[w] : w;
+        const C *p = psi + (uint64_t)b * 1024 + lane;
+        double c = R[b], keep[2];                     // lane t keeps the checkpoints of values 32 t .. 32 t + 31
+        for (int t0 = 0; t0 < 32; t0 += kAhead) {
+            C a[kAhead];
+#pragma unroll
+            for (int t = 0; t < kAhead; t++) a[t] = p[32 * (t0 + t)];
+#pragma unroll
+            for (int t = 0; t < kAhead; t++) {
+                double half;
+                c = chain_add(c, prob(a[t]), half);
+                if (lane == t0 + t) {
+                    keep[0] = half;
+                    keep[1] = c;
                 }
-            __syncwarp();
-            for (int r = 0; r < nblk; r++) p[(b0 + r) * 1024 + x0 + lane] = tile[wl][r][lane];
-            __syncwarp();
+            }
         }
+        *reinterpret_cast<double2 *>(ck + (uint64_t)w * kCks + 2 * lane) = make_double2(keep[0], keep[1]);
     }
 }
 
-__global__ void k_draw_search(const double *__restrict__ c, const double *__restrict__ Q,
-                              const double *__restrict__ R, uint64_t ns, uint64_t G, uint64_t seed, int64_t m,
-                              uint64_t *__restrict__ out)
+template <typename C>
+__global__ void k_draw_run(const C *__restrict__ psi, const double *__restrict__ R, const double *__restrict__ ck,
+                           const uint32_t *__restrict__ blk, const uint32_t *__restrict__ slot, uint64_t seed, int64_t m,
+                           uint64_t *__restrict__ out)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += stride) {
         const double u = (double)(splitmix64(seed, (uint64_t)j) >> 11) * 0x1.0p-53;
-        const uint64_t s = last_le(Q, ns, u);
-        const uint64_t b = s * G + last_le(R + s * G, G, u);
-        const double *cb = c + b * 1024;
-        uint64_t lo = 0, hi = 1024;          // first x with cb[x] > u, 1023 when none
+        const uint64_t b = blk[j];
+        const double *cb = ck + (uint64_t)(slot ? slot[b] : b) * kCks;
+        int lo = 0, hi = kCks;               // first run whose last sum passes u
         while (lo < hi) {
-            const uint64_t mid = (lo + hi) / 2;
+            const int mid = (lo + hi) / 2;
             if (cb[mid] > u) hi = mid; else lo = mid + 1;
         }
-        out[j] = b * 1024 + (lo < 1024 ? lo : 1023);
+        int x = 1023;                        // none: the block's last value
+        if (lo < kCks) {
+            double c = lo ? cb[lo - 1] : R[b];
+            const C *p = psi + b * 1024 + (uint64_t)lo * kCkRun;
+            for (x = 0; x < kCkRun - 1; x++) {
+                c = c + prob(p[x]);
+                if (c > u) break;
+            }
+            x += lo * kCkRun;
+        }
+        out[j] = b * 1024 + (uint64_t)x;
     }
 }
 
@@ -600,10 +739,10 @@ int stats_impl(qs_state *s, double *out, int nstat)
     if (nstat == 4 && (rc = ensure_fflog(st))) return rc;
     if (nstat == 1) {
         k_stats_partial<C, 1><<<grid, block, 0, st>>>((const C *)s->amp, N, part);
-        k_stats_final<1><<<1, 32, 0, st>>>(part, grid, res);
+        k_stats_final<1><<<1, kFinalThreads, 0, st>>>(part, grid, res);
     } else {
         k_stats_partial<C, 4><<<grid, block, 0, st>>>((const C *)s->amp, N, part);
-        k_stats_final<4><<<1, 32, 0, st>>>(part, grid, res);
+        k_stats_final<4><<<1, kFinalThreads, 0, st>>>(part, grid, res);
     }
     QS_CUDA(cudaGetLastError(), "stats launch");
     QS_CUDA(cudaMemcpyAsync(out, res, sizeof(double) * nstat, cudaMemcpyDeviceToHost, st), "stats copy");
@@ -666,63 +805,64 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
     const size_t m_slots = (size_t)std::max<int64_t>(m, 1);
     size_t bytes = sizeof(double) * (2 * nb + 2 * ns) + sizeof(uint64_t) * m_slots;
     if (fused) bytes += sizeof(double) * ((size_t)gb * 4 + 4);
-    // complex128 with blocks of 1024: the running sums of every block are
-    // stored (N doubles of scratch) and the draws search them; without room
-    // for them, the draws scan the block as before (the same outcomes)
-    bool search = !c64 && B == 1024 && m > 0;
+    // blocks of 1024: checkpoints of the running sums of every block, or of those
+    // hit when the draws cannot hit most of them; without room for them the
+    // draws scan their blocks (the same outcomes)
+    bool runs = B == 1024 && m > 0;
+    const bool listed = m < 2 * (int64_t)nb;
+    const size_t n_work = listed ? (size_t)std::min<uint64_t>(nb, m_slots) : nb;
+    const size_t runs_bytes = sizeof(double) * n_work * kCks + sizeof(uint32_t) * (m_slots + (listed ? nb + n_work + 1 : 0)) + 16;
     void *scr = nullptr;
-    int rc = qs_state_scratch(s, bytes + stats_bytes + (search ? sizeof(double) * N : 0), &scr);
-    if (rc && search) {
+    int rc = qs_state_scratch(s, bytes + stats_bytes + (runs ? runs_bytes : 0), &scr);
+    if (rc && runs) {
         cudaGetLastError();   // the failed allocation is not an error of the later launches
-        search = false;
+        runs = false;
         rc = qs_state_scratch(s, bytes + stats_bytes, &scr);
     }
     if (rc) return rc;
-    // the statistics' partial sums at the end of the scratch
-    double *spart = (double *)((char *)scr + bytes + (search ? sizeof(double) * N : 0));
-    double *sres = spart + (size_t)sgrid * 4;
-    double *P = (double *)scr;                       // probabilities, then running sums
-    if (search) scr = (void *)(P + N);
     double *S = (double *)scr, *R = S + nb, *T = R + nb, *Q = T + ns;
     uint64_t *dout = (uint64_t *)(Q + ns);
     double *part = (double *)(dout + m_slots), *res = part + (size_t)gb * 4;
+    // the statistics' partial sums (complex128), then the draws' tables
+    double *spart = (double *)((char *)scr + bytes), *sres = spart + (size_t)sgrid * 4;
+    double *ck = (double *)(((uintptr_t)scr + bytes + stats_bytes + 15) & ~(uintptr_t)15);
+    uint32_t *blk = (uint32_t *)(ck + n_work * kCks), *slot = listed ? blk + m_slots : nullptr;
+    uint32_t *list = listed ? slot + nb : nullptr, *n_list = listed ? list + n_work : nullptr;
     const C *psi = (const C *)s->amp;
     if (beside) {
         QS_CUDA(cudaEventRecord((cudaEvent_t)s->side_ev[0], st), "side fork");
         QS_CUDA(cudaStreamWaitEvent(ss, (cudaEvent_t)s->side_ev[0], 0), "side fork");
         k_stats_partial<C, 4><<<sgrid, 256, 0, ss>>>(psi, N, spart);
-        k_stats_final<4><<<1, 32, 0, ss>>>(spart, sgrid, sres);
+        k_stats_final<4><<<1, kFinalThreads, 0, ss>>>(spart, sgrid, sres);
         QS_CUDA(cudaGetLastError(), "stats launch");
         QS_CUDA(cudaEventRecord((cudaEvent_t)s->side_ev[1], ss), "side join");
     }
     if (fused) {
         if constexpr (c64) k_segment_sums_stats<C><<<gb, 256, 0, st>>>(psi, nb, S, part);
-        k_stats_final<4><<<1, 32, 0, st>>>(part, gb, res);
-    } else if (search)
-        k_block_sums_store<C><<<gb, 256, 0, st>>>(psi, nb, S, P);
-    else if (B == 1024)
+        k_stats_final<4><<<1, kFinalThreads, 0, st>>>(part, gb, res);
+    } else if (B == 1024)
         k_segment_sums<C, 32><<<gb, 256, 0, st>>>(psi, nb, (int)B, S);
     else if (B >= 32)
         k_segment_sums<C, 0><<<gb, 256, 0, st>>>(psi, nb, (int)B, S);
     else
         k_segment_sums_small<C><<<1, 32, 0, st>>>(psi, nb, (int)B, S);
-    const int gs = (int)std::min<uint64_t>((ns * 32 + 255) / 256, (uint64_t)sms * 16);
-    if (G == 1024)
+    if (ns > 1) {   // G = 1024
+        const int gs = (int)std::min<uint64_t>((ns * 32 + 255) / 256, (uint64_t)sms * 16);
         k_segment_sums<double, 32><<<gs, 256, 0, st>>>(S, ns, (int)G, T);
-    else if (G >= 32)
-        k_segment_sums<double, 0><<<gs, 256, 0, st>>>(S, ns, (int)G, T);
-    else
-        k_segment_sums_small<double><<<1, 32, 0, st>>>(S, ns, (int)G, T);
-    k_prefix_super<<<1, 1, 0, st>>>(T, ns, Q);
-    k_prefix_blocks<<<(int)std::min<uint64_t>((ns + 127) / 128, 1024), 128, 0, st>>>(S, Q, ns, G, R);
-    if (search) {
-        const int gr = (int)std::min<uint64_t>((nb + kRunThreads - 1) / kRunThreads, (uint64_t)sms * 16);
-        k_running_sums<<<gr, kRunThreads, 0, st>>>(P, R, nb);
-        k_draw_search<<<(int)std::min<int64_t>((m + 255) / 256, (int64_t)sms * 16), 256, 0, st>>>(
-            P, Q, R, ns, G, seed, m, dout);
+        k_prefix_super<<<1, 32, 0, st>>>(T, ns, Q);
+    }
+    k_prefix_blocks<<<(int)((ns + 3) / 4), 128, 0, st>>>(S, ns > 1 ? Q : nullptr, ns, G, R);
+    const int gd = (int)std::min<int64_t>((m + 127) / 128, (int64_t)sms * 16);
+    if (runs) {
+        if (listed) QS_CUDA(cudaMemsetAsync(slot, 0xFF, sizeof(uint32_t) * nb, st), "draw table");
+        if (listed) QS_CUDA(cudaMemsetAsync(n_list, 0, sizeof(uint32_t), st), "draw table");
+        k_locate<<<gd, 128, 0, st>>>(Q, R, ns, G, seed, m, blk, slot, list, n_list);
+        if (listed) k_slots<<<gd, 128, 0, st>>>(list, n_list, slot);
+        const int gr = (int)std::min<uint64_t>((n_work + 3) / 4, (uint64_t)sms * 12);
+        k_checkpoints<C><<<gr, 128, 0, st>>>(psi, R, (uint32_t)nb, list, n_list, ck);
+        k_draw_run<C><<<gd, 128, 0, st>>>(psi, R, ck, blk, slot, seed, m, dout);
     } else if (m > 0) {
-        k_draw<C><<<(int)std::min<int64_t>((m + 255) / 256, (int64_t)sms * 16), 256, 0, st>>>(
-            psi, Q, R, ns, G, B, seed, m, dout);
+        k_draw<C><<<gd, 128, 0, st>>>(psi, Q, R, ns, G, B, seed, m, dout);
     }
     QS_CUDA(cudaGetLastError(), "sampling launch");
     if (m > 0)
@@ -1263,7 +1403,7 @@ int stats_static_impl(const void *amp, int n, void *stream, double *out)
     if ((rc = ensure_fflog(st))) return rc;
     // every partial slot in [0, grid) and every result slot is written before it is read
     k_stats_partial<C, 4><<<grid, block, 0, st>>>((const C *)amp, N, part);
-    k_stats_final<4><<<1, 32, 0, st>>>(part, grid, res);
+    k_stats_final<4><<<1, kFinalThreads, 0, st>>>(part, grid, res);
     QS_CUDA(cudaGetLastError(), "qs_stats_static launch");
     QS_CUDA(cudaMemcpyAsync(out, res, sizeof(double) * 4, cudaMemcpyDeviceToHost, st), "qs_stats_static copy");
     QS_CUDA(cudaStreamSynchronize(st), "qs_stats_static sync");
