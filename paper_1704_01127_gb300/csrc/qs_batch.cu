@@ -3,18 +3,13 @@
 // Every circuit keeps its own state (2^n amplitudes) in one device buffer.  A
 // thread-block cluster of C CTAs owns one circuit at a time (static
 // round-robin over circuits sorted by descending cost) and applies all of its
-// ops in order.  Consecutive ops form a pass: their targets fit kLocalBits index
-// bits, so the 2^kLocalBits amplitudes that agree on the other bits (a chunk)
-// go through all of them in shared memory, and the state is read and written
-// once per pass instead of once per op.  The CTAs of a cluster split a pass's
-// chunks and meet at a hardware cluster barrier between passes, so a circuit's
-// ops stay ordered and no CTA ever waits on another cluster.  From |0...0> only
-// chunks in the support so far are visited (zeros elsewhere are neither read
-// nor written until a pass covers them).  The per-group arithmetic is the
-// single-state kernels' (qs_device.cuh), so a batch reproduces single-state
-// CUDA-core runs bit for bit.  The launch configuration (C, threads per CTA)
-// and the cluster bound k_max of the scheduler are chosen by a timing
-// autotuner; a launch can be captured once in a CUDA graph and replayed.
+// ops in order; the CTAs of a cluster split each sweep and meet at a hardware
+// cluster barrier between ops, so a circuit's ops stay ordered and no CTA ever
+// waits on another cluster.  The per-group arithmetic is the single-state
+// kernels' (qs_device.cuh), so a batch reproduces single-state CUDA-core runs
+// bit for bit.  The launch configuration (C, threads per CTA) and the cluster
+// bound k_max of the scheduler are chosen by a timing autotuner; a launch can
+// be captured once in a CUDA graph and replayed.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,35 +29,18 @@ struct BatchOp {
     int32_t kind;      // QS_OP_DENSE or QS_OP_PHASE
     int32_t k;
     int32_t n_act;
-    int32_t q[5];      // targets as bits of the chunk's local index
+    int32_t q[5];
     uint64_t data;     // byte offset into the pool
-};
-
-// Consecutive ops of one circuit whose targets lie in the bits `local`.  A
-// chunk's local index l spells those bits (ascending); the chunk index spells
-// the bits `outer`, the support's other bits before the pass.
-struct BatchPass {
-    int32_t n_ops;
-    int32_t first;     // the circuit's first pass: starts from |0...0>
-    int64_t op_first;
-    uint32_t local, outer;
-    uint32_t support;  // bits that may be set in the index of a nonzero amplitude before the pass
-    uint32_t clear;    // last pass: bits no pass covered (zeros are written there)
 };
 
 struct BatchCirc {
     int32_t n;
-    int32_t n_pass;
-    int64_t pass_first;
+    int32_t n_ops;
+    int64_t op_first;
     int64_t amp_off;   // in amplitudes
 };
 
-// Chunks of 64 KB (2^13 complex64, 2^12 complex128 amplitudes): with the
-// unitary three CTAs share an SM, so one loads while others compute.  The low
-// kRunBits bits are always local (runs of 64 bytes).
-template <typename R> constexpr int kLocalBits = sizeof(R) == 4 ? 13 : 12;
-template <typename R> constexpr int kRunBits = sizeof(R) == 4 ? 3 : 2;
-constexpr size_t kChunkBytes = 65536;
+constexpr int kBatchLowBits = 12;
 
 __device__ __forceinline__ void cluster_sync_all(int C)
 {
@@ -74,199 +52,80 @@ __device__ __forceinline__ void cluster_sync_all(int C)
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Where local index l sits in shared memory: the upper bits are folded into
-// the bank bits (four of 8-byte, three of 16-byte elements), so that lanes that
-// differ in any few neighbouring bits fall in different banks.  Linear:
-// place(a ^ b) = place(a) ^ place(b).
-template <typename R>
-__device__ __forceinline__ uint32_t place(uint32_t l)
-{
-    if constexpr (sizeof(R) == 4) return l ^ (((l >> 4) ^ (l >> 8) ^ (l >> 12)) & 15u);
-    else return l ^ (((l >> 3) ^ (l >> 6) ^ (l >> 9)) & 7u);
-}
-
-// The bits of x at the set positions of mask, lowest first.
-__device__ __forceinline__ uint32_t deposit(uint32_t x, uint32_t mask)
-{
-    uint32_t r = 0;
-    for (; mask; mask &= mask - 1, x >>= 1)
-        if (x & 1) r |= mask & (0u - mask);
-    return r;
-}
-
-// A dense k-qubit cluster on a chunk in shared memory: one thread per group, two
-// rows of U at a time; per output the same FMA sequence as qsd::dense_group.
 template <typename R, int K>
-__device__ __forceinline__ void dense_chunk(typename cplx<R>::t *sm, int W, const int *q, const typename cplx<R>::t *Us)
+__device__ __forceinline__ void dense_sweep(typename cplx<R>::t *psi, uint64_t N, const Targets &t,
+                                            const typename cplx<R>::t *Us, uint64_t g0, uint64_t gstride)
 {
-    using C = typename cplx<R>::t;
-    constexpr int D = 1 << K;
-    uint32_t pq[K];
-#pragma unroll
-    for (int j = 0; j < K; j++) pq[j] = place<R>(1u << q[j]);
-    auto at = [&](uint32_t pb, int x) {
-#pragma unroll
-        for (int j = 0; j < K; j++)
-            if ((x >> j) & 1) pb ^= pq[j];
-        return pb;
-    };
-    for (uint32_t g = threadIdx.x; g < (1u << (W - K)); g += blockDim.x) {
-        uint32_t l = g;
-#pragma unroll
-        for (int j = 0; j < K; j++) {
-            const uint32_t lo = l & ((1u << q[j]) - 1u);
-            l = ((l ^ lo) << 1) | lo;
-        }
-        const uint32_t pb = place<R>(l);
-        C v[D];
-#pragma unroll
-        for (int x = 0; x < D; x++) v[x] = sm[at(pb, x)];
-#pragma unroll 1
-        for (int r = 0; r < D; r += 2) {
-            R ar[2] = {0, 0}, ai[2] = {0, 0};
-#pragma unroll
-            for (int x = 0; x < D; x++) {
-#pragma unroll
-                for (int i = 0; i < 2; i++) {
-                    const C m = Us[(r + i) * D + x];
-                    ar[i] = fma(v[x].x, m.x, ar[i]);
-                    ai[i] = fma(v[x].y, m.x, ai[i]);
-                    ar[i] = fma(-v[x].y, m.y, ar[i]);
-                    ai[i] = fma(v[x].x, m.y, ai[i]);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 2; i++) {
-                C o;
-                o.x = ar[i];
-                o.y = ai[i];
-                sm[at(pb, r + i)] = o;
-            }
-        }
-    }
+    const uint64_t G = N >> K;
+    for (uint64_t g = g0; g < G; g += gstride) qsd::dense_group<R, K, true>(psi + qsd::group_base<K>(g, t), t, Us);
 }
 
 template <typename R>
 __global__ void __launch_bounds__(512)
-k_batch(const BatchCirc *__restrict__ circ, const int *__restrict__ order, int n_circ,
-        const BatchPass *__restrict__ passes, const BatchOp *__restrict__ ops, const uint8_t *__restrict__ pool,
-        typename cplx<R>::t *__restrict__ amp, int C)
+k_batch(const BatchCirc *__restrict__ circ, const int *__restrict__ order, int n_circ, const BatchOp *__restrict__ ops,
+        const uint8_t *__restrict__ pool, typename cplx<R>::t *__restrict__ amp, int C)
 {
     using C2 = typename cplx<R>::t;
-    extern __shared__ __align__(16) uint8_t smem[];
-    C2 *sm = reinterpret_cast<C2 *>(smem);
-    C2 *Us = reinterpret_cast<C2 *>(smem + kChunkBytes);
+    __shared__ __align__(16) C2 Us[32 * 32];
+    __shared__ uint8_t tab[1 << kBatchLowBits];
     __shared__ uint64_t part[64];
     __shared__ int act[64];
     __shared__ uint64_t cm[3];
-    __shared__ uint32_t hoff[2][64];          // index bits of the local bits kRunBits .. kRunBits + 5 and those above
     const int rank = blockIdx.x % C, cid = blockIdx.x / C, ncl = gridDim.x / C;
-    const int tid = threadIdx.x, T = blockDim.x;
+    const uint64_t gi0 = (uint64_t)rank * blockDim.x + threadIdx.x, gstride = (uint64_t)C * blockDim.x;
     for (int w = cid; w < n_circ; w += ncl) {
         const BatchCirc cc = circ[order[w]];
         C2 *psi = amp + cc.amp_off;
-        for (int ip = 0; ip < cc.n_pass; ip++) {
-            const BatchPass ps = passes[cc.pass_first + ip];
-            const int W = __popc(ps.local), rb = min(W, kRunBits<R>);
-            const uint32_t run = 1u << rb, runmask = run - 1u;
-            __syncthreads();                  // the last pass is done with hoff
-            {
-                uint32_t hi = ps.local;       // the local bits above the runs, six at a time
-                for (int j = 0; j < rb; j++) hi &= hi - 1;
-                uint32_t lo6 = 0;
-                for (int j = 0; j < 6 && hi; j++) {
-                    lo6 |= hi & (0u - hi);
-                    hi &= hi - 1;
-                }
-                if (tid < 64) hoff[0][tid] = deposit(tid, lo6);
-                else if (tid < 128) hoff[1][tid - 64] = deposit(tid - 64, hi);
-            }
-            __syncthreads();
-            auto off = [&](uint32_t l) {
-                const uint32_t h = l >> rb;
-                return hoff[0][h & 63u] | hoff[1][h >> 6] | (l & runmask);
-            };
-            const uint32_t n_chunks = 1u << __popc(ps.outer);
-            for (uint32_t ch = rank; ch < n_chunks; ch += C) {
-                C2 *base = psi + deposit(ch, ps.outer);
-                constexpr int kAhead = 8;
-                for (uint32_t l0 = tid; l0 < (1u << W); l0 += T * kAhead) {
-                    C2 z[kAhead];
+        const uint64_t N = 1ULL << cc.n;
+        for (uint64_t i = gi0; i < N; i += gstride) {
+            C2 z;
+            z.x = i == 0 ? (R)1 : (R)0;
+            z.y = 0;
+            psi[i] = z;
+        }
+        cluster_sync_all(C);
+        for (int o = 0; o < cc.n_ops; o++) {
+            const BatchOp op = ops[cc.op_first + o];
+            if (op.kind == QS_OP_DENSE) {
+                const int D = 1 << op.k;
+                const C2 *U = reinterpret_cast<const C2 *>(pool + op.data);
+                for (int i = threadIdx.x; i < D * D; i += blockDim.x) Us[i] = U[i];
+                __syncthreads();
+                Targets t;
 #pragma unroll
-                    for (int k = 0; k < kAhead; k++) {
-                        const uint32_t l = l0 + T * k, o = l < (1u << W) ? off(l) : 0;
-                        z[k].x = ps.first && l == 0 ? (R)1 : (R)0;   // the first pass has one chunk, from |0...0>
-                        z[k].y = 0;
-                        if (!ps.first && l < (1u << W) && !(o & ~ps.support)) z[k] = __ldcg(base + o);
+                for (int j = 0; j < 5; j++) t.q[j] = op.q[j];
+                switch (op.k) {
+                case 1: dense_sweep<R, 1>(psi, N, t, Us, gi0, gstride); break;
+                case 2: dense_sweep<R, 2>(psi, N, t, Us, gi0, gstride); break;
+                case 3: dense_sweep<R, 3>(psi, N, t, Us, gi0, gstride); break;
+                case 4: dense_sweep<R, 4>(psi, N, t, Us, gi0, gstride); break;
+                default: dense_sweep<R, 5>(psi, N, t, Us, gi0, gstride); break;
+                }
+            } else {
+                const qs_phase_dev *ph = reinterpret_cast<const qs_phase_dev *>(pool + op.data);
+                const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
+                if (threadIdx.x < 3) cm[threadIdx.x] = ph->cmask[threadIdx.x];
+                for (int i = threadIdx.x; i < op.n_act; i += blockDim.x) {
+                    part[i] = terms[i].partners;
+                    act[i] = terms[i].a;
+                }
+                __syncthreads();
+                const int L = cc.n < kBatchLowBits ? cc.n : kBatchLowBits;
+                for (int l = threadIdx.x; l < (1 << L); l += blockDim.x)
+                    tab[l] = qsd::phase_low((uint64_t)l, cm, act, part, op.n_act, L);
+                __syncthreads();
+                const uint64_t n_chunks = N >> L;
+                for (uint64_t ch = rank; ch < n_chunks; ch += C) {
+                    const uint64_t h = ch << L;
+                    uint64_t Mh;
+                    const int mh = qsd::phase_high(h, cm, act, part, op.n_act, L, Mh);
+                    C2 *base = psi + h;
+                    for (int l = threadIdx.x; l < (1 << L); l += blockDim.x) {
+                        const int m = (tab[l] + mh + 4 * __popcll((uint64_t)l & Mh)) & 7;
+                        if (m) base[l] = qsd::rotate8<C2, R>(qsd::ld<true>(base + l), m);
                     }
-#pragma unroll
-                    for (int k = 0; k < kAhead; k++)
-                        if (l0 + T * k < (1u << W)) sm[place<R>(l0 + T * k)] = z[k];
                 }
-                for (int o = 0; o < ps.n_ops; o++) {
-                    const BatchOp op = ops[ps.op_first + o];
-                    if (op.kind == QS_OP_DENSE) {
-                        const int D = 1 << op.k;
-                        const C2 *U = reinterpret_cast<const C2 *>(pool + op.data);
-                        for (int i = tid; i < D * D; i += T) Us[i] = U[i];
-                        __syncthreads();
-                        switch (op.k) {
-                        case 1: dense_chunk<R, 1>(sm, W, op.q, Us); break;
-                        case 2: dense_chunk<R, 2>(sm, W, op.q, Us); break;
-                        case 3: dense_chunk<R, 3>(sm, W, op.q, Us); break;
-                        case 4: dense_chunk<R, 4>(sm, W, op.q, Us); break;
-                        default: dense_chunk<R, 5>(sm, W, op.q, Us); break;
-                        }
-                    } else {
-                        // qubits numbered by local bit, then by chunk bit: the
-                        // exponent of (ch, l) is m_lo(l) + m_hi(ch) + 4 popc(l & M_ch)
-                        const qs_phase_dev *ph = reinterpret_cast<const qs_phase_dev *>(pool + op.data);
-                        const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
-                        if (tid < 3) cm[tid] = ph->cmask[tid];
-                        for (int i = tid; i < op.n_act; i += T) {
-                            part[i] = terms[i].partners;
-                            act[i] = terms[i].a;
-                        }
-                        __syncthreads();
-                        uint64_t Mh;
-                        const int mh = qsd::phase_high((uint64_t)ch << W, cm, act, part, op.n_act, W, Mh);
-                        // columns of 64 rows: a thread's column part, its warp's row parts
-                        const int lane = tid & 31, cb = min(W, 31 - __clz(T));
-                        const uint32_t col = (uint32_t)tid & ((1u << cb) - 1u);
-                        const int mc = qsd::phase_low(col, cm, act, part, op.n_act, cb);
-                        const uint32_t rows = 1u << (W - cb);
-                        int rm[2];
-                        uint32_t rx[2];
-#pragma unroll
-                        for (int i = 0; i < 2; i++) {
-                            const uint64_t r = (uint64_t)(lane + 32 * i) << cb;
-                            uint32_t x = 0;
-                            if (lane + 32u * i < rows) {
-                                for (int t = 0; t < op.n_act && act[t] < cb; t++)
-                                    x |= ((uint32_t)__popcll(r & part[t]) & 1u) << act[t];
-                                rm[i] = qsd::phase_low(r, cm, act, part, op.n_act, W);
-                            } else {
-                                rm[i] = 0;
-                            }
-                            rx[i] = x;
-                        }
-                        for (uint32_t r = 0; r < rows; r++) {
-                            const int m1 = __shfl_sync(0xffffffffu, r & 32 ? rm[1] : rm[0], r & 31);
-                            const uint32_t x1 = __shfl_sync(0xffffffffu, r & 32 ? rx[1] : rx[0], r & 31);
-                            const uint32_t l = (r << cb) | col;
-                            const int m = (mc + m1 + mh + 4 * (__popc(col & x1) + __popc(l & (uint32_t)Mh))) & 7;
-                            if (m && (uint32_t)tid < (1u << cb)) sm[place<R>(l)] = qsd::rotate8<C2, R>(sm[place<R>(l)], m);
-                        }
-                    }
-                    __syncthreads();
-                }
-                if (ps.n_ops == 0) __syncthreads();
-                for (uint32_t l = tid; l < (1u << W); l += T) base[off(l)] = sm[place<R>(l)];
-                __syncthreads();              // the chunk is out of shared memory
             }
-            if (ps.clear)                     // index bits no pass covered: zeros
-                for (uint64_t i = (uint64_t)rank * T + tid; i < (1ULL << cc.n); i += (uint64_t)C * T)
-                    if (i & ps.clear) psi[i] = C2{};
             cluster_sync_all(C);
         }
     }
@@ -360,7 +219,7 @@ struct qs_batch {
     int n_circ = 0;
     void *stream = nullptr;
     void *amp = nullptr;
-    void *ops = nullptr, *passes = nullptr, *circ = nullptr, *order = nullptr, *pool = nullptr, *stats = nullptr;
+    void *ops = nullptr, *circ = nullptr, *order = nullptr, *pool = nullptr, *stats = nullptr;
     // statistics: (circuit, part) of every CTA, the first CTA of every circuit, their sums, the log table
     void *sblk = nullptr, *sfirst = nullptr, *spart = nullptr, *slog = nullptr;
     int n_sblk = 0;
@@ -387,23 +246,19 @@ int upload(void **dst, const std::vector<T> &v)
     return QS_OK;
 }
 
-template <typename R>
-int launch_batch_r(qs_batch *b, int C, int block)
+int launch_batch(qs_batch *b, int C, int block)
 {
-    using C2 = typename cplx<R>::t;
-    const size_t smem = kChunkBytes + sizeof(C2) * 32 * 32;
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaFuncSetAttribute(k_batch<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return qs_fail(QS_ECUDA, "batch smem attribute: %s", cudaGetErrorString(e));
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<R>, block, smem);
+    cudaError_t e = b->dtype == QS_C128
+                        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<double>, block, 0)
+                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<float>, block, 0);
     if (e != cudaSuccess || occ < 1) occ = 1;
-    const int clusters = std::max(1, std::min(b->n_circ, sms * occ / C));
+    int clusters = std::max(1, std::min(b->n_circ, sms * occ / C));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(clusters * C);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
     cfg.stream = (cudaStream_t)b->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -412,48 +267,15 @@ int launch_batch_r(qs_batch *b, int C, int block)
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_batch<R>, (const BatchCirc *)b->circ, (const int *)b->order, b->n_circ,
-                           (const BatchPass *)b->passes, (const BatchOp *)b->ops, (const uint8_t *)b->pool, (C2 *)b->amp, C);
+    const BatchCirc *circ = (const BatchCirc *)b->circ;
+    const int *order = (const int *)b->order;
+    const BatchOp *ops = (const BatchOp *)b->ops;
+    const uint8_t *pool = (const uint8_t *)b->pool;
+    if (b->dtype == QS_C128)
+        e = cudaLaunchKernelEx(&cfg, k_batch<double>, circ, order, b->n_circ, ops, pool, (double2 *)b->amp, C);
+    else
+        e = cudaLaunchKernelEx(&cfg, k_batch<float>, circ, order, b->n_circ, ops, pool, (float2 *)b->amp, C);
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "batch launch: %s", cudaGetErrorString(e));
-}
-
-int launch_batch(qs_batch *b, int C, int block)
-{
-    return b->dtype == QS_C128 ? launch_batch_r<double>(b, C, block) : launch_batch_r<float>(b, C, block);
-}
-
-// A circuit's ops split into passes: a pass takes ops in order while their dense
-// targets fit W bits together with the run bits, then fills its bits up from
-// the lowest.  *ranges: the ops of every pass.
-void plan_passes(const qs_schedule *sc, int wmax, int run_bits, std::vector<BatchPass> &out, std::vector<int> &op_end)
-{
-    const int n = sc->n, W = std::min(n, wmax);
-    const uint32_t all = (uint32_t)qs_index_mask(n), runs = (uint32_t)qs_index_mask(std::min(n, run_bits));
-    uint32_t support = 0;
-    size_t i = 0;
-    do {
-        BatchPass p;
-        std::memset(&p, 0, sizeof(p));
-        uint32_t mask = runs;
-        for (; i < sc->ops.size(); i++) {
-            const qs_op_host &op = sc->ops[i];
-            uint32_t with = mask;
-            if (op.kind == QS_OP_DENSE)
-                for (int j = 0; j < op.k; j++) with |= 1u << op.qubits[j];
-            if (__builtin_popcount(with) > W) break;
-            mask = with;
-            p.n_ops++;
-        }
-        for (int b = 0; b < n && __builtin_popcount(mask) < W; b++) mask |= 1u << b;
-        p.first = out.empty() || support == 0;
-        p.local = mask;
-        p.support = support;
-        p.outer = support & ~mask;
-        support |= mask;
-        if (i == sc->ops.size()) p.clear = all & ~support;
-        out.push_back(p);
-        op_end.push_back((int)i);
-    } while (i < sc->ops.size());
 }
 
 bool valid_config(int C, int block)
@@ -485,7 +307,6 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
         const size_t rsz = dtype == QS_C128 ? 8 : 4;
         std::vector<BatchCirc> circ(n_circ);
         std::vector<BatchOp> ops;
-        std::vector<BatchPass> passes;
         std::vector<uint8_t> pool;
         std::vector<double> cost(n_circ, 0.0);
         qs_batch *b = new (std::nothrow) qs_batch();
@@ -505,63 +326,42 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
                 return qs_fail(QS_EINVAL, "qs_batch_create: circuit %d has a remapped schedule", c);
             }
             circ[c].n = sc->n;
-            circ[c].pass_first = (int64_t)passes.size();
+            circ[c].n_ops = (int32_t)sc->ops.size();
+            circ[c].op_first = (int64_t)ops.size();
             circ[c].amp_off = (int64_t)amp_total;
             b->nq.push_back(sc->n);
             b->amp_off.push_back(amp_total);
             amp_total += ((1ULL << sc->n) + 31) & ~31ULL;   // 256-byte aligned states
-            std::vector<BatchPass> plan;
-            std::vector<int> op_end;
-            plan_passes(sc, dtype == QS_C128 ? kLocalBits<double> : kLocalBits<float>,
-                        dtype == QS_C128 ? kRunBits<double> : kRunBits<float>, plan, op_end);
-            circ[c].n_pass = (int32_t)plan.size();
-            size_t at_op = 0;
-            for (size_t ip = 0; ip < plan.size(); ip++) {
-                BatchPass &ps = plan[ip];
-                ps.op_first = (int64_t)ops.size();
-                // a pass's numbering of the qubits: local bits, chunk bits, the rest
-                // (not in the support before the pass)
-                int pos[32], next = 0;
-                for (uint32_t m : {ps.local, ps.outer, (uint32_t)qs_index_mask(sc->n) & ~(ps.local | ps.outer)})
-                    for (int q = 0; q < sc->n; q++)
-                        if ((m >> q) & 1) pos[q] = next++;
-                for (; at_op < (size_t)op_end[ip]; at_op++) {
-                    const qs_op_host &op = sc->ops[at_op];
-                    BatchOp bo;
-                    std::memset(&bo, 0, sizeof(bo));
-                    bo.kind = op.kind;
-                    bo.k = op.k;
-                    size_t at = (pool.size() + 255) & ~(size_t)255;
-                    if (op.kind == QS_OP_DENSE) {
-                        for (int j = 0; j < op.k; j++) bo.q[j] = pos[op.qubits[j]];
-                        pool.resize(at + op.matrix.size() * rsz);
-                        for (size_t i = 0; i < op.matrix.size(); i++) {
-                            if (dtype == QS_C128) std::memcpy(pool.data() + at + 8 * i, &op.matrix[i], 8);
-                            else {
-                                float f = (float)op.matrix[i];
-                                std::memcpy(pool.data() + at + 4 * i, &f, 4);
-                            }
+            for (const qs_op_host &op : sc->ops) {
+                BatchOp bo;
+                std::memset(&bo, 0, sizeof(bo));
+                bo.kind = op.kind;
+                bo.k = op.k;
+                size_t at = (pool.size() + 255) & ~(size_t)255;
+                if (op.kind == QS_OP_DENSE) {
+                    for (int j = 0; j < op.k; j++) bo.q[j] = op.qubits[j];
+                    pool.resize(at + op.matrix.size() * rsz);
+                    for (size_t i = 0; i < op.matrix.size(); i++) {
+                        if (dtype == QS_C128) std::memcpy(pool.data() + at + 8 * i, &op.matrix[i], 8);
+                        else {
+                            float f = (float)op.matrix[i];
+                            std::memcpy(pool.data() + at + 4 * i, &f, 4);
                         }
-                        cost[c] += (double)(1ULL << sc->n) * (1 + (1 << op.k) / 8.0);
-                    } else if (op.kind == QS_OP_PHASE) {
-                        int n_act = 0;
-                        std::vector<int32_t> coeff(sc->n);
-                        for (int q = 0; q < sc->n; q++) coeff[pos[q]] = op.coeff[q];
-                        std::vector<std::pair<int, int>> edges;
-                        for (const auto &e : op.edges) edges.push_back({pos[e.first], pos[e.second]});
-                        std::vector<uint8_t> ph = qs_pack_phase(sc->n, coeff, edges, &n_act);
-                        bo.n_act = n_act;
-                        pool.resize(at + ph.size());
-                        std::memcpy(pool.data() + at, ph.data(), ph.size());
-                        cost[c] += (double)(1ULL << sc->n);
-                    } else {
-                        delete b;
-                        return qs_fail(QS_EUNSUPPORTED, "qs_batch_create: table diagonals are not batched");
                     }
-                    bo.data = at;
-                    ops.push_back(bo);
+                    cost[c] += (double)(1ULL << sc->n) * (1 + (1 << op.k) / 8.0);
+                } else if (op.kind == QS_OP_PHASE) {
+                    int n_act = 0;
+                    std::vector<uint8_t> ph = qs_pack_phase(sc->n, op.coeff, op.edges, &n_act);
+                    bo.n_act = n_act;
+                    pool.resize(at + ph.size());
+                    std::memcpy(pool.data() + at, ph.data(), ph.size());
+                    cost[c] += (double)(1ULL << sc->n);
+                } else {
+                    delete b;
+                    return qs_fail(QS_EUNSUPPORTED, "qs_batch_create: table diagonals are not batched");
                 }
-                passes.push_back(ps);
+                bo.data = at;
+                ops.push_back(bo);
             }
         }
         std::vector<int> order(n_circ);
@@ -571,7 +371,6 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
         cudaError_t e = cudaMalloc(&b->amp, amp_total * 2 * rsz);
         if (e != cudaSuccess) rc = qs_fail(QS_ENOMEM, "qs_batch_create: states: %s", cudaGetErrorString(e));
         if (!rc) rc = upload(&b->ops, ops);
-        if (!rc) rc = upload(&b->passes, passes);
         if (!rc) rc = upload(&b->circ, circ);
         if (!rc) rc = upload(&b->order, order);
         if (!rc) rc = upload(&b->pool, pool);
@@ -609,7 +408,7 @@ extern "C" void qs_batch_free(qs_batch *b)
     if (b->stream) cudaStreamSynchronize((cudaStream_t)b->stream);
     else cudaDeviceSynchronize();
     if (b->exec) cudaGraphExecDestroy(b->exec);
-    for (void *p : {b->amp, b->ops, b->passes, b->circ, b->order, b->pool, b->stats, b->sblk, b->sfirst, b->spart, b->slog})
+    for (void *p : {b->amp, b->ops, b->circ, b->order, b->pool, b->stats, b->sblk, b->sfirst, b->spart, b->slog})
         if (p) cudaFree(p);
     delete b;
 }
