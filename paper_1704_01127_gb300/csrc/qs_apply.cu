@@ -9,6 +9,7 @@
 
 #include "qs_device.cuh"
 #include "qs_internal.h"
+#include "qs_launch.cuh"
 
 namespace {
 
@@ -44,9 +45,11 @@ k_dense(typename cplx<R>::t *__restrict__ psi, uint64_t n_groups, Targets t,
     using C = typename cplx<R>::t;
     constexpr int D = 1 << K;
     __shared__ C Us[D * D];
+    chain_start();
     for (int i = threadIdx.x; i < D * D; i += blockDim.x)
         Us[i] = reinterpret_cast<const C *>(Ug)[i];
     __syncthreads();
+    chain_wait();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_groups; g += stride)
         qsd::dense_group<R, K, false>(psi + group_base<K>(g, t), t, Us);
@@ -77,6 +80,7 @@ k_diag(typename cplx<R>::t *__restrict__ psi, int n, int L, int k, const int *__
     __shared__ int row_x[kDiagChunkRows];
     const C *d = reinterpret_cast<const C *>(dg);
     const int tid = threadIdx.x;
+    chain_start();
     if (tid < k) q[tid] = qg[tid];
     __syncthreads();
     auto bits = [&](uint64_t i) {
@@ -92,6 +96,7 @@ k_diag(typename cplx<R>::t *__restrict__ psi, int n, int L, int k, const int *__
 #pragma unroll
     for (int v = 0; v < VEC; v++) xe[v] = bits(e + v);
     __syncthreads();
+    chain_wait();
     if (!in) return;
     const uint64_t n_chunks = 1ULL << (n - L);
     for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
@@ -165,6 +170,7 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
     __shared__ int act[64];
     __shared__ uint32_t row_x[kDiagChunkRows];
     __shared__ uint8_t row_m[kDiagChunkRows];
+    chain_start();
     const uint64_t cm[3] = {ph->cmask[0], ph->cmask[1], ph->cmask[2]};
     const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
     const int tid = threadIdx.x, lane = tid & 31;
@@ -195,6 +201,7 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
     const bool any_odd = cm[0] != 0;
     const bool pairs = odd != 0 && rows > 1 && rb == RB;
     __syncthreads();
+    chain_wait();
     const uint64_t n_chunks = 1ULL << (n - L);
     constexpr int kAhead = kDiagAhead;
     for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
@@ -291,9 +298,8 @@ int launch_dense_t(qs_state *s, const int *q, const void *U)
     uint64_t groups = 1ULL << (s->n - K);
     const int block = 128;
     int grid = grid_for(groups, block, 8);
-    k_dense<R, K><<<grid, block, 0, (cudaStream_t)s->stream>>>(
-        reinterpret_cast<typename cplx<R>::t *>(s->amp), groups, t, reinterpret_cast<const R *>(U));
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_sweep(s, k_dense<R, K>, grid, block, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), groups,
+                                       t, reinterpret_cast<const R *>(U));
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_dense launch: %s", cudaGetErrorString(e));
 }
 
@@ -348,21 +354,21 @@ static int diag_chunk(int n, int *grid)
 }
 
 template <typename R>
-static void launch_diag_r(qs_state *s, const int *dev_qubits, int k, const void *dev_table)
+static cudaError_t launch_diag_r(qs_state *s, const int *dev_qubits, int k, const void *dev_table)
 {
     int grid;
     const int L = diag_chunk<R>(s->n, &grid);
-    k_diag<R><<<grid, kDiagThreads, 0, (cudaStream_t)s->stream>>>(
-        reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, k, dev_qubits, reinterpret_cast<const R *>(dev_table));
+    return launch_sweep(s, k_diag<R>, grid, kDiagThreads, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, k,
+                        dev_qubits, reinterpret_cast<const R *>(dev_table));
 }
 
 template <typename R>
-static void launch_phase_r(qs_state *s, const void *dev_phase, int n_act)
+static cudaError_t launch_phase_r(qs_state *s, const void *dev_phase, int n_act)
 {
     int grid;
     const int L = diag_chunk<R>(s->n, &grid);
-    k_phase<R><<<grid, kDiagThreads, 0, (cudaStream_t)s->stream>>>(
-        reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, (const qs_phase_dev *)dev_phase, n_act);
+    return launch_sweep(s, k_phase<R>, grid, kDiagThreads, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L,
+                        (const qs_phase_dev *)dev_phase, n_act);
 }
 
 int qs_launch_diag(qs_state *s, const int *dev_qubits, int k, const void *dev_table)
@@ -370,9 +376,8 @@ int qs_launch_diag(qs_state *s, const int *dev_qubits, int k, const void *dev_ta
     s->perm_invariant = false;
     int rc = qs_materialize(s);
     if (rc) return rc;
-    if (s->dtype == QS_C128) launch_diag_r<double>(s, dev_qubits, k, dev_table);
-    else launch_diag_r<float>(s, dev_qubits, k, dev_table);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = s->dtype == QS_C128 ? launch_diag_r<double>(s, dev_qubits, k, dev_table)
+                                              : launch_diag_r<float>(s, dev_qubits, k, dev_table);
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_diag launch: %s", cudaGetErrorString(e));
 }
 
@@ -381,9 +386,8 @@ int qs_launch_phase(qs_state *s, const void *dev_phase, int n_act)
     s->perm_invariant = false;
     int rc = qs_materialize(s);
     if (rc) return rc;
-    if (s->dtype == QS_C128) launch_phase_r<double>(s, dev_phase, n_act);
-    else launch_phase_r<float>(s, dev_phase, n_act);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = s->dtype == QS_C128 ? launch_phase_r<double>(s, dev_phase, n_act)
+                                              : launch_phase_r<float>(s, dev_phase, n_act);
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_phase launch: %s", cudaGetErrorString(e));
 }
 
@@ -816,6 +820,10 @@ extern "C" int qs_run_circuit(qs_state *s, const qs_schedule *sc)
         // the schedule's ops name index bits: put the qubits where it expects them
         if ((rc = qs_order_set(s, sc->remap.empty() ? nullptr : sc->remap.data()))) return rc;
         const qs_dev_sched &d = sc->dev[s->dtype];
+        struct ChainEnd {                 // whatever ends the run
+            qs_state *s;
+            ~ChainEnd() { s->chain = false; }
+        } chain_end{s};
         for (size_t i = 0; i < sc->ops.size(); i++) {
             const qs_op_host &op = sc->ops[i];
             const uint8_t *data = (const uint8_t *)d.pool + d.offset[i];
@@ -832,6 +840,7 @@ extern "C" int qs_run_circuit(qs_state *s, const qs_schedule *sc)
                 rc = qs_launch_phase(s, data, d.n_act[i]);
             }
             if (rc) return rc;
+            s->chain = !s->pair_sweeps;   // the next op's sweep follows this one directly
         }
         return QS_OK;
     });

@@ -49,6 +49,7 @@ struct qs_state {
     int path = 0;                 // QS_PATH_*
     bool fold_phase = true;       // qs_set_phase_fold
     bool pair_sweeps = false;     // qs_set_pair_sweeps
+    bool chain = false;           // the next launch follows a sweep of the same run (qs_launch.cuh)
     // every amplitude equal (qs_init_uniform, nothing applied since): any
     // exchange of qubits leaves the state as it is
     bool perm_invariant = false;

@@ -1,0 +1,39 @@
+// Launches whose start may overlap the end of the kernel before them on the
+// state's stream.  Inside qs_run_circuit consecutive sweeps are chained
+// (qs_state::chain): the next sweep's blocks start once every block of the
+// present one has started, set up what does not depend on the state (operands
+// to shared memory, tensor memory, tables) and wait for the present sweep to
+// finish before they touch an amplitude.  Every kernel launched this way calls
+// chain_start() first and chain_wait() before its first access to the state;
+// without a chain both do nothing.  20 qubits complex64, 16 sweeps: 149 -> 95 us a
+// circuit; 83 gates on 16 qubits: 401 -> 323 us (a sweep of a small state is
+// launch, set-up and one tile); large states gain the ramp between sweeps
+// (28 qubits complex64 1.5%).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "qs_internal.h"
+
+namespace {
+
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_sweep(const qs_state *s, void (*kernel)(P...), int grid, int block, size_t smem, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = (cudaStream_t)s->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = s->chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+}  // namespace

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "qs_internal.h"
+#include "qs_launch.cuh"
 #include "qs_tcgen05.cuh"
 
 namespace {
@@ -51,6 +52,7 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
     __shared__ PostSmem ps;
 
     const int tid = threadIdx.x, warp = tid >> 5;
+    chain_start();
     {
         const float4 *src = reinterpret_cast<const float4 *>(bpack);
         float4 *dst = reinterpret_cast<float4 *>(B_h);
@@ -69,6 +71,7 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    chain_wait();
     const uint32_t tmem = tmem_base_s;
     const uint32_t mbar_a = smem_u32(&mbar);
     const uint32_t a_h = smem_u32(A_h), a_t = smem_u32(A_t), b_h = smem_u32(B_h), b_t = smem_u32(B_t);
@@ -487,6 +490,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
     __shared__ uint8_t postR[kRows];      // kPost: the same for the row part, by row of the tile
 
     const int tid = threadIdx.x, warp = tid >> 5;
+    chain_start();
     // kSub: M = 2^m of the 32 members lie in the support (the others read as
     // zero); they take K positions 0 .. M-1, in order, and the rows of B^T
     // follow them, so only the first M K positions of A can be nonzero
@@ -562,6 +566,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             post_tile(ps, tile_base((uint64_t)blockIdx.x * kRows, t), tile_base(kRows - 1, t) ^ tile_base(0, t), postX[0], postC[0]);
         __syncthreads();
     }
+    chain_wait();
 
     if (kSub && tid < kSplitThreads && kMPT * (tid >> 7) >= M) {
         // ------------------------------------------------- idle splitters (kSub)
@@ -1056,26 +1061,21 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     int rc = qs_state_status(s, &status);
     if (rc) return rc;
     const qs_post_phase *post = (const qs_post_phase *)dev_post;
-    cudaStream_t st = (cudaStream_t)s->stream;
+    cudaError_t e;
     if (c64) {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms * 2);
-        if (fold)
-            k_dense5_tc_c64<true><<<grid, kRows, kSmemF32, st>>>((float2 *)s->amp, groups, t,
-                                                                (const float *)dev_pack, post, status);
-        else
-            k_dense5_tc_c64<false><<<grid, kRows, kSmemF32, st>>>((float2 *)s->amp, groups, t,
-                                                                 (const float *)dev_pack, post, status);
+        e = launch_sweep(s, fold ? k_dense5_tc_c64<true> : k_dense5_tc_c64<false>, grid, kRows, kSmemF32, (float2 *)s->amp,
+                         groups, t, (const float *)dev_pack, post, status);
     } else {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms);
-        c128<<<grid, kC128Threads, kSmemC128Pipe, st>>>((double2 *)s->amp, groups, t, (const uint8_t *)dev_pack,
-                                                       post, status);
+        e = launch_sweep(s, c128, grid, kC128Threads, kSmemC128Pipe, (double2 *)s->amp, groups, t,
+                         (const uint8_t *)dev_pack, post, status);
     }
     // amplitudes on the padding targets of an embedded cluster keep their
     // fixed values (U (x) 1 leaves zero inputs zero), so only the cluster's own
     // qubits join the support
     s->sup_free = (fr | (grow & tm)) == all ? ~0ULL : (fr | (grow & tm));
     s->sup_fix = fx & ~(grow & tm);
-    cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "tc launch: %s", cudaGetErrorString(e));
 }
 
