@@ -115,11 +115,12 @@ k_probs(const C *__restrict__ psi, uint64_t first, uint64_t count, double *__res
 }
 
 using qsd::ff;
-using qsd::ff_add;
-using qsd::ff_from_double;
-using qsd::ff_mul;
+using qsd::ff_abs_double;
+using qsd::ff_accumulate;
 using qsd::ff_p_ln_p;
-using qsd::ff_sqr_f;
+using qsd::ff_fast_two_sum;
+using qsd::ff_sqr_loose;
+using qsd::ff_two_sum;
 using qsd::FFLogTable;
 using qsd::ff_log_table_init;
 
@@ -152,22 +153,23 @@ struct StatsAcc {
     template <int NSTAT>
     __device__ __forceinline__ void add(const double2 a, const FFLogTable &lt)
     {
-        // magnitude tests on the exponent fields (integer compares; FP64
-        // compares would run on the FP64 pipe): field < 1053 is |v| < 2^30,
-        // field >= 963 is |v| >= 2^-60
-        const uint32_t ex = ((uint32_t)__double2hiint(a.x) >> 20) & 0x7FFu;
-        const uint32_t ey = ((uint32_t)__double2hiint(a.y) >> 20) & 0x7FFu;
-        if (ex < 1053u && ey < 1053u) {
-            // x and y as float-float (values below 2^-60 add less than 2^-120
-            // to p and count as zero), p and its sums in float-float
-            const ff x = ex >= 963u ? ff_from_double(a.x) : ff{0.f, 0.f};
-            const ff y = ey >= 963u ? ff_from_double(a.y) : ff{0.f, 0.f};
-            const ff p = ff_add(ff_mul(x, x), ff_mul(y, y));
-            f0 = ff_add(f0, p);
+        // magnitude tests on the high words (integer compares; FP64 compares
+        // would run on the FP64 pipe): below 2^30, and 2^-60 or more
+        const uint32_t hx = (uint32_t)__double2hiint(a.x) & 0x7FFFFFFFu, hy = (uint32_t)__double2hiint(a.y) & 0x7FFFFFFFu;
+        if (max(hx, hy) < 1053u << 20) {
+            // |x| and |y| as float-float (values below 2^-60 add less than 2^-120
+            // to p and count as zero); p = x^2 + y^2 with the low parts' errors added
+            // once, then normalised
+            const ff x = hx >= 963u << 20 ? ff_abs_double(hx, (uint32_t)__double2loint(a.x)) : ff{0.f, 0.f};
+            const ff y = hy >= 963u << 20 ? ff_abs_double(hy, (uint32_t)__double2loint(a.y)) : ff{0.f, 0.f};
+            const ff xx = ff_sqr_loose(x), yy = ff_sqr_loose(y);
+            const ff t = ff_two_sum(xx.hi, yy.hi);
+            const ff p = ff_fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(xx.lo, yy.lo)));
+            ff_accumulate(f0, p);
             if (NSTAT == 4) {
-                f3 = ff_add(f3, ff_mul(p, p));
+                ff_accumulate(f3, ff_sqr_loose(p));
                 if (p.hi >= 0x1p-79f) {
-                    fent = ff_add(fent, ff_p_ln_p(lt, p));
+                    ff_accumulate(fent, ff_p_ln_p(lt, p));
                 } else if (p.hi > 0.f) {
                     const double pd = (double)p.hi + (double)p.lo;
                     if (pd >= 2.2250738585072014e-308) dent += pd * log(pd);

@@ -275,24 +275,10 @@ __device__ __forceinline__ ff ff_fast_two_sum(float a, float b)   // |a| >= |b| 
     const float s = __fadd_rn(a, b);
     return ff{s, __fsub_rn(b, __fsub_rn(s, a))};
 }
-__device__ __forceinline__ ff ff_add(ff a, ff b)
-{
-    ff s = ff_two_sum(a.hi, b.hi);
-    s.lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-    return ff_fast_two_sum(s.hi, s.lo);
-}
 __device__ __forceinline__ ff ff_add_f(ff a, float b)
 {
     ff s = ff_two_sum(a.hi, b);
     return ff_fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
-}
-__device__ __forceinline__ ff ff_mul(ff a, ff b)
-{
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return ff_fast_two_sum(p, e);
 }
 // x^2 exactly as hi + lo (the FMA gives the rounding error of the product)
 __device__ __forceinline__ ff ff_sqr_f(float x)
@@ -300,17 +286,42 @@ __device__ __forceinline__ ff ff_sqr_f(float x)
     const float p = __fmul_rn(x, x);
     return ff{p, fmaf(x, x, -p)};
 }
-// The top 48 bits of a double d with |d| in [2^-126, 2^128), by bit
-// manipulation only: hi = its top 24 significant bits, lo = the next 24
-// (0 when they fall below the normal float range).  Relative error < 2^-47.
+// x^2 with its low part left unnormalised (the product's rounding error plus
+// 2 x.hi x.lo; x.lo^2 is below 2^-48 of the result)
+__device__ __forceinline__ ff ff_sqr_loose(ff x)
+{
+    const float p = __fmul_rn(x.hi, x.hi);
+    return ff{p, fmaf(__fadd_rn(x.hi, x.hi), x.lo, fmaf(x.hi, x.hi, -p))};
+}
+// s += a, the error of the high parts' sum and a's low part collected in s.lo and
+// never folded back (Ogita, Rump and Oishi's Sum2, SIAM J. Sci. Comput. 26,
+// 2005): the sum's error is that of adding the low parts in FP32
+__device__ __forceinline__ void ff_accumulate(ff &s, ff a)
+{
+    const ff t = ff_two_sum(s.hi, a.hi);
+    s.hi = t.hi;
+    s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, a.lo));
+}
+// |d| of a double with |d| in [2^-60, 2^30), its high word h without the sign:
+// hi = its top 24 significant bits (the exponent rebased by flipping one bit),
+// lo = the other 29, rounded to 24
+__device__ __forceinline__ ff ff_abs_double(uint32_t h, uint32_t l)
+{
+    const uint32_t b = (__funnelshift_l(l, h, 3) ^ 0x40000000u) & 0x7FFFFFFFu;
+    const float scale = __uint_as_float((b & 0x7F800000u) - (52u << 23));   // a unit of d's last place
+    return ff{__uint_as_float(b), __fmul_rn(__uint2float_rn(l & 0x1FFFFFFFu), scale)};
+}
+// A double d with |d| in [2^-126, 2^128) by bit manipulation only: hi = its top 24
+// significant bits, lo = the other 29 rounded to 24 (0 when they fall below the
+// normal float range).  Relative error 2^-48 at most.
 __device__ __forceinline__ ff ff_from_double(double d)
 {
     const uint32_t hw = (uint32_t)__double2hiint(d), lw = (uint32_t)__double2loint(d);
     const int E = (int)((hw >> 20) & 0x7FFu) - 1023;
     const uint32_t sign = hw & 0x80000000u;
     const float hi = __uint_as_float(sign | ((uint32_t)(E + 127) << 23) | ((hw & 0xFFFFFu) << 3) | (lw >> 29));
-    const float scale = __uint_as_float((uint32_t)max(E - 47 + 127, 0) << 23);   // 2^(E-47) or 0
-    const float lo = __uint2float_rn((lw >> 5) & 0xFFFFFFu) * scale;
+    const float scale = __uint_as_float((uint32_t)max(E - 52 + 127, 0) << 23);   // 2^(E-52) or 0
+    const float lo = __uint2float_rn(lw & 0x1FFFFFFFu) * scale;
     return ff{hi, sign ? -lo : lo};
 }
 
@@ -343,16 +354,24 @@ __device__ __forceinline__ ff ff_p_ln_p(const FFLogTable &t, ff p)
     const int j = (int)((b >> (23 - kFFLogBits)) & ((1u << kFFLogBits) - 1));
     // m = p 2^-e: the exponent of hi replaced, lo scaled by the same power of two
     const ff m = ff{__uint_as_float((b & 0x807FFFFFu) | (127u << 23)), p.lo * __uint_as_float((uint32_t)(127 - e) << 23)};
-    ff r = ff_mul(m, t.inv[j]);
-    r = ff_two_sum(__fsub_rn(r.hi, 1.0f), r.lo);            // hi - 1 is exact (hi within 2^-10 of 1)
+    // r = m / c_j - 1: hi - 1 is exact (hi within 2^-10 of 1)
+    const ff inv = t.inv[j];
+    const float ph = __fmul_rn(m.hi, inv.hi);
+    const float pl = fmaf(m.hi, inv.lo, fmaf(m.lo, inv.hi, fmaf(m.hi, inv.hi, -ph)));
+    const ff r = ff_fast_two_sum(__fsub_rn(ph, 1.0f), pl);
     // ln(1 + r) = r - r^2/2 + r^3/3 - r^4/4: -x^2/2 (x = r.hi) exactly as
-    // float-float, the rest (below 2^-32) in FP32, -x r.lo for the cross term
+    // float-float, the rest (below 2^-32) in FP32, -x r.lo for the cross term.
+    // e ln 2, x and -x^2/2 are summed with their errors; the low parts add up in FP32
     const float x = r.hi;
     const ff sq = ff_sqr_f(x);
-    const ff half = ff{-0.5f * sq.hi, -0.5f * sq.lo};
     const float tail = fmaf(x * x * x, fmaf(x, -0.25f, 0.33333334f), -x * r.lo);
-    const ff lnp = ff_add(ff_add(t.eln2[e + 127], t.ln[j]), ff_add(ff_add_f(r, tail), half));
-    return ff_mul(p, lnp);
+    const ff el = t.eln2[e + 127], lc = t.ln[j];
+    const ff s0 = ff_fast_two_sum(el.hi, lc.hi);        // |e ln 2| >= ln c_j, or e = 0
+    const ff s1 = ff_two_sum(s0.hi, x), s2 = ff_two_sum(s1.hi, -0.5f * sq.hi);
+    const float lo = ((s0.lo + s1.lo) + (s2.lo + (el.lo + lc.lo))) + (r.lo + fmaf(-0.5f, sq.lo, tail));
+    // p ln p, the low part left unnormalised
+    const float q = __fmul_rn(p.hi, s2.hi);
+    return ff{q, fmaf(p.lo, s2.hi, fmaf(p.hi, lo, fmaf(p.hi, s2.hi, -q)))};
 }
 
 }  // namespace qsd
