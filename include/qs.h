@@ -457,7 +457,7 @@ int qs_run_circuit(qs_state *s, const qs_schedule *sc);
 int qs_run_circuit_timed(qs_state *s, const qs_schedule *sc, float *op_ms);
 
 /* ------------------------------------------------------------------------
- * Batched simulation of many small circuits (one persistent launch).
+ * Batched simulation of many small circuits.
  * ---------------------------------------------------------------------- */
 typedef struct qs_batch qs_batch;   /* opaque, owned by the library */
 
@@ -470,18 +470,19 @@ int qs_batch_circuit_params(uint64_t seed, int *rows, int *cols, int *cz_cycles)
 
 /* One state per schedule (1..26 qubits, dense and phase ops), all in one
  * device allocation, plus the packed op list.  Each run starts every state at
- * |0...0> and applies its schedule; a cluster of CTAs owns one circuit at a
- * time (ops in order, a cluster barrier between ops), circuits sorted by
- * descending cost.  stream: cudaStream_t (non-NULL for graph replay). */
+ * |0...0> and applies its schedule, several ops per read and write of the state
+ * (a pass); one launch runs the j-th pass of every circuit, a CTA per chunk of up
+ * to 64 KB.  stream: cudaStream_t (non-NULL for graph replay). */
 int qs_batch_create(int n_circuits, const qs_schedule *const *schedules, int dtype, void *stream,
                     qs_batch **out);
 void qs_batch_free(qs_batch *b);
-/* Launch configuration: CTAs per cluster in {1, 2, 4, 8}, threads in {128, 256, 512}. */
+/* Launch configuration: CTAs (neighbouring chunks) per thread-block cluster in
+ * {1, 2, 4, 8}, threads per CTA in {128, 256, 512}. */
 int qs_batch_set_config(qs_batch *b, int cluster_ctas, int threads);
 int qs_batch_get_config(const qs_batch *b, int *cluster_ctas, int *threads);
-/* One persistent launch of the whole batch on the batch's stream. */
+/* The whole batch on the batch's stream: one launch per pass. */
 int qs_batch_run(qs_batch *b);
-/* The same launch, captured once into a CUDA graph (re-captured when the
+/* The same launches, captured once into a CUDA graph (re-captured when the
  * configuration changes) and replayed. */
 int qs_batch_run_graph(qs_batch *b);
 /* Per circuit i: out[4i..4i+3] as qs_stats (FP64); synchronises the stream. */

@@ -726,6 +726,42 @@ int launch_op_dense(qs_state *s, const qs_dev_sched &d, size_t i, const qs_op_ho
     return qs_launch_dense(s, op.qubits, op.k, data, nullptr);
 }
 
+// Ops i, i + 1, ... that run on the CUDA cores as passes (qs_pass.cu), *done of
+// them: two or more ops per read and write of the state, a pass of one op as its
+// own sweep.  A chunk has 2^(n-7) amplitudes, within the kernel's 2^8 .. 2^13
+// (complex64) or 2^12: 128 chunks at least, a CTA each, so a small state still
+// fills the GPU.
+int run_passes(qs_state *s, const qs_schedule *sc, const qs_dev_sched &d, size_t i, size_t *done)
+{
+    *done = 0;
+    if ((uintptr_t)s->amp & 15) return QS_OK;   // the kernel moves 16 bytes at a time
+    std::vector<qs_pass_in> in;
+    for (size_t j = i; j < sc->ops.size(); j++) {
+        const qs_op_host &op = sc->ops[j];
+        if (op.kind == QS_OP_DIAG || (op.kind == QS_OP_DENSE && path_of(s, op) == QS_PATH_TENSOR && d.tc_off[j])) break;
+        const size_t bytes = op.kind == QS_OP_DENSE
+                                 ? op.matrix.size() * (s->dtype == QS_C128 ? sizeof(double) : sizeof(float))
+                                 : sizeof(qs_phase_dev) + sizeof(qs_phase_term) * (size_t)d.n_act[j];
+        in.push_back({op.kind, op.k, d.n_act[j], op.qubits, (uint64_t)(uintptr_t)d.pool + d.offset[j], (uint32_t)bytes});
+    }
+    if (in.size() < 2) return QS_OK;
+    const int wmax = std::max(8, std::min(qs_pass_bits(s->dtype), s->n - 7));
+    for (const qs_pass &p : qs_plan_passes(s->n, s->dtype, wmax, in, false)) {
+        int rc;
+        if (p.n_ops > 1) {
+            rc = qs_launch_pass(s, p);
+        } else {
+            const qs_pass_in &op = in[p.first_op];
+            const void *data = (const void *)(uintptr_t)op.data;
+            rc = op.kind == QS_OP_DENSE ? qs_launch_dense(s, op.qubits, op.k, data, nullptr) : qs_launch_phase(s, data, op.n_act);
+        }
+        if (rc) return rc;
+        s->chain = !s->pair_sweeps;
+    }
+    *done = in.size();
+    return QS_OK;
+}
+
 }  // namespace
 
 extern "C" int qs_apply_cluster(qs_state *s, const int *qubits, int k, const double *U)
@@ -828,6 +864,12 @@ extern "C" int qs_run_circuit(qs_state *s, const qs_schedule *sc)
             const qs_op_host &op = sc->ops[i];
             const uint8_t *data = (const uint8_t *)d.pool + d.offset[i];
             int skip = 0;
+            size_t done = 0;
+            if ((rc = run_passes(s, sc, d, i, &done))) return rc;
+            if (done) {
+                i += done - 1;
+                continue;
+            }
             if (op.kind == QS_OP_DENSE && try_pair(s, sc, d, i, &rc, &skip)) {
                 i += skip;         // the ops after it that ran inside the pair's sweep
             } else if (op.kind == QS_OP_DENSE) {

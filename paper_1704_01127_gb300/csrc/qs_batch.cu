@@ -1,20 +1,20 @@
-// Batched simulation of many small circuits in one persistent launch.
+// Batched simulation of many small circuits.
 //
-// Every circuit keeps its own state (2^n amplitudes) in one device buffer.  A
-// thread-block cluster of C CTAs owns one circuit at a time (static
-// round-robin over circuits sorted by descending cost) and applies all of its
-// ops in order; the CTAs of a cluster split each sweep and meet at a hardware
-// cluster barrier between ops, so a circuit's ops stay ordered and no CTA ever
-// waits on another cluster.  The per-group arithmetic is the single-state
-// kernels' (qs_device.cuh), so a batch reproduces single-state CUDA-core runs
-// bit for bit.  The launch configuration (C, threads per CTA) and the cluster
-// bound k_max of the scheduler are chosen by a timing autotuner; a launch can
-// be captured once in a CUDA graph and replayed.
+// Every circuit keeps its own state (2^n amplitudes) in one device buffer.  Its
+// ops are split into passes (qs_pass.cu: several ops per read and write, chunks
+// in shared memory); one launch runs pass j of every circuit that has one, a CTA
+// per chunk, so the largest circuits spread over the whole GPU and ops of one
+// circuit stay ordered by the launches.  From |0...0> only chunks in the support
+// so far are visited (zeros elsewhere are neither read nor written until a pass
+// covers them).  The arithmetic is the single-state sweeps', so a batch
+// reproduces single-state CUDA-core runs bit for bit.  The launch configuration
+// (thread-block clusters of C neighbouring chunks, threads per CTA) and the
+// cluster bound k_max of the scheduler are chosen by a timing autotuner; the
+// launches can be captured once in a CUDA graph and replayed.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstring>
-#include <numeric>
 #include <vector>
 
 #include "qs_device.cuh"
@@ -23,113 +23,12 @@
 namespace {
 
 using qsd::cplx;
-using qsd::Targets;
-
-struct BatchOp {
-    int32_t kind;      // QS_OP_DENSE or QS_OP_PHASE
-    int32_t k;
-    int32_t n_act;
-    int32_t q[5];
-    uint64_t data;     // byte offset into the pool
-};
 
 struct BatchCirc {
     int32_t n;
-    int32_t n_ops;
-    int64_t op_first;
+    int32_t pad;
     int64_t amp_off;   // in amplitudes
 };
-
-constexpr int kBatchLowBits = 12;
-
-__device__ __forceinline__ void cluster_sync_all(int C)
-{
-    if (C == 1) {
-        __syncthreads();
-        return;
-    }
-    __threadfence();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-template <typename R, int K>
-__device__ __forceinline__ void dense_sweep(typename cplx<R>::t *psi, uint64_t N, const Targets &t,
-                                            const typename cplx<R>::t *Us, uint64_t g0, uint64_t gstride)
-{
-    const uint64_t G = N >> K;
-    for (uint64_t g = g0; g < G; g += gstride) qsd::dense_group<R, K, true>(psi + qsd::group_base<K>(g, t), t, Us);
-}
-
-template <typename R>
-__global__ void __launch_bounds__(512)
-k_batch(const BatchCirc *__restrict__ circ, const int *__restrict__ order, int n_circ, const BatchOp *__restrict__ ops,
-        const uint8_t *__restrict__ pool, typename cplx<R>::t *__restrict__ amp, int C)
-{
-    using C2 = typename cplx<R>::t;
-    __shared__ __align__(16) C2 Us[32 * 32];
-    __shared__ uint8_t tab[1 << kBatchLowBits];
-    __shared__ uint64_t part[64];
-    __shared__ int act[64];
-    __shared__ uint64_t cm[3];
-    const int rank = blockIdx.x % C, cid = blockIdx.x / C, ncl = gridDim.x / C;
-    const uint64_t gi0 = (uint64_t)rank * blockDim.x + threadIdx.x, gstride = (uint64_t)C * blockDim.x;
-    for (int w = cid; w < n_circ; w += ncl) {
-        const BatchCirc cc = circ[order[w]];
-        C2 *psi = amp + cc.amp_off;
-        const uint64_t N = 1ULL << cc.n;
-        for (uint64_t i = gi0; i < N; i += gstride) {
-            C2 z;
-            z.x = i == 0 ? (R)1 : (R)0;
-            z.y = 0;
-            psi[i] = z;
-        }
-        cluster_sync_all(C);
-        for (int o = 0; o < cc.n_ops; o++) {
-            const BatchOp op = ops[cc.op_first + o];
-            if (op.kind == QS_OP_DENSE) {
-                const int D = 1 << op.k;
-                const C2 *U = reinterpret_cast<const C2 *>(pool + op.data);
-                for (int i = threadIdx.x; i < D * D; i += blockDim.x) Us[i] = U[i];
-                __syncthreads();
-                Targets t;
-#pragma unroll
-                for (int j = 0; j < 5; j++) t.q[j] = op.q[j];
-                switch (op.k) {
-                case 1: dense_sweep<R, 1>(psi, N, t, Us, gi0, gstride); break;
-                case 2: dense_sweep<R, 2>(psi, N, t, Us, gi0, gstride); break;
-                case 3: dense_sweep<R, 3>(psi, N, t, Us, gi0, gstride); break;
-                case 4: dense_sweep<R, 4>(psi, N, t, Us, gi0, gstride); break;
-                default: dense_sweep<R, 5>(psi, N, t, Us, gi0, gstride); break;
-                }
-            } else {
-                const qs_phase_dev *ph = reinterpret_cast<const qs_phase_dev *>(pool + op.data);
-                const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
-                if (threadIdx.x < 3) cm[threadIdx.x] = ph->cmask[threadIdx.x];
-                for (int i = threadIdx.x; i < op.n_act; i += blockDim.x) {
-                    part[i] = terms[i].partners;
-                    act[i] = terms[i].a;
-                }
-                __syncthreads();
-                const int L = cc.n < kBatchLowBits ? cc.n : kBatchLowBits;
-                for (int l = threadIdx.x; l < (1 << L); l += blockDim.x)
-                    tab[l] = qsd::phase_low((uint64_t)l, cm, act, part, op.n_act, L);
-                __syncthreads();
-                const uint64_t n_chunks = N >> L;
-                for (uint64_t ch = rank; ch < n_chunks; ch += C) {
-                    const uint64_t h = ch << L;
-                    uint64_t Mh;
-                    const int mh = qsd::phase_high(h, cm, act, part, op.n_act, L, Mh);
-                    C2 *base = psi + h;
-                    for (int l = threadIdx.x; l < (1 << L); l += blockDim.x) {
-                        const int m = (tab[l] + mh + 4 * __popcll((uint64_t)l & Mh)) & 7;
-                        if (m) base[l] = qsd::rotate8<C2, R>(qsd::ld<true>(base + l), m);
-                    }
-                }
-            }
-            cluster_sync_all(C);
-        }
-    }
-}
 
 __global__ void k_log_table(qsd::LogTable *t) { qsd::log_table_init(*t); }
 
@@ -219,7 +118,12 @@ struct qs_batch {
     int n_circ = 0;
     void *stream = nullptr;
     void *amp = nullptr;
-    void *ops = nullptr, *circ = nullptr, *order = nullptr, *pool = nullptr, *stats = nullptr;
+    size_t amp_bytes = 0;
+    bool clear = false;             // some circuit has amplitudes that no pass covers: zeroed first
+    int W = 0;                      // bits of a chunk
+    // passes of all circuits, (pass, chunk) of every CTA by launch, operands
+    void *passes = nullptr, *items = nullptr, *circ = nullptr, *pool = nullptr, *stats = nullptr;
+    std::vector<size_t> level;      // first item of every launch, then their number
     // statistics: (circuit, part) of every CTA, the first CTA of every circuit, their sums, the log table
     void *sblk = nullptr, *sfirst = nullptr, *spart = nullptr, *slog = nullptr;
     int n_sblk = 0;
@@ -248,34 +152,17 @@ int upload(void **dst, const std::vector<T> &v)
 
 int launch_batch(qs_batch *b, int C, int block)
 {
-    int dev = 0, sms = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = b->dtype == QS_C128
-                        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<double>, block, 0)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<float>, block, 0);
-    if (e != cudaSuccess || occ < 1) occ = 1;
-    int clusters = std::max(1, std::min(b->n_circ, sms * occ / C));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(clusters * C);
-    cfg.blockDim = dim3(block);
-    cfg.stream = (cudaStream_t)b->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const BatchCirc *circ = (const BatchCirc *)b->circ;
-    const int *order = (const int *)b->order;
-    const BatchOp *ops = (const BatchOp *)b->ops;
-    const uint8_t *pool = (const uint8_t *)b->pool;
-    if (b->dtype == QS_C128)
-        e = cudaLaunchKernelEx(&cfg, k_batch<double>, circ, order, b->n_circ, ops, pool, (double2 *)b->amp, C);
-    else
-        e = cudaLaunchKernelEx(&cfg, k_batch<float>, circ, order, b->n_circ, ops, pool, (float2 *)b->amp, C);
-    return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "batch launch: %s", cudaGetErrorString(e));
+    if (b->clear) {
+        const cudaError_t e = cudaMemsetAsync(b->amp, 0, b->amp_bytes, (cudaStream_t)b->stream);
+        if (e != cudaSuccess) return qs_fail(QS_ECUDA, "batch clear: %s", cudaGetErrorString(e));
+    }
+    for (size_t l = 0; l + 1 < b->level.size(); l++) {
+        const size_t first = b->level[l], n = b->level[l + 1] - first;
+        if (int rc = qs_launch_pass_items(b->dtype, b->passes, (const uint2 *)b->items + first, (uint32_t)n, b->amp, b->W, C,
+                                          block, l > 0, b->stream))
+            return rc;
+    }
+    return QS_OK;
 }
 
 bool valid_config(int C, int block)
@@ -306,40 +193,32 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
             return qs_fail(QS_EINVAL, "qs_batch_create: bad arguments");
         const size_t rsz = dtype == QS_C128 ? 8 : 4;
         std::vector<BatchCirc> circ(n_circ);
-        std::vector<BatchOp> ops;
+        std::vector<std::vector<qs_pass_in>> in(n_circ);   // operands as offsets into the pool
         std::vector<uint8_t> pool;
-        std::vector<double> cost(n_circ, 0.0);
         qs_batch *b = new (std::nothrow) qs_batch();
         if (!b) return qs_fail(QS_ENOMEM, "qs_batch_create: out of host memory");
+        struct Owner {   // until the batch is handed out
+            qs_batch *b;
+            ~Owner() { qs_batch_free(b); }
+        } owner{b};
         b->dtype = dtype;
         b->n_circ = n_circ;
         b->stream = stream;
         uint64_t amp_total = 0;
         for (int c = 0; c < n_circ; c++) {
             const qs_schedule *sc = scheds[c];
-            if (!sc || sc->n < 1 || sc->n > 26) {
-                delete b;
+            if (!sc || sc->n < 1 || sc->n > 26)
                 return qs_fail(QS_EINVAL, "qs_batch_create: circuit %d must have 1..26 qubits", c);
-            }
-            if (!sc->remap.empty()) {
-                delete b;
-                return qs_fail(QS_EINVAL, "qs_batch_create: circuit %d has a remapped schedule", c);
-            }
+            if (!sc->remap.empty()) return qs_fail(QS_EINVAL, "qs_batch_create: circuit %d has a remapped schedule", c);
             circ[c].n = sc->n;
-            circ[c].n_ops = (int32_t)sc->ops.size();
-            circ[c].op_first = (int64_t)ops.size();
             circ[c].amp_off = (int64_t)amp_total;
             b->nq.push_back(sc->n);
             b->amp_off.push_back(amp_total);
             amp_total += ((1ULL << sc->n) + 31) & ~31ULL;   // 256-byte aligned states
             for (const qs_op_host &op : sc->ops) {
-                BatchOp bo;
-                std::memset(&bo, 0, sizeof(bo));
-                bo.kind = op.kind;
-                bo.k = op.k;
-                size_t at = (pool.size() + 255) & ~(size_t)255;
+                const size_t at = (pool.size() + 255) & ~(size_t)255;
+                int n_act = 0;
                 if (op.kind == QS_OP_DENSE) {
-                    for (int j = 0; j < op.k; j++) bo.q[j] = op.qubits[j];
                     pool.resize(at + op.matrix.size() * rsz);
                     for (size_t i = 0; i < op.matrix.size(); i++) {
                         if (dtype == QS_C128) std::memcpy(pool.data() + at + 8 * i, &op.matrix[i], 8);
@@ -348,32 +227,51 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
                             std::memcpy(pool.data() + at + 4 * i, &f, 4);
                         }
                     }
-                    cost[c] += (double)(1ULL << sc->n) * (1 + (1 << op.k) / 8.0);
                 } else if (op.kind == QS_OP_PHASE) {
-                    int n_act = 0;
                     std::vector<uint8_t> ph = qs_pack_phase(sc->n, op.coeff, op.edges, &n_act);
-                    bo.n_act = n_act;
                     pool.resize(at + ph.size());
                     std::memcpy(pool.data() + at, ph.data(), ph.size());
-                    cost[c] += (double)(1ULL << sc->n);
                 } else {
-                    delete b;
                     return qs_fail(QS_EUNSUPPORTED, "qs_batch_create: table diagonals are not batched");
                 }
-                bo.data = at;
-                ops.push_back(bo);
+                in[c].push_back({op.kind, op.k, n_act, op.qubits, at, (uint32_t)(pool.size() - at)});
             }
         }
-        std::vector<int> order(n_circ);
-        std::iota(order.begin(), order.end(), 0);
-        std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return cost[a] > cost[c]; });
         int rc = QS_OK;
-        cudaError_t e = cudaMalloc(&b->amp, amp_total * 2 * rsz);
-        if (e != cudaSuccess) rc = qs_fail(QS_ENOMEM, "qs_batch_create: states: %s", cudaGetErrorString(e));
-        if (!rc) rc = upload(&b->ops, ops);
+        b->amp_bytes = amp_total * 2 * rsz;
+        cudaError_t e = cudaMalloc(&b->amp, b->amp_bytes);
+        if (e != cudaSuccess) return qs_fail(QS_ENOMEM, "qs_batch_create: states: %s", cudaGetErrorString(e));
+        if ((rc = upload(&b->pool, pool))) return rc;
+        // the largest chunks (fewest passes) that still give every SM two or more
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        b->W = qs_pass_bits(dtype);
+        while (b->W > 9 && (amp_total >> b->W) < 2 * (uint64_t)sms) b->W--;
+        std::vector<qs_pass> passes;
+        std::vector<std::vector<uint2>> levels;
+        for (int c = 0; c < n_circ; c++) {
+            for (qs_pass_in &op : in[c]) op.data += (uint64_t)(uintptr_t)b->pool;
+            const std::vector<qs_pass> plan = qs_plan_passes(circ[c].n, dtype, b->W, in[c], true);
+            for (size_t l = 0; l < plan.size(); l++) {
+                if (levels.size() <= l) levels.emplace_back();
+                const uint32_t chunks = 1u << __builtin_popcountll(plan[l].outer);
+                for (uint32_t ch = 0; ch < chunks; ch++) levels[l].push_back(make_uint2((uint32_t)passes.size(), ch));
+                passes.push_back(plan[l]);
+                passes.back().amp = circ[c].amp_off;
+            }
+            const qs_pass &last = passes.back();
+            if ((last.support | last.local) != qs_index_mask(circ[c].n)) b->clear = true;
+        }
+        std::vector<uint2> items;
+        for (const std::vector<uint2> &l : levels) {
+            b->level.push_back(items.size());
+            items.insert(items.end(), l.begin(), l.end());
+        }
+        b->level.push_back(items.size());
+        if (!rc) rc = upload(&b->passes, passes);
+        if (!rc) rc = upload(&b->items, items);
         if (!rc) rc = upload(&b->circ, circ);
-        if (!rc) rc = upload(&b->order, order);
-        if (!rc) rc = upload(&b->pool, pool);
         std::vector<int2> sblk;
         std::vector<int> sfirst;
         for (int c = 0; c < n_circ; c++) {
@@ -393,11 +291,9 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
             k_log_table<<<1, 256, 0, (cudaStream_t)stream>>>((qsd::LogTable *)b->slog);
             if ((e = cudaGetLastError()) != cudaSuccess) rc = qs_fail(QS_ECUDA, "qs_batch_create: %s", cudaGetErrorString(e));
         }
-        if (rc) {
-            qs_batch_free(b);
-            return rc;
-        }
+        if (rc) return rc;
         *out = b;
+        owner.b = nullptr;
         return QS_OK;
     });
 }
@@ -405,10 +301,12 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
 extern "C" void qs_batch_free(qs_batch *b)
 {
     if (!b) return;
-    if (b->stream) cudaStreamSynchronize((cudaStream_t)b->stream);
-    else cudaDeviceSynchronize();
+    if (b->amp) {
+        if (b->stream) cudaStreamSynchronize((cudaStream_t)b->stream);
+        else cudaDeviceSynchronize();
+    }
     if (b->exec) cudaGraphExecDestroy(b->exec);
-    for (void *p : {b->amp, b->ops, b->circ, b->order, b->pool, b->stats, b->sblk, b->sfirst, b->spart, b->slog})
+    for (void *p : {b->amp, b->passes, b->items, b->circ, b->pool, b->stats, b->sblk, b->sfirst, b->spart, b->slog})
         if (p) cudaFree(p);
     delete b;
 }

@@ -195,6 +195,41 @@ uint64_t qs_swap_index(uint64_t i, const int *a, const int *b, int m);
 // Default kernel-path policy for a dense cluster (qs_apply.cu).
 bool qs_tc_wanted(int dtype, int k, int n);
 
+// Passes (qs_pass.cu): consecutive CUDA-core ops in one read and write of the state.
+constexpr int QS_PASS_OPS = 32;
+struct qs_pass_op {
+    uint8_t kind, k;       // QS_OP_DENSE or QS_OP_PHASE
+    uint8_t q[QS_MAX_K];   // dense: target j as a bit of the chunk's local index
+    uint8_t n_act;         // phase: CZ partner terms
+    uint16_t bytes, at;    // operand size (a multiple of 16), its place in the CTA's operand buffer
+    uint16_t n_stage;      // ops whose operands are brought in together before this one (0: it came in with another)
+    uint16_t pad;
+    uint64_t data;         // operand, device address
+};
+struct qs_pass {
+    uint64_t local;        // index bits inside a chunk
+    uint64_t outer;        // index bits that number the chunks
+    uint64_t support;      // bits that may be set in the index of a nonzero amplitude before the pass
+    int64_t amp;           // batch: the state's first amplitude
+    int32_t n_ops, first_op;
+    int32_t W;             // number of local bits
+    int32_t first;         // the pass starts from |0...0>: nothing is read
+    qs_pass_op op[QS_PASS_OPS];
+};
+struct qs_pass_in {
+    int kind, k, n_act;
+    const int *qubits;
+    uint64_t data;
+    uint32_t bytes;
+};
+int qs_pass_bits(int dtype);   // most local bits
+// Ops in order, as many per pass as fit wmax local bits.
+std::vector<qs_pass> qs_plan_passes(int n, int dtype, int wmax, const std::vector<qs_pass_in> &ops, bool from_basis);
+int qs_launch_pass(qs_state *s, const qs_pass &ps);
+// One launch over (pass, chunk) pairs; chain: it may start before the launch ahead of it has finished.
+int qs_launch_pass_items(int dtype, const void *passes, const void *items, uint32_t n, void *amp, int W, int cluster,
+                         int threads, bool chain, void *stream);
+
 // Pack a phase op into its device layout (qs_circuit.cpp).
 std::vector<uint8_t> qs_pack_phase(int n, const std::vector<int32_t> &coeff,
                                    const std::vector<std::pair<int, int>> &edges, int *n_act);

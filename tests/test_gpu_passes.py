@@ -1,0 +1,78 @@
+"""Passes (several CUDA-core ops per read and write of the state) against the
+same ops as one sweep each (qs_run_circuit_timed runs every op by itself): the
+same bits, at states below, of and above one chunk, with targets everywhere, odd
+phases on the lanes' bits and off them, more ops than one pass holds and operands
+larger than the CTA's buffer."""
+import numpy as np
+import pytest
+
+import paper_1704_01127_gb300.qs as qs
+from inputs import random_phase_poly, random_qubits, random_state, random_unitary
+
+pytestmark = pytest.mark.gpu
+
+
+def random_ops(n, count, seed, kinds):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    ops = []
+    for i in range(count):
+        kind = kinds[rng.integers(len(kinds))]
+        if kind == "phase":
+            coeff, edges = random_phase_poly(n, int(rng.integers(0, 2 * n)) if n > 1 else 0, seed + i)
+            coeff = np.asarray(coeff) * (rng.random(n) < rng.choice([0.1, 0.5, 1.0]))
+            if rng.random() < 0.3:
+                coeff = coeff // 2 * 2
+            ops.append((qs.QS_OP_PHASE, edges, coeff))
+        else:
+            k = min(n, int(kind))
+            q = random_qubits(n, k, seed + i)
+            ops.append((qs.QS_OP_DENSE, q, random_unitary(k, seed + i)))
+    return ops
+
+
+@pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
+@pytest.mark.parametrize("kinds", [("1", "phase"), ("2", "3", "phase"), ("4", "5"), ("phase",)], ids=lambda k: "".join(k))
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 7, 8, 9, 12, 13, 16, 19, 20, 21, 22])
+def test_passes_equal_sweeps(dtype, kinds, n):
+    psi = random_state(n, n)
+    sched = qs.qs_schedule_from_ops(n, random_ops(n, 40 if n <= 20 else 12, 17 * n, kinds))
+    h = qs.qs_alloc(n, dtype)
+    try:
+        qs.qs_set_path(h, qs.QS_PATH_CUDA_CORES)
+        out = []
+        for run in (qs.qs_run_circuit_timed, qs.qs_run_circuit):
+            qs.qs_set_amplitudes(h, psi)
+            run(h, sched)
+            out.append(qs.qs_get_amplitudes(h))
+    finally:
+        qs.qs_free(h)
+        qs.qs_schedule_free(sched)
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
+@pytest.mark.parametrize("sizes", [(1, 2, 4), (8, 9, 3), (16, 1, 17), (22,)])
+def test_batches_from_zero_equal_sweeps(dtype, sizes):
+    """Circuits of few ops leave index bits that no pass covers: zeros there, also in a second run."""
+    torch = pytest.importorskip("torch")
+    scheds = [qs.qs_schedule_from_ops(n, random_ops(n, c, 5 * n + c, ("1", "2", "4", "phase")))
+              for n in sizes for c in (1, 9)]
+    b = qs.qs_batch_create(scheds, dtype, torch.cuda.Stream())
+    try:
+        for threads in (128, 512):
+            qs.qs_batch_set_config(b, 2, threads)
+            for _ in range(2):
+                qs.qs_batch_run(b)
+            for i, sc in enumerate(scheds):
+                n = sizes[i // 2]
+                h = qs.qs_alloc(n, dtype)
+                qs.qs_set_path(h, qs.QS_PATH_CUDA_CORES)
+                qs.qs_init_basis(h, 0)
+                qs.qs_run_circuit_timed(h, sc)
+                want = qs.qs_get_amplitudes(h)
+                qs.qs_free(h)
+                assert np.array_equal(qs.qs_batch_get_amplitudes(b, i, n), want), (threads, i)
+    finally:
+        qs.qs_batch_free(b)
+        for sc in scheds:
+            qs.qs_schedule_free(sc)
