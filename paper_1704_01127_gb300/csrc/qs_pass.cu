@@ -15,10 +15,12 @@
 // What bounds it: the FP32 FMA pipe from k = 4 on in complex64, the FP64 pipe in
 // complex128.  Shared memory returns 128 bytes a clock per SM, broadcast or not:
 // with one group per thread the rows of U alone take twice the FMAs' time, so a
-// complex64 thread carries 512 / threads groups through every row (128 threads:
-// 4, two for k = 5: 128 registers of amplitudes).
+// complex64 thread carries up to four groups through every row (two for k = 5:
+// 128 registers of amplitudes).  Packed FP32 FMAs (fma.rn.f32x2) measured slower:
+// they need U's elements twice over, from shared memory or by moves.
 // 96 circuits of 16 to 21 qubits, k <= 4, complex64 (102 GFMA, 2.7 ms of the FMA
-// pipe; one cluster of CTAs per circuit before): 26.3 -> 7.6 ms.  A plain circuit
+// pipe; one cluster of CTAs per circuit before): 26.3 -> 7.0 ms, two thirds of the
+// issue slots used, half of them by FMAs.  A plain circuit
 // of 83 gates on 16 qubits, complex128: 320 -> 153 us (a sweep per gate before).
 #include <cuda_runtime.h>
 
@@ -70,9 +72,83 @@ struct LocalMap {
     }
 };
 
-// A dense k-qubit cluster on the chunk: G groups per thread and turn, per output
-// the FMA sequence of qsd::dense_group.
-template <typename R, int K, int G, int T>
+// fma(-a, b, c) with the sign in the FMA itself: written as fmaf(-a, b, c) with a
+// from shared memory, the compiler spends an integer instruction on every -a.
+__device__ __forceinline__ float fnma(float a, float b, float c)
+{
+    float r;
+    asm("{\n\t.reg .f32 t;\n\tneg.f32 t, %1;\n\tfma.rn.f32 %0, t, %2, %3;\n\t}" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Local index of group g's member 0.
+template <int K>
+__device__ __forceinline__ uint32_t group_local(uint32_t g, const int *q)
+{
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+        const uint32_t lo = g & ((1u << q[j]) - 1u);
+        g = ((g ^ lo) << 1) | lo;
+    }
+    return g;
+}
+
+// A dense k-qubit cluster on the chunk, complex64, G groups per thread and turn
+// (T G divides the number of groups): the FMA sequence of qsd::dense_group.
+template <int K, int G, int T>
+__device__ __forceinline__ void dense_groups_g(float2 *sm, int W, const int *q, const float2 *Us)
+{
+    constexpr int D = 1 << K;
+    uint32_t pq[K];
+#pragma unroll
+    for (int j = 0; j < K; j++) pq[j] = place<float>(1u << q[j]);
+    const uint32_t ng = 1u << (W - K);
+#pragma unroll 1
+    for (uint32_t g0 = threadIdx.x; g0 < ng; g0 += T * G) {
+        float2 v[G][D];
+        uint32_t pb[G];
+#pragma unroll
+        for (int i = 0; i < G; i++) {
+            pb[i] = place<float>(group_local<K>(g0 + T * i, q));
+#pragma unroll
+            for (int x = 0; x < D; x++) {
+                uint32_t o = 0;
+#pragma unroll
+                for (int j = 0; j < K; j++)
+                    if ((x >> j) & 1) o ^= pq[j];
+                v[i][x] = sm[pb[i] ^ o];
+            }
+        }
+#pragma unroll 1
+        for (int r = 0; r < D; r++) {
+            float ar[G], ai[G];
+#pragma unroll
+            for (int i = 0; i < G; i++) ar[i] = ai[i] = 0;
+            const float4 *row = reinterpret_cast<const float4 *>(Us + r * D);
+#pragma unroll
+            for (int x = 0; x < D; x++) {
+                const float4 w = row[x >> 1];
+                const float mx = x & 1 ? w.z : w.x, my = x & 1 ? w.w : w.y;
+#pragma unroll
+                for (int i = 0; i < G; i++) {
+                    ar[i] = fmaf(v[i][x].x, mx, ar[i]);
+                    ai[i] = fmaf(v[i][x].y, mx, ai[i]);
+                    ar[i] = fnma(v[i][x].y, my, ar[i]);
+                    ai[i] = fmaf(v[i][x].x, my, ai[i]);
+                }
+            }
+            uint32_t o = 0;
+#pragma unroll
+            for (int j = 0; j < K; j++) o ^= (r >> j) & 1 ? pq[j] : 0u;
+#pragma unroll
+            for (int i = 0; i < G; i++) sm[pb[i] ^ o] = make_float2(ar[i], ai[i]);
+        }
+    }
+}
+
+// The same for any number of groups, one per thread and turn; with fewer groups
+// than threads the rows of a group are split over threads.
+template <typename R, int K, int T>
 __device__ __forceinline__ void dense_groups(typename cplx<R>::t *sm, int W, const int *q, const typename cplx<R>::t *Us)
 {
     using C = typename cplx<R>::t;
@@ -81,66 +157,45 @@ __device__ __forceinline__ void dense_groups(typename cplx<R>::t *sm, int W, con
 #pragma unroll
     for (int j = 0; j < K; j++) pq[j] = place<R>(1u << q[j]);
     const uint32_t ng = 1u << (W - K);
+    const bool split = ng < T;
+    int r0 = 0, r1 = D;
+    if (split) {
+        const int part = (int)(threadIdx.x >> (W - K)), rows = max(1, (int)((D * ng) / T));
+        r0 = min(D, part * rows);
+        r1 = min(D, r0 + rows);
+    }
 #pragma unroll 1
-    for (uint32_t g0 = threadIdx.x; g0 < ng; g0 += T * G) {
-        C v[G][D];
-        uint32_t pb[G];
+    for (uint32_t g = split ? threadIdx.x & (ng - 1u) : threadIdx.x; g < ng; g += T) {
+        const uint32_t pb = place<R>(group_local<K>(g, q));
+        C v[D];
 #pragma unroll
-        for (int i = 0; i < G; i++) {
-            uint32_t l = (g0 + T * i) & (ng - 1u);   // past the end (not stored): some group's
+        for (int x = 0; x < D; x++) {
+            uint32_t o = pb;
 #pragma unroll
-            for (int j = 0; j < K; j++) {
-                const uint32_t lo = l & ((1u << q[j]) - 1u);
-                l = ((l ^ lo) << 1) | lo;
-            }
-            pb[i] = place<R>(l);
-#pragma unroll
-            for (int x = 0; x < D; x++) {
-                uint32_t o = pb[i];
-#pragma unroll
-                for (int j = 0; j < K; j++)
-                    if ((x >> j) & 1) o ^= pq[j];
-                v[i][x] = sm[o];
-            }
+            for (int j = 0; j < K; j++)
+                if ((x >> j) & 1) o ^= pq[j];
+            v[x] = sm[o];
         }
+        if (split) __syncthreads();   // every thread of a group has read it (one turn, all threads)
 #pragma unroll 1
-        for (int r = 0; r < D; r++) {
-            R ar[G], ai[G];
-#pragma unroll
-            for (int i = 0; i < G; i++) ar[i] = ai[i] = 0;
+        for (int r = r0; r < r1; r++) {
+            R ar = 0, ai = 0;
             const C *row = Us + r * D;
 #pragma unroll
-            for (int x = 0; x < D; x += 2) {
-                C m[2];
-                if constexpr (sizeof(R) == 4) {
-                    const float4 w = *reinterpret_cast<const float4 *>(row + x);
-                    m[0] = make_float2(w.x, w.y);
-                    m[1] = make_float2(w.z, w.w);
-                } else {
-                    m[0] = row[x];
-                    m[1] = row[x + 1];
-                }
-#pragma unroll
-                for (int y = 0; y < 2; y++)
-#pragma unroll
-                    for (int i = 0; i < G; i++) {
-                        ar[i] = fma(v[i][x + y].x, m[y].x, ar[i]);
-                        ai[i] = fma(v[i][x + y].y, m[y].x, ai[i]);
-                        ar[i] = fma(-v[i][x + y].y, m[y].y, ar[i]);
-                        ai[i] = fma(v[i][x + y].x, m[y].y, ai[i]);
-                    }
+            for (int x = 0; x < D; x++) {
+                const C m = row[x];
+                ar = fma(v[x].x, m.x, ar);
+                ai = fma(v[x].y, m.x, ai);
+                ar = fma(-v[x].y, m.y, ar);
+                ai = fma(v[x].x, m.y, ai);
             }
-            uint32_t o = 0;
+            uint32_t o = pb;
 #pragma unroll
             for (int j = 0; j < K; j++) o ^= (r >> j) & 1 ? pq[j] : 0u;
-#pragma unroll
-            for (int i = 0; i < G; i++)
-                if (i == 0 || g0 + T * i < ng) {
-                    C z;
-                    z.x = ar[i];
-                    z.y = ai[i];
-                    sm[pb[i] ^ o] = z;
-                }
+            C z;
+            z.x = ar;
+            z.y = ai;
+            sm[o] = z;
         }
     }
 }
@@ -148,13 +203,14 @@ __device__ __forceinline__ void dense_groups(typename cplx<R>::t *sm, int W, con
 template <typename R, int K, int T>
 __device__ __forceinline__ void dense_chunk(typename cplx<R>::t *sm, int W, const int *q, const typename cplx<R>::t *Us)
 {
-    constexpr int G = sizeof(R) == 8 ? 1 : K == 5 ? (T < 256 ? 256 / T : 1) : 512 / T;
-    if constexpr (G > 1)
-        if ((1u << (W - K)) > T) {
-            dense_groups<R, K, G, T>(sm, W, q, Us);
-            return;
-        }
-    dense_groups<R, K, 1, T>(sm, W, q, Us);
+    if constexpr (sizeof(R) == 4) {
+        const uint32_t ng = 1u << (W - K);
+        if constexpr (K < 5 && T == 128)
+            if (ng >= 4 * T) return dense_groups_g<K, 4, T>(sm, W, q, Us);
+        if constexpr (T == 128 || (T == 256 && K < 5))
+            if (ng >= 2 * T) return dense_groups_g<K, 2, T>(sm, W, q, Us);
+    }
+    dense_groups<R, K, T>(sm, W, q, Us);
 }
 
 // A phase product on the chunk.  The index splits into a column (as many local
