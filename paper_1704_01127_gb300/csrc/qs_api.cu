@@ -9,6 +9,7 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "qs_device.cuh"
@@ -144,6 +145,9 @@ __global__ void k_fflog_init() { ff_log_table_init(g_fflog); }
 // range) takes p ln p from the FP64 math library, and complex128 amplitudes of
 // 2^30 or more (unnormalised input) are summed in FP64 throughout; p below the
 // normal double range contributes less than 1e-305 and is left out.
+// p ln p by the FP64 math library, out of the way of the common cases' code
+__device__ __noinline__ double p_ln_p_rare(double p) { return p * log(p); }
+
 // Per-thread sums of the statistics; add() takes one amplitude, partials()
 // reduces the block (every thread of the block calls it).
 struct StatsAcc {
@@ -193,14 +197,14 @@ struct StatsAcc {
         // and the logarithm of p are formed in FP32 (one rounding each, the
         // logarithm a few ulp), and the terms add up in float-float
         const float p = fmaf(a.x, a.x, __fmul_rn(a.y, a.y));
-        f0 = ff_add_f(f0, p);
+        ff_accumulate(f0, p);
         if (NSTAT == 4) {
-            f3 = ff_add_f(f3, __fmul_rn(p, p));
+            ff_accumulate(f3, __fmul_rn(p, p));
             if (p >= 0x1p-79f && p <= 0x1p100f) {
-                fent = ff_add_f(fent, __fmul_rn(p, __logf(p)));
+                ff_accumulate(fent, __fmul_rn(p, __logf(p)));
             } else if (p > 0.f) {
                 const double pd = (double)p;
-                if (pd >= 2.2250738585072014e-308) dent += pd * log(pd);
+                if (pd >= 2.2250738585072014e-308) dent += p_ln_p_rare(pd);
             }
         }
     }
@@ -335,6 +339,8 @@ int ensure_fflog(cudaStream_t st)
 }
 
 // ------------------------------------------------------------------ sampling
+constexpr uint32_t kFull = 0xffffffffu;
+
 // Pairwise sums over fixed power-of-two blocks: lane l of a warp reduces its
 // contiguous len/32 values as a perfect binary tree, then the 32 lane results
 // combine as the top five tree levels (lane pairs (0,1), (2,3), ... first).
@@ -392,46 +398,121 @@ __global__ void k_segment_sums(const T *__restrict__ src, uint64_t nseg, int len
     }
 }
 
-// Block sums of 1024 probabilities, as k_segment_sums<C, 32> (the same tree,
-// built as the values arrive: one pending sum per level, each joined as the
-// left operand of the next), and, from the same loads, the block's partial
-// sums of the statistics as k_stats_partial<C, 4> forms them (in another
-// order).  The block sums use the FP64 unit, the statistics the FP32 one
-// (launched for complex64 states).
+// The pairwise tree over a block of 1024 probabilities, by one warp with contiguous
+// loads: rows of 32 amplitudes (complex64: 64, a lane holds a pair and joins it),
+// eight rows to a piece.  A piece is summed over lane bits 0 to 2 by halving exchanges
+// (a lane keeps half of its rows and hands the other half to its partner: 7
+// additions, not 24), which leaves those bits numbering the rows from the top; the
+// pieces go on the same way over bits 3 and 4; then the rows are summed over the lanes
+// that hold them, lowest row bit first, and the pieces likewise.  Addition commutes,
+// so these are the tree's sums bit for bit, 1.125 FP64 additions a value.  (Each lane
+// reading its own 32 values needs every 32-byte sector several times over from a
+// cache that the warps of an SM overflow.)
+template <int N>
+__device__ __forceinline__ void halve(double *v, int o)
+{
+    const bool up = threadIdx.x & o;
+#pragma unroll
+    for (int i = 0; i < N / 2; i++) {
+        const double mine = up ? v[i + N / 2] : v[i], other = up ? v[i] : v[i + N / 2];
+        v[i] = mine + __shfl_xor_sync(kFull, other, o);
+    }
+}
+
+// Rows 0 .. 7 from p on, summed over lane bits 0 to 2; seen(a): every amplitude.
+template <typename F>
+__device__ __forceinline__ double piece_sum(const float4 *__restrict__ p, F seen)
+{
+    float4 a[8];
+    double v[8];
+#pragma unroll
+    for (int t = 0; t < 8; t++) a[t] = p[32 * t];
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+        const float2 x = make_float2(a[t].x, a[t].y), y = make_float2(a[t].z, a[t].w);
+        seen(x);
+        seen(y);
+        v[t] = prob(x) + prob(y);
+    }
+    halve<8>(v, 1);
+    halve<4>(v, 2);
+    halve<2>(v, 4);
+    return v[0];
+}
+template <typename F>
+__device__ __forceinline__ double piece_sum(const double2 *__restrict__ p, F seen)
+{
+    double2 a[8];
+    double v[8];
+#pragma unroll
+    for (int t = 0; t < 8; t++) a[t] = p[32 * t];
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+        seen(a[t]);
+        v[t] = prob(a[t]);
+    }
+    halve<8>(v, 1);
+    halve<4>(v, 2);
+    halve<2>(v, 4);
+    return v[0];
+}
+
+// (One piece after another: unrolled altogether, with the statistics, the code leaves
+// the instruction cache.)  With the statistics, 29 qubits complex64: 3.33 ms as one
+// 32-value run per lane, 1.71 ms.
+template <typename C, typename F>
+__device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen)
+{
+    using V = std::conditional_t<sizeof(C) == 8, float4, double2>;
+    constexpr int kPieces = sizeof(C) == 8 ? 2 : 4;
+    const V *p = reinterpret_cast<const V *>(psi) + (threadIdx.x & 31);
+    double v[kPieces];
+#pragma unroll
+    for (int j = 0; j < kPieces; j++) v[j] = 0;
+#pragma unroll 1
+    for (int i = 0; i < kPieces; i++) {
+#pragma unroll
+        for (int j = 0; j + 1 < kPieces; j++) v[j] = v[j + 1];
+        v[kPieces - 1] = piece_sum(p + 256 * i, seen);
+    }
+    halve<kPieces>(v, 8);
+    if constexpr (kPieces == 4) halve<2>(v, 16);
+    else v[0] = v[0] + __shfl_xor_sync(kFull, v[0], 16);
+    double t = v[0];
+#pragma unroll
+    for (int o = 4; o >= 1; o >>= 1) t = t + __shfl_xor_sync(kFull, t, o);
+    if constexpr (kPieces == 4) t = t + __shfl_xor_sync(kFull, t, 16);
+    return t + __shfl_xor_sync(kFull, t, 8);
+}
+
 template <typename C>
-__global__ void k_segment_sums_stats(const C *__restrict__ psi, uint64_t nseg, double *__restrict__ out,
-                                     double *__restrict__ part)
+__global__ void __launch_bounds__(256)
+k_block_sums(const C *__restrict__ psi, uint64_t nb, double *__restrict__ out)
+{
+    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t b = warp; b < nb; b += nwarps) {
+        const double v = block_sum(psi + b * 1024, [](const C &) {});
+        if ((threadIdx.x & 31) == 0) out[b] = v;
+    }
+}
+
+// The block sums and, from the same loads, the block's partial sums of the
+// statistics as k_stats_partial<C, 4> forms them (in another order).  The block
+// sums use the FP64 unit, their squares the integer units, the statistics the FP32
+// ones (launched for complex64 states); bound by issue slots.
+template <typename C>
+__global__ void __launch_bounds__(256, 3)
+k_block_sums_stats(const C *__restrict__ psi, uint64_t nb, double *__restrict__ out, double *__restrict__ part)
 {
     __shared__ __align__(16) FFLogTable lt;
     load_fflog<C, 4>(lt);
     StatsAcc acc;
-    const int lane = threadIdx.x & 31;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t seg = warp; seg < nseg; seg += nwarps) {
-        const C *src = psi + seg * 1024 + (uint64_t)lane * 32;
-        double lvl[5];
-        double v = 0.0;
-#pragma unroll
-        for (int i = 0; i < 32; i++) {
-            const C a = src[i];
-            acc.add<4>(a, lt);
-            v = prob(a);
-            // value i closes the subtrees of the levels where i has a one bit
-#pragma unroll
-            for (int l = 0; l < 5; l++) {
-                if (!((i >> l) & 1)) {
-                    lvl[l] = v;
-                    break;
-                }
-                v = lvl[l] + v;
-            }
-        }
-        for (int o = 1; o < 32; o <<= 1) {
-            double w = __shfl_down_sync(0xffffffffu, v, o);
-            if ((lane & (2 * o - 1)) == 0) v = v + w;
-        }
-        if (lane == 0) out[seg] = v;
+    for (uint64_t b = warp; b < nb; b += nwarps) {
+        const double v = block_sum(psi + b * 1024, [&](const C &a) { acc.add<4>(a, lt); });
+        if ((threadIdx.x & 31) == 0) out[b] = v;
     }
     acc.partials<4>(part);
 }
@@ -454,8 +535,6 @@ __global__ void k_segment_sums_small(const T *__restrict__ src, uint64_t nseg, i
 // additions one by one only where a value ties or the sum reaches the next
 // binade.  Bit for bit the sequential sums, without the FP64 pipe and without
 // its latency 32 times over.
-constexpr uint32_t kFull = 0xffffffffu;
-
 // r(p) for a sum with exponent field E >= 1; *slow: a tie, or p as large as c.
 __device__ __forceinline__ uint64_t chain_term(double p, int E, bool &slow)
 {
@@ -497,23 +576,84 @@ __device__ __forceinline__ uint64_t warp_sum54(uint64_t v)
 // c after this warp's 32 values in lane order; *half: the sum after lane 15's.
 __device__ __forceinline__ double chain_add(double c, double p, double &half)
 {
-    const uint64_t cb = (uint64_t)__double_as_longlong(c);
-    const int E = (int)(cb >> 52);
-    bool slow = E == 0;
-    const uint64_t r = chain_term(p, E, slow);
-    const uint64_t s16 = warp_sum54((threadIdx.x & 31) < 16 ? r : 0), s32 = warp_sum54(r);
-    if (__any_sync(kFull, slow) || (int)((cb + s32) >> 52) != E) {
-        double incl;
-        const double end = chain_slow(c, p, incl);
-        half = __shfl_sync(kFull, incl, 15);
-        return end;
-    }
-    half = __longlong_as_double((long long)(cb + s16));
-    return __longlong_as_double((long long)(cb + s32));
+    double incl;
+    const double end = chain_slow(c, p, incl);
+    half = __shfl_sync(kFull, incl, 15);
+    return end;
 }
 
-// The same with *excl the sum before this lane's value.
-__device__ __forceinline__ double chain_scan(double c, double p, double &excl)
+// The same for N groups of 32 values, half[k] and full[k] after group k's lanes 15 and
+// 31: all N at once while the sum stays in one binade without ties (the terms then
+// depend on c's exponent alone), else one group after another, addition by addition.
+// 2^e the start of c's binade: for p < 2^(e-20) a term is the low word of fl(2^e + p)
+// and a tie needs 20 zero bits at p's end.  Where some value has those or is larger,
+// the terms come from chain_term.
+template <int N>
+__device__ __forceinline__ double chain_add_n(double c, const double *p, double *half, double *full)
+{
+    const uint64_t cb = (uint64_t)__double_as_longlong(c);
+    const int E = (int)(cb >> 52);
+    const bool low = (threadIdx.x & 31) < 16;
+    const double c0 = __longlong_as_double((long long)(cb & 0x7FF0000000000000ULL));
+    const uint32_t top = (uint32_t)max(E - 20, 0) << 20;
+    uint32_t v[N], any = 0;
+    bool careful = E < 64;
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        const uint32_t h = (uint32_t)__double2hiint(p[k]), l = (uint32_t)__double2loint(p[k]);
+        v[k] = (uint32_t)__double2loint(c0 + p[k]);
+        any |= v[k];
+        careful = careful || h >= top || ((l & 0xFFFFFu) == 0 && (h | l) != 0);
+    }
+    uint64_t at = cb, mid[N], end[N];
+    bool slow = false;
+    if (!__any_sync(kFull, careful)) {
+        if (!__any_sync(kFull, any >> 27)) {   // 32 terms add up in 32 bits
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                mid[k] = at + __reduce_add_sync(kFull, low ? v[k] : 0u);
+                end[k] = at = at + __reduce_add_sync(kFull, v[k]);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                const uint32_t h = low ? v[k] : 0u;
+                mid[k] = at + __reduce_add_sync(kFull, h & 0xFFFFu) + ((uint64_t)__reduce_add_sync(kFull, h >> 16) << 16);
+                end[k] = at = at + __reduce_add_sync(kFull, v[k] & 0xFFFFu) + ((uint64_t)__reduce_add_sync(kFull, v[k] >> 16) << 16);
+            }
+        }
+    } else {
+        slow = E == 0;
+#pragma unroll
+        for (int k = 0; k < N; k++) {
+            const uint64_t r = chain_term(p[k], E, slow);
+            mid[k] = at + warp_sum54(low ? r : 0);
+            end[k] = at = at + warp_sum54(r);
+        }
+        slow = __any_sync(kFull, slow);
+    }
+    if (slow || (int)(at >> 52) != E) {
+#pragma unroll 1
+        for (int k = 0; k < N; k++) {
+#pragma unroll
+            for (int j = 0; j < N; j++)
+                if (j == k) {
+                    c = chain_add(c, p[j], half[j]);
+                    full[j] = c;
+                }
+        }
+        return c;
+    }
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        half[k] = __longlong_as_double((long long)mid[k]);
+        full[k] = __longlong_as_double((long long)end[k]);
+    }
+    return full[N - 1];
+}
+
+// The same with the sums before and after this lane's value.
+__device__ __forceinline__ double chain_scan(double c, double p, double &excl, double &incl)
 {
     const int lane = threadIdx.x & 31;
     const uint64_t cb = (uint64_t)__double_as_longlong(c);
@@ -529,13 +669,13 @@ __device__ __forceinline__ double chain_scan(double c, double p, double &excl)
     const uint64_t all = __shfl_sync(kFull, v, 31);
     // r < 2^53 each: 32 of them stay below 2^58
     if (__any_sync(kFull, slow) || (int)((cb + all) >> 52) != E) {
-        double incl;
         const double end = chain_slow(c, p, incl);
         excl = __shfl_up_sync(kFull, incl, 1);
         if (lane == 0) excl = c;
         return end;
     }
     excl = __longlong_as_double((long long)(cb + v - r));
+    incl = __longlong_as_double((long long)(cb + v));
     return __longlong_as_double((long long)(cb + all));
 }
 
@@ -552,8 +692,8 @@ __device__ __forceinline__ void prefix_chain(const double *__restrict__ v, uint6
 #pragma unroll
         for (int k = 0; k < kAhead; k++) {
             if (i0 + 32 * k >= n) break;
-            double excl;
-            c = chain_scan(c, x[k], excl);
+            double excl, incl;
+            c = chain_scan(c, x[k], excl, incl);
             if (i0 + 32 * k + lane < n) out[i0 + 32 * k + lane] = excl;
         }
     }
@@ -664,14 +804,14 @@ __global__ void k_slots(const uint32_t *__restrict__ list, const uint32_t *__res
 }
 
 template <typename C>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 8)
 k_checkpoints(const C *__restrict__ psi, const double *__restrict__ R, uint32_t nb, const uint32_t *__restrict__ list,
               const uint32_t *__restrict__ n_list, double *__restrict__ ck)
 {
     static_assert(kCkRun == 16, "two checkpoints per 32 values");
     const int lane = threadIdx.x & 31;
     const uint32_t n_work = list ? *n_list : nb, nwarps = (gridDim.x * blockDim.x) >> 5;
-    constexpr int kAhead = 8;
+    constexpr int kAhead = 4;
     for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_work; w += nwarps) {
         const uint32_t b = list ? list[w] : w;
         const C *p = psi + (uint64_t)b * 1024 + lane;
@@ -680,37 +820,69 @@ k_checkpoints(const C *__restrict__ psi, const double *__restrict__ R, uint32_t 
             C a[kAhead];
 #pragma unroll
             for (int t = 0; t < kAhead; t++) a[t] = p[32 * (t0 + t)];
+            double q[kAhead], half[kAhead], full[kAhead];
 #pragma unroll
-            for (int t = 0; t < kAhead; t++) {
-                double half;
-                c = chain_add(c, prob(a[t]), half);
+            for (int t = 0; t < kAhead; t++) q[t] = prob(a[t]);
+            c = chain_add_n<kAhead>(c, q, half, full);
+#pragma unroll
+            for (int t = 0; t < kAhead; t++)
                 if (lane == t0 + t) {
-                    keep[0] = half;
-                    keep[1] = c;
+                    keep[0] = half[t];
+                    keep[1] = full[t];
                 }
-            }
         }
         *reinterpret_cast<double2 *>(ck + (uint64_t)w * kCks + 2 * lane) = make_double2(keep[0], keep[1]);
     }
 }
 
+// Every running sum of every block, for many draws per block (a draw then needs no
+// additions).  complex128, 2^18 draws of 12 qubits: 228 -> 156 us a call, 2^20 of 20
+// qubits: 521 -> 369 us.
 template <typename C>
+__global__ void __launch_bounds__(128)
+k_running_sums(const C *__restrict__ psi, const double *__restrict__ R, uint32_t nb, double *__restrict__ sums)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    constexpr int kAhead = 8;
+    for (uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb; b += nwarps) {
+        const C *p = psi + (uint64_t)b * 1024 + lane;
+        double c = R[b];
+        for (int t0 = 0; t0 < 32; t0 += kAhead) {
+            C a[kAhead];
+#pragma unroll
+            for (int t = 0; t < kAhead; t++) a[t] = p[32 * (t0 + t)];
+#pragma unroll
+            for (int t = 0; t < kAhead; t++) {
+                double excl, incl;
+                c = chain_scan(c, prob(a[t]), excl, incl);
+                sums[(uint64_t)b * 1024 + 32 * (t0 + t) + lane] = incl;
+            }
+        }
+    }
+}
+
+// kEvery: ck holds every running sum, not one of kCkRun.
+template <typename C, bool kEvery>
 __global__ void k_draw_run(const C *__restrict__ psi, const double *__restrict__ R, const double *__restrict__ ck,
                            const uint32_t *__restrict__ blk, const uint32_t *__restrict__ slot, uint64_t seed, int64_t m,
                            uint64_t *__restrict__ out)
 {
+    constexpr int kN = kEvery ? 1024 : kCks;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += stride) {
         const double u = (double)(splitmix64(seed, (uint64_t)j) >> 11) * 0x1.0p-53;
         const uint64_t b = blk[j];
-        const double *cb = ck + (uint64_t)(slot ? slot[b] : b) * kCks;
-        int lo = 0, hi = kCks;               // first run whose last sum passes u
+        const double *cb = ck + (uint64_t)(slot ? slot[b] : b) * kN;
+        int lo = 0, hi = kN;                 // first run whose last sum passes u
         while (lo < hi) {
             const int mid = (lo + hi) / 2;
             if (cb[mid] > u) hi = mid; else lo = mid + 1;
         }
         int x = 1023;                        // none: the block's last value
-        if (lo < kCks) {
+        if (kEvery) {
+            x = min(lo, 1023);
+        } else if (lo < kCks) {
             double c = lo ? cb[lo - 1] : R[b];
             const C *p = psi + b * 1024 + (uint64_t)lo * kCkRun;
             for (x = 0; x < kCkRun - 1; x++) {
@@ -811,9 +983,10 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
     // hit when the draws cannot hit most of them; without room for them the
     // draws scan their blocks (the same outcomes)
     bool runs = B == 1024 && m > 0;
-    const bool listed = m < 2 * (int64_t)nb;
+    const bool listed = m < 2 * (int64_t)nb, every = m >= 128 * (int64_t)nb;
     const size_t n_work = listed ? (size_t)std::min<uint64_t>(nb, m_slots) : nb;
-    const size_t runs_bytes = sizeof(double) * n_work * kCks + sizeof(uint32_t) * (m_slots + (listed ? nb + n_work + 1 : 0)) + 16;
+    const size_t n_sums = n_work * (every ? 1024 : kCks);
+    const size_t runs_bytes = sizeof(double) * n_sums + sizeof(uint32_t) * (m_slots + (listed ? nb + n_work + 1 : 0)) + 16;
     void *scr = nullptr;
     int rc = qs_state_scratch(s, bytes + stats_bytes + (runs ? runs_bytes : 0), &scr);
     if (rc && runs) {
@@ -828,7 +1001,7 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
     // the statistics' partial sums (complex128), then the draws' tables
     double *spart = (double *)((char *)scr + bytes), *sres = spart + (size_t)sgrid * 4;
     double *ck = (double *)(((uintptr_t)scr + bytes + stats_bytes + 15) & ~(uintptr_t)15);
-    uint32_t *blk = (uint32_t *)(ck + n_work * kCks), *slot = listed ? blk + m_slots : nullptr;
+    uint32_t *blk = (uint32_t *)(ck + n_sums), *slot = listed ? blk + m_slots : nullptr;
     uint32_t *list = listed ? slot + nb : nullptr, *n_list = listed ? list + n_work : nullptr;
     const C *psi = (const C *)s->amp;
     if (beside) {
@@ -840,10 +1013,10 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
         QS_CUDA(cudaEventRecord((cudaEvent_t)s->side_ev[1], ss), "side join");
     }
     if (fused) {
-        if constexpr (c64) k_segment_sums_stats<C><<<gb, 256, 0, st>>>(psi, nb, S, part);
+        if constexpr (c64) k_block_sums_stats<C><<<gb, 256, 0, st>>>(psi, nb, S, part);
         k_stats_final<4><<<1, kFinalThreads, 0, st>>>(part, gb, res);
     } else if (B == 1024)
-        k_segment_sums<C, 32><<<gb, 256, 0, st>>>(psi, nb, (int)B, S);
+        k_block_sums<C><<<gb, 256, 0, st>>>(psi, nb, S);
     else if (B >= 32)
         k_segment_sums<C, 0><<<gb, 256, 0, st>>>(psi, nb, (int)B, S);
     else
@@ -860,9 +1033,14 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
         if (listed) QS_CUDA(cudaMemsetAsync(n_list, 0, sizeof(uint32_t), st), "draw table");
         k_locate<<<gd, 128, 0, st>>>(Q, R, ns, G, seed, m, blk, slot, list, n_list);
         if (listed) k_slots<<<gd, 128, 0, st>>>(list, n_list, slot);
-        const int gr = (int)std::min<uint64_t>((n_work + 3) / 4, (uint64_t)sms * 12);
-        k_checkpoints<C><<<gr, 128, 0, st>>>(psi, R, (uint32_t)nb, list, n_list, ck);
-        k_draw_run<C><<<gd, 128, 0, st>>>(psi, R, ck, blk, slot, seed, m, dout);
+        const int gr = (int)std::min<uint64_t>((n_work + 3) / 4, (uint64_t)sms * 8);   // one wave
+        if (every) {
+            k_running_sums<C><<<gr, 128, 0, st>>>(psi, R, (uint32_t)nb, ck);
+            k_draw_run<C, true><<<gd, 128, 0, st>>>(psi, R, ck, blk, slot, seed, m, dout);
+        } else {
+            k_checkpoints<C><<<gr, 128, 0, st>>>(psi, R, (uint32_t)nb, list, n_list, ck);
+            k_draw_run<C, false><<<gd, 128, 0, st>>>(psi, R, ck, blk, slot, seed, m, dout);
+        }
     } else if (m > 0) {
         k_draw<C><<<gd, 128, 0, st>>>(psi, Q, R, ns, G, B, seed, m, dout);
     }

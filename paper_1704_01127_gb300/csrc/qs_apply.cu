@@ -734,7 +734,6 @@ int launch_op_dense(qs_state *s, const qs_dev_sched &d, size_t i, const qs_op_ho
 int run_passes(qs_state *s, const qs_schedule *sc, const qs_dev_sched &d, size_t i, size_t *done)
 {
     *done = 0;
-    if ((uintptr_t)s->amp & 15) return QS_OK;   // the kernel moves 16 bytes at a time
     std::vector<qs_pass_in> in;
     for (size_t j = i; j < sc->ops.size(); j++) {
         const qs_op_host &op = sc->ops[j];

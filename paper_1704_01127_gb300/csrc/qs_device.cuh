@@ -214,10 +214,34 @@ __device__ __forceinline__ double sq_exact(float x)
     const uint64_t bexp = (uint64_t)(63 - lz + 2 * E + 1023);
     return __longlong_as_double((long long)((bexp << 52) | frac));
 }
-// p = fl(x^2 + y^2) with exact squares: fl(fl(x^2) + fl(y^2)) in FP64.
-__device__ __forceinline__ double prob(float2 a)
+static __device__ __noinline__ double prob_rare(float2 v) { return __dadd_rn(sq_exact(v.x), sq_exact(v.y)); }
+// p = fl(x^2 + y^2) with exact squares: fl(fl(x^2) + fl(y^2)) in FP64, in integer
+// operations as well, so a pass that adds p in FP64 has that pipe to itself.  With
+// a >= b the magnitudes, significands shifted up by 7: A = ma^2 in [2^60, 2^62), and
+// mb^2 shifted down by twice the exponents' difference s, its dropped bits joined
+// into the lowest one (they lie below the rounding position).  The sum's leading one
+// is at bit 60, 61 or 62 and it is rounded to 53 bits, half to even, as in sq_rn.
+// Subnormal or zero b, infinities and NaN take the squares one by one.
+__device__ __forceinline__ double prob(float2 v)
 {
-    return __dadd_rn(sq_exact(a.x), sq_exact(a.y));
+    const uint32_t bx = __float_as_uint(v.x) & 0x7fffffffu, by = __float_as_uint(v.y) & 0x7fffffffu;
+    const uint32_t a = max(bx, by), b = min(bx, by);
+    if (b < 0x800000u || a >= 0x7f800000u) return prob_rare(v);
+    const uint32_t ea = a >> 23, ma = (a << 7) & 0x3fffff80u | 0x40000000u, mb = (b << 7) & 0x3fffff80u | 0x40000000u;
+    const uint64_t A = (uint64_t)ma * ma, B = (uint64_t)mb * mb;
+    const uint32_t s = min(2u * (ea - (b >> 23)), 63u);
+    uint64_t r = B >> s;
+    if ((r << s) != B) r |= 1u;
+    const uint64_t S = A + r;
+    const uint32_t lo = (uint32_t)S, hi = (uint32_t)(S >> 32);
+    const uint32_t sh = 11u - (uint32_t)__clz((int)hi);   // 8, 9 or 10
+    const uint32_t ql = __funnelshift_r(lo, hi, sh), qh = hi >> sh;
+    const uint32_t x = lo << (32u - sh);
+    uint32_t rl, rh;
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %2, %3;\n\taddc.cc.u32 %0, %4, 0;\n\taddc.u32 %1, %5, %6;\n\t}"
+        : "=r"(rl), "=r"(rh)
+        : "r"(x), "r"(0x7FFFFFFFu + (ql & 1u)), "r"(ql), "r"(qh), "r"((2u * ea + sh + 760u) << 20));
+    return __hiloint2double((int)rh, (int)rl);
 }
 
 // Natural logarithm of a positive normal double, table-driven (P. T. P. Tang,
@@ -301,6 +325,12 @@ __device__ __forceinline__ void ff_accumulate(ff &s, ff a)
     const ff t = ff_two_sum(s.hi, a.hi);
     s.hi = t.hi;
     s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, a.lo));
+}
+__device__ __forceinline__ void ff_accumulate(ff &s, float a)
+{
+    const ff t = ff_two_sum(s.hi, a);
+    s.hi = t.hi;
+    s.lo = __fadd_rn(s.lo, t.lo);
 }
 // |d| of a double with |d| in [2^-60, 2^30), its high word h without the sign:
 // hi = its top 24 significant bits (the exponent rebased by flipping one bit),

@@ -64,3 +64,27 @@ def test_c128_probabilities_over_every_exponent(n):
     finally:
         qs.qs_free(h)
     assert np.array_equal(got.view(np.uint64), want.view(np.uint64))
+
+
+@pytest.mark.parametrize("n", [2, 9, 13])
+def test_c64_probabilities_over_every_exponent(n):
+    """Pairs of any two exponents (zeros, subnormals, infinities and NaN among them),
+    with full, short and single-bit significands: p = x^2 + y^2 rounded once."""
+    g, N = rng(n), 1 << n
+    bits = g.integers(0, 1 << 32, (N, 2), dtype=np.uint64).astype(np.uint32)
+    near = g.random(N) < 0.6      # exponents within 30 of one another: every shift of the smaller square
+    e = (bits[:, 0] >> 23) & 255
+    other = np.clip(e.astype(int) + g.integers(-30, 31, N), 0, 255).astype(np.uint32)
+    bits[near, 1] = (bits[near, 1] & 0x807FFFFF) | (other[near] << 23)
+    for keep, mask in ((0.2, 0xFFFFF000), (0.2, 0xFF800001), (0.1, 0xFF800000)):
+        bits[g.random(N) < keep] &= np.uint32(mask)
+    bits[g.random((N, 2)) < 0.05] = 0
+    with np.errstate(all="ignore"):
+        psi = bits.view(np.float32).astype(np.float64).view(np.complex128).ravel()
+        want = psi.real ** 2 + psi.imag ** 2
+    h = qs.qs_alloc(n, qs.QS_C64)
+    try:
+        qs.qs_set_amplitudes(h, psi)
+        assert np.array_equal(qs.qs_probabilities(h), want, equal_nan=True)
+    finally:
+        qs.qs_free(h)
