@@ -203,7 +203,7 @@ struct qs_pass_op {
     uint8_t n_act;         // phase: CZ partner terms
     uint16_t bytes, at;    // operand size (a multiple of 16), its place in the CTA's operand buffer
     uint16_t n_stage;      // ops whose operands are brought in together before this one (0: it came in with another)
-    uint16_t pad;
+    uint16_t own;          // phase: threads keep to their own amplitudes on a small chunk
     uint64_t data;         // operand, device address
 };
 struct qs_pass {
@@ -221,6 +221,7 @@ struct qs_pass_in {
     const int *qubits;
     uint64_t data;
     uint32_t bytes;
+    bool odd;              // phase: some coefficient is odd
 };
 int qs_pass_bits(int dtype);   // most local bits
 // Ops in order, as many per pass as fit wmax local bits.
@@ -230,6 +231,13 @@ int qs_launch_pass(qs_state *s, const qs_pass &ps);
 int qs_launch_pass_items(int dtype, const void *passes, const void *items, uint32_t n, void *amp, int W, int cluster,
                          int threads, bool chain, void *stream);
 
+// A phase op with an odd coefficient (a factor that is no power of i).
+inline bool qs_phase_odd(const qs_op_host &op)
+{
+    for (int32_t c : op.coeff)
+        if (c & 1) return true;
+    return false;
+}
 // Pack a phase op into its device layout (qs_circuit.cpp).
 std::vector<uint8_t> qs_pack_phase(int n, const std::vector<int32_t> &coeff,
                                    const std::vector<std::pair<int, int>> &edges, int *n_act);

@@ -39,7 +39,9 @@ using qsd::cplx;
 template <typename R> constexpr int kRunBits = sizeof(R) == 4 ? 3 : 2;
 template <typename R> constexpr int kPassBits = sizeof(R) == 4 ? 13 : 12;    // most local bits
 template <typename R> constexpr int kOpBytes = 32 * 32 * 2 * (int)sizeof(R);  // operands held at a time
-constexpr int kOneThreads = 128;                                             // CTAs of a single state's passes
+template <typename R> constexpr int kOneThreads = sizeof(R) == 4 ? 128 : 256;   // a single state's passes
+
+constexpr int kFewTerms = 2, kFewRows = 8;   // phase ops evaluated amplitude by amplitude
 
 // Where local index l sits in shared memory: the upper bits are folded into the
 // bank bits (four of 8-byte, three of 16-byte elements), so that lanes that
@@ -177,7 +179,7 @@ __device__ __forceinline__ void dense_groups(typename cplx<R>::t *sm, int W, con
             v[x] = sm[o];
         }
         if (split) __syncthreads();   // every thread of a group has read it (one turn, all threads)
-#pragma unroll 1
+#pragma unroll (K <= 1 ? 2 : 1)
         for (int r = r0; r < r1; r++) {
             R ar = 0, ai = 0;
             const C *row = Us + r * D;
@@ -213,62 +215,80 @@ __device__ __forceinline__ void dense_chunk(typename cplx<R>::t *sm, int W, cons
     dense_groups<R, K, T>(sm, W, q, Us);
 }
 
+// The exponent of index i for a phase op of few CZ terms, term by term.
+__device__ __forceinline__ int phase_at(uint64_t i, const qs_phase_dev *ph, int n_act)
+{
+    const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
+    int m = __popcll(i & ph->cmask[0]) + 2 * __popcll(i & ph->cmask[1]) + 4 * __popcll(i & ph->cmask[2]);
+    for (int t = 0; t < n_act; t++) m += 4 * ((int)(i >> terms[t].a) & __popcll(i & terms[t].partners) & 1);
+    return m & 7;
+}
+
 // A phase product on the chunk.  The index splits into a column (as many local
 // bits as the CTA has threads), a row of the chunk and the chunk's base; with
 // m(x) the exponent of the bits x alone and M(x) the bits whose CZ partners meet
 // x an odd number of times,
 //   m(x | c) = m(x) + m(c) + 4 popc(c & M(x)),
 // x = base and row, formed by one thread per row.  complex128 pairs rows so that
-// one FP64 rotation serves two amplitudes, as k_phase does.
+// one FP64 rotation serves two amplitudes, as k_phase does.  On a small chunk (few
+// rows) an op of one or two CZ terms is evaluated amplitude by amplitude without
+// the rows' table and its barrier: with four or eight warps on an SM each
+// instruction's latency shows (83 gates on 16 qubits: 153 -> FIG us).
 template <typename R, int T>
 __device__ __forceinline__ void phase_chunk(typename cplx<R>::t *sm, int W, const LocalMap &map, uint64_t base,
                                             const qs_phase_dev *ph, int n_act, uint64_t *row_M, int *row_m)
 {
     using C = typename cplx<R>::t;
     constexpr int kT = T == 128 ? 7 : T == 256 ? 8 : 9;
-    const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
-    const uint64_t c0 = ph->cmask[0], c1 = ph->cmask[1], c2 = ph->cmask[2];
-    auto exponent = [&](uint64_t x, uint64_t &M) {
-        int m = __popcll(x & c0) + 2 * __popcll(x & c1) + 4 * __popcll(x & c2), par = 0;
-        M = 0;
-        for (int t = 0; t < n_act; t++) {
-            const uint64_t P = terms[t].partners;
-            const int a = terms[t].a, o = __popcll(x & P) & 1;
-            if ((x >> a) & 1) {
-                par ^= o;
-                M ^= P;
-            }
-            M ^= (uint64_t)o << a;
-        }
-        return m + 4 * par;
-    };
     const int tid = threadIdx.x, cb = min(W, kT), rows = 1 << (W - cb);
     const uint32_t col = (uint32_t)tid & ((1u << cb) - 1u);
-    const bool in = tid < (1 << cb);
-    uint64_t M;
-    if (tid < rows) {
-        row_m[tid] = exponent(base | map.at((uint32_t)tid << cb), M);
-        row_M[tid] = M;
-    }
-    const uint64_t xc = map.at(col);
-    const int mc = exponent(xc, M);
+    const bool in = tid < (1 << cb), direct = n_act <= kFewTerms && rows <= kFewRows;
+    const uint64_t c0 = ph->cmask[0], xc = map.at(col);
     uint32_t flip = 0;   // complex128: a lane bit whose coefficient is odd
     if constexpr (sizeof(R) == 8)
-        for (int j = min(cb, 5) - 1; j >= 0; j--)
-            if (map.at(1u << j) & c0) flip = 1u << j;
-    uint64_t xc2 = xc;
-    int mc2 = mc;
-    if (flip) {
-        xc2 = map.at(col ^ flip);
-        mc2 = exponent(xc2, M);
+        if (c0)
+            for (int j = min(cb, 5) - 1; j >= 0; j--)
+                if (map.at(1u << j) & c0) flip = 1u << j;
+    const uint64_t xc2 = flip ? map.at(col ^ flip) : xc;
+    int mc = 0, mc2 = 0;
+    if (!direct) {
+        const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
+        const uint64_t c1 = ph->cmask[1], c2 = ph->cmask[2];
+        auto exponent = [&](uint64_t x, uint64_t &M) {
+            int m = __popcll(x & c0) + 2 * __popcll(x & c1) + 4 * __popcll(x & c2), par = 0;
+            M = 0;
+            for (int t = 0; t < n_act; t++) {
+                const uint64_t P = terms[t].partners;
+                const int a = terms[t].a, o = __popcll(x & P) & 1;
+                if ((x >> a) & 1) {
+                    par ^= o;
+                    M ^= P;
+                }
+                M ^= (uint64_t)o << a;
+            }
+            return m + 4 * par;
+        };
+        uint64_t M;
+        if (tid < rows) {
+            row_m[tid] = exponent(base | map.at((uint32_t)tid << cb), M);
+            row_M[tid] = M;
+        }
+        mc = exponent(xc, M);
+        if (flip) mc2 = exponent(xc2, M);
+        __syncthreads();
     }
-    __syncthreads();
+    // exponent at row r and this thread's column (or the flipped one)
+    auto at = [&](int r, bool other) {
+        const uint64_t x = other ? xc2 : xc;
+        if (direct) return phase_at(base | map.at((uint32_t)r << cb) | x, ph, n_act);
+        return ((other ? mc2 : mc) + row_m[r] + 4 * __popcll(x & row_M[r])) & 7;
+    };
     if (flip && rows > 1) {
         for (int r = 0; r < rows; r += 2) {
-            const int ma = (mc + row_m[r] + 4 * __popcll(xc & row_M[r])) & 7;
+            const int ma = at(r, false);
             // the second row's column: exactly one of the two amplitudes is odd
-            const bool other = !((row_m[r] ^ row_m[r + 1]) & 1);
-            const int mb = ((other ? mc2 : mc) + row_m[r + 1] + 4 * __popcll((other ? xc2 : xc) & row_M[r + 1])) & 7;
+            const bool other = direct ? !(__popcll(map.at((uint32_t)1 << cb) & c0) & 1) : !((row_m[r] ^ row_m[r + 1]) & 1);
+            const int mb = at(r + 1, other);
             C *pa = sm + place<R>(((uint32_t)r << cb) | col);
             C *pb = sm + place<R>(((uint32_t)(r + 1) << cb) | (other ? col ^ flip : col));
             if (!in) continue;
@@ -282,9 +302,9 @@ __device__ __forceinline__ void phase_chunk(typename cplx<R>::t *sm, int W, cons
         return;
     }
     for (int r = 0; r < rows; r++) {
-        const int m = (mc + row_m[r] + 4 * __popcll(xc & row_M[r])) & 7;
+        const int m = at(r, false);
         C *p = sm + place<R>(((uint32_t)r << cb) | col);
-        if (m && in) *p = qsd::rotate8<C, R>(*p, m);
+        if (m && in) *p = c0 ? qsd::rotate8<C, R>(*p, m) : qsd::quarter_turns<C>(*p, m >> 1);
     }
 }
 
@@ -389,6 +409,8 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
             }
         } else {
             phase_chunk<R, T>(sm, W, map, base, reinterpret_cast<const qs_phase_dev *>(data), op.n_act, row_M, row_m);
+            // the next op's threads keep to the same amplitudes: no barrier
+            if (op.own && o + 1 < ps.n_ops && ps.op[o + 1].own && !ps.op[o + 1].n_stage && (1 << W) <= kFewRows * T) continue;
         }
         __syncthreads();
     }
@@ -407,12 +429,12 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
 
 // One state: the pass in the launch's parameters, a CTA per chunk.
 template <typename R>
-__global__ void __launch_bounds__(kOneThreads, sizeof(R) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(kOneThreads<R>, sizeof(R) == 4 ? 3 : 1)
 k_pass(const __grid_constant__ qs_pass ps, typename cplx<R>::t *__restrict__ psi)
 {
     extern __shared__ __align__(16) uint8_t smem[];
     chain_start();
-    run_chunk<R, kOneThreads>(ps, psi, blockIdx.x, smem, [] { chain_wait(); });
+    run_chunk<R, kOneThreads<R>>(ps, psi, blockIdx.x, smem, [] { chain_wait(); });
 }
 
 // Many states: items[i] = (pass, chunk).
@@ -457,7 +479,7 @@ int launch_pass_r(qs_state *s, const qs_pass &ps)
 {
     static bool ready[64] = {};
     if (int rc = allow_smem(k_pass<R>, pass_smem<R>(kPassBits<R>), ready)) return rc;
-    const cudaError_t e = launch_sweep(s, k_pass<R>, 1 << (s->n - ps.W), kOneThreads, pass_smem<R>(ps.W), ps,
+    const cudaError_t e = launch_sweep(s, k_pass<R>, 1 << (s->n - ps.W), kOneThreads<R>, pass_smem<R>(ps.W), ps,
                                        reinterpret_cast<typename cplx<R>::t *>(s->amp));
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_pass launch: %s", cudaGetErrorString(e));
 }
@@ -537,6 +559,8 @@ std::vector<qs_pass> qs_plan_passes(int n, int dtype, int wmax, const std::vecto
             op.kind = (uint8_t)in.kind;
             op.k = (uint8_t)in.k;
             op.n_act = (uint8_t)in.n_act;
+            // evaluated amplitude by amplitude, each by its own thread (no rows paired over columns)
+            op.own = in.kind == QS_OP_PHASE && in.n_act <= kFewTerms && (dtype == QS_C64 || !in.odd);
             op.bytes = (uint16_t)in.bytes;
             op.data = in.data;
             if (in.kind == QS_OP_DENSE)
