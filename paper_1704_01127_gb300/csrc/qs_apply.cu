@@ -742,7 +742,7 @@ int run_passes(qs_state *s, const qs_schedule *sc, const qs_dev_sched &d, size_t
                                  ? op.matrix.size() * (s->dtype == QS_C128 ? sizeof(double) : sizeof(float))
                                  : sizeof(qs_phase_dev) + sizeof(qs_phase_term) * (size_t)d.n_act[j];
         in.push_back({op.kind, op.k, d.n_act[j], op.qubits, (uint64_t)(uintptr_t)d.pool + d.offset[j], (uint32_t)bytes,
-                      qs_phase_odd(op)});
+                      &op});
     }
     if (in.size() < 2) return QS_OK;
     const int wmax = std::max(8, std::min(qs_pass_bits(s->dtype), s->n - 7));

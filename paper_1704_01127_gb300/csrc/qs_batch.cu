@@ -234,7 +234,7 @@ extern "C" int qs_batch_create(int n_circ, const qs_schedule *const *scheds, int
                 } else {
                     return qs_fail(QS_EUNSUPPORTED, "qs_batch_create: table diagonals are not batched");
                 }
-                in[c].push_back({op.kind, op.k, n_act, op.qubits, at, (uint32_t)(pool.size() - at), qs_phase_odd(op)});
+                in[c].push_back({op.kind, op.k, n_act, op.qubits, at, (uint32_t)(pool.size() - at), &op});
             }
         }
         int rc = QS_OK;

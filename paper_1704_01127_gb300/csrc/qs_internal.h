@@ -197,14 +197,15 @@ bool qs_tc_wanted(int dtype, int k, int n);
 
 // Passes (qs_pass.cu): consecutive CUDA-core ops in one read and write of the state.
 constexpr int QS_PASS_OPS = 32;
+constexpr int QS_PASS_TURN = 16;   // a pass's op kind besides QS_OP_*: one factor of a phase product
 struct qs_pass_op {
-    uint8_t kind, k;       // QS_OP_DENSE or QS_OP_PHASE
-    uint8_t q[QS_MAX_K];   // dense: target j as a bit of the chunk's local index
-    uint8_t n_act;         // phase: CZ partner terms
+    uint8_t kind, k;       // QS_OP_DENSE, QS_OP_PHASE or QS_PASS_TURN
+    uint8_t q[QS_MAX_K];   // dense, turn: target j as a bit of the chunk's local index (ascending)
+    uint8_t n_act;         // phase: CZ partner terms; turn: eighths of a turn
     uint16_t bytes, at;    // operand size (a multiple of 16), its place in the CTA's operand buffer
     uint16_t n_stage;      // ops whose operands are brought in together before this one (0: it came in with another)
-    uint16_t own;          // phase: threads keep to their own amplitudes on a small chunk
-    uint64_t data;         // operand, device address
+    uint16_t pad;
+    uint64_t data;         // operand, device address; a turn: its index bits outside the chunk
 };
 struct qs_pass {
     uint64_t local;        // index bits inside a chunk
@@ -221,7 +222,7 @@ struct qs_pass_in {
     const int *qubits;
     uint64_t data;
     uint32_t bytes;
-    bool odd;              // phase: some coefficient is odd
+    const qs_op_host *op;
 };
 int qs_pass_bits(int dtype);   // most local bits
 // Ops in order, as many per pass as fit wmax local bits.
@@ -231,13 +232,6 @@ int qs_launch_pass(qs_state *s, const qs_pass &ps);
 int qs_launch_pass_items(int dtype, const void *passes, const void *items, uint32_t n, void *amp, int W, int cluster,
                          int threads, bool chain, void *stream);
 
-// A phase op with an odd coefficient (a factor that is no power of i).
-inline bool qs_phase_odd(const qs_op_host &op)
-{
-    for (int32_t c : op.coeff)
-        if (c & 1) return true;
-    return false;
-}
 // Pack a phase op into its device layout (qs_circuit.cpp).
 std::vector<uint8_t> qs_pack_phase(int n, const std::vector<int32_t> &coeff,
                                    const std::vector<std::pair<int, int>> &edges, int *n_act);

@@ -19,9 +19,13 @@
 // 128 registers of amplitudes).  Packed FP32 FMAs (fma.rn.f32x2) measured slower:
 // they need U's elements twice over, from shared memory or by moves.
 // 96 circuits of 16 to 21 qubits, k <= 4, complex64 (102 GFMA, 2.7 ms of the FMA
-// pipe; one cluster of CTAs per circuit before): 26.3 -> 7.0 ms, two thirds of the
-// issue slots used, half of them by FMAs.  A plain circuit
-// of 83 gates on 16 qubits, complex128: 320 -> 153 us (a sweep per gate before).
+// pipe; one cluster of CTAs per circuit before): 26.3 -> 6.0 ms, two thirds of the
+// issue slots used, two thirds of them by FMAs.  What the kernel holds across an op
+// has to stay out of the registers (spills inside the rows: 6.9 ms).  A plain circuit
+// of 83 gates on 16 qubits, complex128: 320 -> 98 us (a sweep per gate before); there
+// a chunk has 512 amplitudes and the instructions' latency shows, so gates that are one
+// factor of a phase product visit just the amplitudes they turn (115 us with an exponent
+// for every amplitude).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,8 +44,6 @@ template <typename R> constexpr int kRunBits = sizeof(R) == 4 ? 3 : 2;
 template <typename R> constexpr int kPassBits = sizeof(R) == 4 ? 13 : 12;    // most local bits
 template <typename R> constexpr int kOpBytes = 32 * 32 * 2 * (int)sizeof(R);  // operands held at a time
 template <typename R> constexpr int kOneThreads = sizeof(R) == 4 ? 128 : 256;   // a single state's passes
-
-constexpr int kFewTerms = 2, kFewRows = 8;   // phase ops evaluated amplitude by amplitude
 
 // Where local index l sits in shared memory: the upper bits are folded into the
 // bank bits (four of 8-byte, three of 16-byte elements), so that lanes that
@@ -66,6 +68,7 @@ __device__ __forceinline__ uint64_t deposit(uint64_t x, uint64_t mask)
 // Index bits of the local bits above the runs, six at a time.
 struct LocalMap {
     uint64_t lo[64], hi[64];
+    uint64_t base;   // the chunk's own index bits; here, not in registers that the ops need
     int rb;
     __device__ __forceinline__ uint64_t at(uint32_t l) const
     {
@@ -121,22 +124,33 @@ __device__ __forceinline__ void dense_groups_g(float2 *sm, int W, const int *q, 
                 v[i][x] = sm[pb[i] ^ o];
             }
         }
+        // U's elements two at a time, four ahead (past the last row: the chunk's first
+        // bytes, unused)
+        const float4 *u = reinterpret_cast<const float4 *>(Us);
+        float4 next = u[0], next2 = *++u;
 #pragma unroll 1
         for (int r = 0; r < D; r++) {
             float ar[G], ai[G];
 #pragma unroll
             for (int i = 0; i < G; i++) ar[i] = ai[i] = 0;
-            const float4 *row = reinterpret_cast<const float4 *>(Us + r * D);
 #pragma unroll
-            for (int x = 0; x < D; x++) {
-                const float4 w = row[x >> 1];
-                const float mx = x & 1 ? w.z : w.x, my = x & 1 ? w.w : w.y;
+            for (int x = 0; x < D; x += 2) {
+                const float4 w = next;
+                next = next2;
+                next2 = *++u;
 #pragma unroll
                 for (int i = 0; i < G; i++) {
-                    ar[i] = fmaf(v[i][x].x, mx, ar[i]);
-                    ai[i] = fmaf(v[i][x].y, mx, ai[i]);
-                    ar[i] = fnma(v[i][x].y, my, ar[i]);
-                    ai[i] = fmaf(v[i][x].x, my, ai[i]);
+                    ar[i] = fmaf(v[i][x].x, w.x, ar[i]);
+                    ai[i] = fmaf(v[i][x].y, w.x, ai[i]);
+                    ar[i] = fnma(v[i][x].y, w.y, ar[i]);
+                    ai[i] = fmaf(v[i][x].x, w.y, ai[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < G; i++) {
+                    ar[i] = fmaf(v[i][x + 1].x, w.z, ar[i]);
+                    ai[i] = fmaf(v[i][x + 1].y, w.z, ai[i]);
+                    ar[i] = fnma(v[i][x + 1].y, w.w, ar[i]);
+                    ai[i] = fmaf(v[i][x + 1].x, w.w, ai[i]);
                 }
             }
             uint32_t o = 0;
@@ -215,80 +229,62 @@ __device__ __forceinline__ void dense_chunk(typename cplx<R>::t *sm, int W, cons
     dense_groups<R, K, T>(sm, W, q, Us);
 }
 
-// The exponent of index i for a phase op of few CZ terms, term by term.
-__device__ __forceinline__ int phase_at(uint64_t i, const qs_phase_dev *ph, int n_act)
-{
-    const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
-    int m = __popcll(i & ph->cmask[0]) + 2 * __popcll(i & ph->cmask[1]) + 4 * __popcll(i & ph->cmask[2]);
-    for (int t = 0; t < n_act; t++) m += 4 * ((int)(i >> terms[t].a) & __popcll(i & terms[t].partners) & 1);
-    return m & 7;
-}
-
 // A phase product on the chunk.  The index splits into a column (as many local
 // bits as the CTA has threads), a row of the chunk and the chunk's base; with
 // m(x) the exponent of the bits x alone and M(x) the bits whose CZ partners meet
 // x an odd number of times,
 //   m(x | c) = m(x) + m(c) + 4 popc(c & M(x)),
 // x = base and row, formed by one thread per row.  complex128 pairs rows so that
-// one FP64 rotation serves two amplitudes, as k_phase does.  On a small chunk (few
-// rows) an op of one or two CZ terms is evaluated amplitude by amplitude without
-// the rows' table and its barrier: with four or eight warps on an SM each
-// instruction's latency shows (83 gates on 16 qubits: 153 -> FIG us).
+// one FP64 rotation serves two amplitudes, as k_phase does.
 template <typename R, int T>
 __device__ __forceinline__ void phase_chunk(typename cplx<R>::t *sm, int W, const LocalMap &map, uint64_t base,
                                             const qs_phase_dev *ph, int n_act, uint64_t *row_M, int *row_m)
 {
     using C = typename cplx<R>::t;
     constexpr int kT = T == 128 ? 7 : T == 256 ? 8 : 9;
+    const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
+    const uint64_t c0 = ph->cmask[0], c1 = ph->cmask[1], c2 = ph->cmask[2];
+    auto exponent = [&](uint64_t x, uint64_t &M) {
+        int m = __popcll(x & c0) + 2 * __popcll(x & c1) + 4 * __popcll(x & c2), par = 0;
+        M = 0;
+        for (int t = 0; t < n_act; t++) {
+            const uint64_t P = terms[t].partners;
+            const int a = terms[t].a, o = __popcll(x & P) & 1;
+            if ((x >> a) & 1) {
+                par ^= o;
+                M ^= P;
+            }
+            M ^= (uint64_t)o << a;
+        }
+        return m + 4 * par;
+    };
     const int tid = threadIdx.x, cb = min(W, kT), rows = 1 << (W - cb);
     const uint32_t col = (uint32_t)tid & ((1u << cb) - 1u);
-    const bool in = tid < (1 << cb), direct = n_act <= kFewTerms && rows <= kFewRows;
-    const uint64_t c0 = ph->cmask[0], xc = map.at(col);
+    const bool in = tid < (1 << cb);
+    uint64_t M;
+    if (tid < rows) {
+        row_m[tid] = exponent(base | map.at((uint32_t)tid << cb), M);
+        row_M[tid] = M;
+    }
+    const uint64_t xc = map.at(col);
+    const int mc = exponent(xc, M);
     uint32_t flip = 0;   // complex128: a lane bit whose coefficient is odd
     if constexpr (sizeof(R) == 8)
-        if (c0)
-            for (int j = min(cb, 5) - 1; j >= 0; j--)
-                if (map.at(1u << j) & c0) flip = 1u << j;
-    const uint64_t xc2 = flip ? map.at(col ^ flip) : xc;
-    int mc = 0, mc2 = 0;
-    if (!direct) {
-        const qs_phase_term *terms = reinterpret_cast<const qs_phase_term *>(ph + 1);
-        const uint64_t c1 = ph->cmask[1], c2 = ph->cmask[2];
-        auto exponent = [&](uint64_t x, uint64_t &M) {
-            int m = __popcll(x & c0) + 2 * __popcll(x & c1) + 4 * __popcll(x & c2), par = 0;
-            M = 0;
-            for (int t = 0; t < n_act; t++) {
-                const uint64_t P = terms[t].partners;
-                const int a = terms[t].a, o = __popcll(x & P) & 1;
-                if ((x >> a) & 1) {
-                    par ^= o;
-                    M ^= P;
-                }
-                M ^= (uint64_t)o << a;
-            }
-            return m + 4 * par;
-        };
-        uint64_t M;
-        if (tid < rows) {
-            row_m[tid] = exponent(base | map.at((uint32_t)tid << cb), M);
-            row_M[tid] = M;
-        }
-        mc = exponent(xc, M);
-        if (flip) mc2 = exponent(xc2, M);
-        __syncthreads();
+        for (int j = min(cb, 5) - 1; j >= 0; j--)
+            if (map.at(1u << j) & c0) flip = 1u << j;
+    uint64_t xc2 = xc;
+    int mc2 = mc;
+    if (flip) {
+        xc2 = map.at(col ^ flip);
+        mc2 = exponent(xc2, M);
     }
-    // exponent at row r and this thread's column (or the flipped one)
-    auto at = [&](int r, bool other) {
-        const uint64_t x = other ? xc2 : xc;
-        if (direct) return phase_at(base | map.at((uint32_t)r << cb) | x, ph, n_act);
-        return ((other ? mc2 : mc) + row_m[r] + 4 * __popcll(x & row_M[r])) & 7;
-    };
+    __syncthreads();
     if (flip && rows > 1) {
         for (int r = 0; r < rows; r += 2) {
-            const int ma = at(r, false);
+            const int ma = (mc + row_m[r] + 4 * __popcll(xc & row_M[r])) & 7;
             // the second row's column: exactly one of the two amplitudes is odd
-            const bool other = direct ? !(__popcll(map.at((uint32_t)1 << cb) & c0) & 1) : !((row_m[r] ^ row_m[r + 1]) & 1);
-            const int mb = at(r + 1, other);
+            const bool other = !((row_m[r] ^ row_m[r + 1]) & 1);
+            const int mb = ((other ? mc2 : mc) + row_m[r + 1] + 4 * __popcll((other ? xc2 : xc) & row_M[r + 1])) & 7;
             C *pa = sm + place<R>(((uint32_t)r << cb) | col);
             C *pb = sm + place<R>(((uint32_t)(r + 1) << cb) | (other ? col ^ flip : col));
             if (!in) continue;
@@ -302,9 +298,29 @@ __device__ __forceinline__ void phase_chunk(typename cplx<R>::t *sm, int W, cons
         return;
     }
     for (int r = 0; r < rows; r++) {
-        const int m = at(r, false);
+        const int m = (mc + row_m[r] + 4 * __popcll(xc & row_M[r])) & 7;
         C *p = sm + place<R>(((uint32_t)r << cb) | col);
-        if (m && in) *p = c0 ? qsd::rotate8<C, R>(*p, m) : qsd::quarter_turns<C>(*p, m >> 1);
+        if (m && in) *p = qsd::rotate8<C, R>(*p, m);
+    }
+}
+
+// One factor of a phase op by itself (a T-type gate on one qubit, a CZ): the
+// amplitudes whose k (0, 1 or 2) local bits q are set turn by c eighths.  Only those
+// are visited, and every lane of an odd turn's FP64 instructions has work.
+template <typename R, int T>
+__device__ __forceinline__ void turn_chunk(typename cplx<R>::t *sm, int W, int k, int q0, int q1, int c)
+{
+    using C = typename cplx<R>::t;
+    auto with_bit = [](uint32_t l, int q) {
+        const uint32_t lo = l & ((1u << q) - 1u);
+        return ((l ^ lo) << 1) | lo | 1u << q;
+    };
+    for (uint32_t h = threadIdx.x; h < (1u << (W - k)); h += T) {
+        uint32_t l = h;
+        if (k > 0) l = with_bit(l, q0);
+        if (k > 1) l = with_bit(l, q1);
+        C *p = sm + place<R>(l);
+        *p = qsd::rotate8<C, R>(*p, c);
     }
 }
 
@@ -346,15 +362,18 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
         }
         if (tid < 64) map.lo[tid] = deposit(tid, lo6);
         else if (tid < 128) map.hi[tid - 64] = deposit(tid - 64, hi);
-        if (tid == 0) map.rb = rb;
+        if (tid == 0) {
+            map.rb = rb;
+            map.base = deposit(ch, ps.outer);
+        }
     }
-    const uint64_t base = deposit(ch, ps.outer), outside = ~ps.support;
-    C *p = psi + base;
     __syncthreads();
     wait();
     // 16 bytes an access: two complex64 amplitudes (bit 0 is always local)
     constexpr int VEC = sizeof(R) == 4 ? 2 : 1, kAhead = 8;
     const uint32_t units = (1u << W) / VEC;
+    const uint64_t outside = ~ps.support;
+    const C *from = psi + ps.amp + map.base;
     for (uint32_t u0 = tid; u0 < units; u0 += T * kAhead) {
         uint4 z[kAhead];
 #pragma unroll
@@ -371,7 +390,7 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
                     *reinterpret_cast<C *>(&z[k]) = one;
                 }
             } else if (!(o & outside)) {
-                z[k] = __ldcg(reinterpret_cast<const uint4 *>(p + o));
+                z[k] = __ldcg(reinterpret_cast<const uint4 *>(from + o));
             }
         }
 #pragma unroll
@@ -396,10 +415,10 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
         }
         const void *data = operands + op.at;
         if (op.kind == QS_OP_DENSE) {
-            const C *U = reinterpret_cast<const C *>(data);
             int q[QS_MAX_K];
 #pragma unroll
             for (int j = 0; j < QS_MAX_K; j++) q[j] = op.q[j];
+            const C *U = reinterpret_cast<const C *>(data);
             switch (op.k) {
             case 1: dense_chunk<R, 1, T>(sm, W, q, U); break;
             case 2: dense_chunk<R, 2, T>(sm, W, q, U); break;
@@ -407,13 +426,15 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
             case 4: dense_chunk<R, 4, T>(sm, W, q, U); break;
             default: dense_chunk<R, 5, T>(sm, W, q, U); break;
             }
+        } else if (op.kind == QS_PASS_TURN) {
+            if ((map.base & op.data) != op.data) continue;   // the factor's bits outside the chunk: the same for all of it
+            turn_chunk<R, T>(sm, W, op.k, op.q[0], op.q[1], op.n_act);
         } else {
-            phase_chunk<R, T>(sm, W, map, base, reinterpret_cast<const qs_phase_dev *>(data), op.n_act, row_M, row_m);
-            // the next op's threads keep to the same amplitudes: no barrier
-            if (op.own && o + 1 < ps.n_ops && ps.op[o + 1].own && !ps.op[o + 1].n_stage && (1 << W) <= kFewRows * T) continue;
+            phase_chunk<R, T>(sm, W, map, map.base, reinterpret_cast<const qs_phase_dev *>(data), op.n_act, row_M, row_m);
         }
         __syncthreads();
     }
+    C *to = psi + ps.amp + map.base;
     for (uint32_t u = tid; u < units; u += T) {
         const uint32_t l = place<R>(VEC * u);
         uint4 z;
@@ -423,7 +444,7 @@ __device__ __forceinline__ void run_chunk(const qs_pass &ps, typename cplx<R>::t
         } else {
             z = reinterpret_cast<const uint4 *>(sm)[l];
         }
-        *reinterpret_cast<uint4 *>(p + map.at(VEC * u)) = z;
+        *reinterpret_cast<uint4 *>(to + map.at(VEC * u)) = z;
     }
 }
 
@@ -454,7 +475,7 @@ k_pass_items(const qs_pass *__restrict__ passes, const uint2 *__restrict__ items
         for (int i = threadIdx.x; i < (int)(sizeof(qs_pass) / 4); i += T) dst[i] = src[i];
     }
     __syncthreads();
-    run_chunk<R, T>(ps, amp + ps.amp, it.y, smem, [] { chain_wait(); });
+    run_chunk<R, T>(ps, amp, it.y, smem, [] { chain_wait(); });
 }
 
 template <typename R>
@@ -519,6 +540,20 @@ int launch_items_r(const qs_pass *passes, const uint2 *items, uint32_t n, void *
 
 }  // namespace
 
+// A phase op that is one factor: e^{i pi turns / 4} where the one or two index bits
+// `bits` are set (a coefficient, or a CZ pair).
+static bool single_factor(int n, const qs_op_host &op, uint64_t *bits, int *turns)
+{
+    uint64_t coeff = 0;
+    for (int q = 0; q < n; q++)
+        if (op.coeff[q] & 7) coeff |= 1ULL << q;
+    const int nc = __builtin_popcountll(coeff);
+    if (nc + (int)op.edges.size() != 1) return false;
+    *bits = nc ? coeff : 1ULL << op.edges[0].first | 1ULL << op.edges[0].second;
+    *turns = nc ? op.coeff[__builtin_ctzll(coeff)] & 7 : 4;
+    return true;
+}
+
 int qs_pass_bits(int dtype) { return dtype == QS_C128 ? kPassBits<double> : kPassBits<float>; }
 
 std::vector<qs_pass> qs_plan_passes(int n, int dtype, int wmax, const std::vector<qs_pass_in> &ops, bool from_basis)
@@ -559,13 +594,22 @@ std::vector<qs_pass> qs_plan_passes(int n, int dtype, int wmax, const std::vecto
             op.kind = (uint8_t)in.kind;
             op.k = (uint8_t)in.k;
             op.n_act = (uint8_t)in.n_act;
-            // evaluated amplitude by amplitude, each by its own thread (no rows paired over columns)
-            op.own = in.kind == QS_OP_PHASE && in.n_act <= kFewTerms && (dtype == QS_C64 || !in.odd);
             op.bytes = (uint16_t)in.bytes;
             op.data = in.data;
+            auto local = [&](int b) { return (uint8_t)__builtin_popcountll(mask & ((1ULL << b) - 1)); };
             if (in.kind == QS_OP_DENSE)
-                for (int j = 0; j < in.k; j++) op.q[j] = (uint8_t)__builtin_popcountll(mask & ((1ULL << in.qubits[j]) - 1));
-            const uint32_t need = (in.bytes + 15u) & ~15u;
+                for (int j = 0; j < in.k; j++) op.q[j] = local(in.qubits[j]);
+            uint64_t bits;
+            int turns;
+            if (in.kind == QS_OP_PHASE && single_factor(n, *in.op, &bits, &turns)) {
+                op.kind = QS_PASS_TURN;
+                op.n_act = (uint8_t)turns;
+                op.bytes = 0;
+                op.data = bits & ~mask;
+                op.k = 0;
+                for (uint64_t x = bits & mask; x; x &= x - 1) op.q[op.k++] = local(__builtin_ctzll(x));
+            }
+            const uint32_t need = (op.bytes + 15u) & ~15u;
             if (at + need > op_bytes) {
                 at = 0;
                 batch = o;
