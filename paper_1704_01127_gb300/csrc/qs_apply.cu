@@ -50,9 +50,26 @@ k_dense(typename cplx<R>::t *__restrict__ psi, uint64_t n_groups, Targets t,
         Us[i] = reinterpret_cast<const C *>(Ug)[i];
     __syncthreads();
     chain_wait();
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_groups; g += stride)
-        qsd::dense_group<R, K, false>(psi + group_base<K>(g, t), t, Us);
+    // complex64, k = 1: four groups' loads in flight per thread (28 qubits: 787 -> 661
+    // us); with more members a group has enough of them (k = 2: 643 us, 684 with two
+    // groups), and complex128 is bound by the FP64 pipe
+    constexpr int G = sizeof(R) == 4 && K == 1 ? 4 : 1;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * G;
+    for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x * G + threadIdx.x; g < n_groups; g += stride) {
+        if constexpr (G == 1) {
+            qsd::dense_group<R, K, false>(psi + group_base<K>(g, t), t, Us);
+        } else {
+            C *p[G], v[G][D];
+#pragma unroll
+            for (int i = 0; i < G; i++) {
+                p[i] = psi + group_base<K>(min(g + (uint64_t)i * blockDim.x, n_groups - 1), t);
+                qsd::dense_load<R, K, false>(p[i], t, v[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < G; i++)
+                if (g + (uint64_t)i * blockDim.x < n_groups) qsd::dense_rows<R, K>(p[i], t, Us, v[i]);
+        }
+    }
 }
 
 // The diagonal sweeps split an index into a column (the kDiagRowBits lowest

@@ -54,14 +54,18 @@ __device__ __forceinline__ C ld(const C *p)
 // CG: loads bypass L1 (the batched kernel shares states between the CTAs of a
 // cluster).
 template <typename R, int K, bool CG>
-__device__ __forceinline__ void dense_group(typename cplx<R>::t *p, const Targets &t,
-                                            const typename cplx<R>::t *Us)
+__device__ __forceinline__ void dense_load(const typename cplx<R>::t *p, const Targets &t, typename cplx<R>::t *v)
+{
+#pragma unroll
+    for (int x = 0; x < (1 << K); x++) v[x] = ld<CG>(p + member_offset<K>(x, t));
+}
+
+template <typename R, int K>
+__device__ __forceinline__ void dense_rows(typename cplx<R>::t *p, const Targets &t, const typename cplx<R>::t *Us,
+                                           const typename cplx<R>::t *v)
 {
     using C = typename cplx<R>::t;
     constexpr int D = 1 << K;
-    C v[D];
-#pragma unroll
-    for (int x = 0; x < D; x++) v[x] = ld<CG>(p + member_offset<K>(x, t));
     // rows of U one at a time (kept rolled so v[] stays in registers)
 #pragma unroll 1
     for (int l = 0; l < D; l++) {
@@ -80,6 +84,15 @@ __device__ __forceinline__ void dense_group(typename cplx<R>::t *p, const Target
         o.y = ai;
         p[member_offset<K>(l, t)] = o;
     }
+}
+
+template <typename R, int K, bool CG>
+__device__ __forceinline__ void dense_group(typename cplx<R>::t *p, const Targets &t,
+                                            const typename cplx<R>::t *Us)
+{
+    typename cplx<R>::t v[1 << K];
+    dense_load<R, K, CG>(p, t, v);
+    dense_rows<R, K>(p, t, Us, v);
 }
 
 // Multiply by e^{i pi m / 4}: an odd m first takes one factor
