@@ -37,7 +37,14 @@ constexpr size_t kSmemF32 = 2 * kTileBytesF32 + 2 * kBBytesF32;
 // One CTA of 128 threads; thread r owns row r (group) of each tile.  Tiles are
 // taken in a grid-stride loop; warp 0 holds 128 TMEM columns for the CTA.
 // kPost: a phase op folded into the sweep is applied to the outputs.
-template <bool kPost>
+// kTwo (bit 0 numbers groups, no partial tile): rows 2 i and 2 i + 1 are neighbours in
+// memory, so thread (i, h) loads half of their members, 16 bytes (both rows) at a time.
+// The threads of rows 8 i' + 4 .. 7 write their second row first, so that eight
+// neighbouring threads' 16-byte stores fall in different banks.  With a low target
+// (t.join) the outputs leave in 16-byte stores too, two members exchanged between the
+// threads of neighbouring rows.  28 qubits: targets 1, 2, 11, 26, 27 1004 -> 838 us;
+// 1, 9, 15, 20, 22 776 -> 733; 1 to 5 1320 -> 1172.
+template <bool kPost, bool kTwo>
 __global__ void __launch_bounds__(128, 2)
 k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const float *__restrict__ bpack,
                 const qs_post_phase *__restrict__ post, int *__restrict__ status)
@@ -80,15 +87,25 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
     uint32_t parity = 0;
     // software pipeline: the next tile's amplitudes are loaded into registers
     // while the tensor cores work on the current one
-    float2 v[32];
+    float2 v[32];   // kTwo: v[2 x], v[2 x + 1]: member 16 h + x of the row written first and of the other
     uint64_t tile = blockIdx.x;
     bool valid = false;
     float2 *p = psi;
+    const int pi = tid & 63, ph = tid >> 6, second = (pi >> 2) & 1;   // kTwo
     auto load_tile = [&](uint64_t tl, float2 *vv, bool &val, float2 *&pp) {
-        const uint64_t g = tl * kRows + tid;
+        const uint64_t g = tl * kRows + (kTwo ? 2 * pi : tid);
         val = tl < n_tiles && g < n_groups;
         pp = psi + (val ? tile_base(g, t) : 0);
-        if (t.pairs) {
+        if constexpr (kTwo) {
+            const uint32_t in = val ? t.mmask >> (16 * ph) : 0u;
+            const float2 *from = pp + (ph ? 1ULL << t.q[4] : 0);
+#pragma unroll
+            for (int x = 0; x < 16; x++) {
+                const float4 w = (in >> x) & 1 ? *reinterpret_cast<const float4 *>(from + off5(x, t)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                vv[2 * x] = second ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+                vv[2 * x + 1] = second ? make_float2(w.x, w.y) : make_float2(w.z, w.w);
+            }
+        } else if (t.pairs) {
             // members 2i and 2i+1 differ in qubit 0: one 16-byte load each
             // (a member outside the support is read but replaced by zero)
 #pragma unroll
@@ -102,17 +119,25 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
             for (int x = 0; x < 32; x++) vv[x] = val && ((t.mmask >> x) & 1) ? pp[off5(x, t)] : make_float2(0.f, 0.f);
         }
     };
+    auto split = [&](int row, int c, float2 v0, float2 v1) {
+        float4 h = make_float4(tf32_head(v0.x), tf32_head(v0.y), tf32_head(v1.x), tf32_head(v1.y));
+        float4 tl = make_float4(tf32_round(v0.x - h.x), tf32_round(v0.y - h.y), tf32_round(v1.x - h.z),
+                                tf32_round(v1.y - h.w));
+        *reinterpret_cast<float4 *>(A_h + cm_off(row, 4 * c)) = h;
+        *reinterpret_cast<float4 *>(A_t + cm_off(row, 4 * c)) = tl;
+    };
     load_tile(tile, v, valid, p);
     for (; tile < n_tiles; tile += gridDim.x) {
         // split: members 2c and 2c+1 fill K columns 4c..4c+3
+        if constexpr (kTwo) {
 #pragma unroll
-        for (int c = 0; c < 16; c++) {
-            const float2 v0 = v[2 * c], v1 = v[2 * c + 1];
-            float4 h = make_float4(tf32_head(v0.x), tf32_head(v0.y), tf32_head(v1.x), tf32_head(v1.y));
-            float4 tl = make_float4(tf32_round(v0.x - h.x), tf32_round(v0.y - h.y), tf32_round(v1.x - h.z),
-                                    tf32_round(v1.y - h.w));
-            *reinterpret_cast<float4 *>(A_h + cm_off(tid, 4 * c)) = h;
-            *reinterpret_cast<float4 *>(A_t + cm_off(tid, 4 * c)) = tl;
+            for (int c = 0; c < 8; c++) {
+                split(2 * pi + second, 8 * ph + c, v[4 * c], v[4 * c + 2]);
+                split(2 * pi + 1 - second, 8 * ph + c, v[4 * c + 1], v[4 * c + 3]);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 16; c++) split(tid, c, v[2 * c], v[2 * c + 1]);
         }
         fence_proxy_async();
         tc_fence_before();
@@ -131,7 +156,7 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
             }
             mma_commit(mbar_a);
         }
-        float2 *const p_cur = p;
+        float2 *const p_cur = kTwo ? psi + tile_base(tile * kRows + tid, t) : p;   // this thread's row
         const bool valid_cur = valid;
         load_tile(tile + gridDim.x, v, valid, p);
         bool ok = false;
@@ -167,7 +192,18 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
             tmem_ld16(lane_addr + c * 16, r);
             tmem_ld16(lane_addr + kN + c * 16, q);
             tmem_wait_ld();
-            if (valid_cur && t.pairs) {
+            if (kTwo && t.join) {
+                const bool odd = tid & 1;
+                float2 *const to = p_cur - odd;   // the even row's group
+#pragma unroll
+                for (int l = 0; l < 8; l += 2) {
+                    const float2 v0 = out_of(r, q, l, 8 * c + l), v1 = out_of(r, q, l + 1, 8 * c + l + 1);
+                    const float2 give = odd ? v0 : v1;
+                    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1));
+                    *reinterpret_cast<float4 *>(to + off5(8 * c + l, t) + (odd ? 1ULL << t.q[0] : 0)) =
+                        odd ? make_float4(got.x, got.y, v1.x, v1.y) : make_float4(v0.x, v0.y, got.x, got.y);
+                }
+            } else if (!kTwo && valid_cur && t.pairs) {
 #pragma unroll
                 for (int l = 0; l < 8; l += 2) {
                     const float2 v0 = out_of(r, q, l, 8 * c + l), v1 = out_of(r, q, l + 1, 8 * c + l + 1);
@@ -895,8 +931,9 @@ __global__ void k_wait_selftest(int *__restrict__ status, long polls)
     if (!done) atomicExch(status, 1);
 }
 
-bool g_attr_c64[2][64] = {};       // [folded phase][device]
+bool g_attr_c64[2][2][64] = {};    // [folded phase][row pairs][device]
 bool g_attr_c128[2][3][64] = {};   // [folded phase][staging mode][device]
+using C64Kernel = void (*)(float2 *, uint64_t, TileLayout, const float *, const qs_post_phase *, int *);
 using C128Kernel = void (*)(double2 *, uint64_t, TileLayout, const uint8_t *, const qs_post_phase *, int *);
 
 }  // namespace
@@ -1006,12 +1043,6 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (dev < 0 || dev >= 64) return qs_fail(QS_EUNSUPPORTED, "device %d", dev);
-    if (c64 && !g_attr_c64[fold][dev]) {
-        const void *fn = fold ? (const void *)k_dense5_tc_c64<true> : (const void *)k_dense5_tc_c64<false>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemF32);
-        if (e != cudaSuccess) return qs_fail(QS_ECUDA, "tc smem attribute: %s", cudaGetErrorString(e));
-        g_attr_c64[fold][dev] = true;
-    }
     // the sweep covers the support after it: the support's free bits plus the
     // targets; groups enumerate the free bits that are not targets
     const uint64_t all = qs_index_mask(s->n);
@@ -1033,9 +1064,23 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     t.zmask = all & ~G;
     t.fix = fx & ~tm;
     t.full = fr == all;
-    t.pairs = c64 && t.q[0] == 0 && ((uintptr_t)s->amp & 15) == 0;
+    t.pairs = c64 && t.q[0] == 0;
     const uint64_t groups = 1ULL << __builtin_popcountll(G);
     const uint64_t tiles = (groups + kRows - 1) / kRows;
+    // neighbouring rows in 16-byte accesses: targets 1 to 4, where a row's 8 bytes leave
+    // half a sector or more unused, and enough tiles that throughput counts (high
+    // targets 2% slower that way; 20 qubits 95 -> 105 us a circuit: a longer way to the
+    // first MMA)
+    const bool two = c64 && t.q[0] >= 1 && t.q[0] <= 4 && !(t.zmask & 1) && tiles >= 16 * (uint64_t)sms;
+    t.join = two && t.q[0] <= 3;
+    static const C64Kernel c64s[2][2] = {{k_dense5_tc_c64<false, false>, k_dense5_tc_c64<false, true>},
+                                         {k_dense5_tc_c64<true, false>, k_dense5_tc_c64<true, true>}};
+    if (c64 && !g_attr_c64[fold][two][dev]) {
+        cudaError_t e = cudaFuncSetAttribute((const void *)c64s[fold][two], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kSmemF32);
+        if (e != cudaSuccess) return qs_fail(QS_ECUDA, "tc smem attribute: %s", cudaGetErrorString(e));
+        g_attr_c64[fold][two][dev] = true;
+    }
     // complex128 tiles of 128 consecutive amplitudes per member (no inserted
     // bit below bit 7), all members read: bulk copies of the stage
     const bool bulk = !c64 && (t.zmask & 0x7Full) == 0 && groups % kRows == 0 && t.mmask == 0xFFFFFFFFu;
@@ -1064,7 +1109,7 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     cudaError_t e;
     if (c64) {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms * 2);
-        e = launch_sweep(s, fold ? k_dense5_tc_c64<true> : k_dense5_tc_c64<false>, grid, kRows, kSmemF32, (float2 *)s->amp,
+        e = launch_sweep(s, c64s[fold][two], grid, kRows, kSmemF32, (float2 *)s->amp,
                          groups, t, (const float *)dev_pack, post, status);
     } else {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms);

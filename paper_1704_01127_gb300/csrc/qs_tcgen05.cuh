@@ -166,7 +166,8 @@ struct TileLayout {
     uint32_t mmask;
     uint64_t fix;
     uint64_t zmask;
-    int pairs;   // complex64: qubit 0 is a target and the buffer 16-byte aligned
+    int pairs;   // complex64: qubit 0 is a target
+    int join;    // complex64, qubit 0 is none: outputs of neighbouring groups joined to 16-byte stores
 };
 
 __device__ __forceinline__ uint64_t tile_base(uint64_t g, const TileLayout &t)
