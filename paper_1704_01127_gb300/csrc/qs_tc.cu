@@ -509,7 +509,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
     uint8_t *A = smem;
     uint8_t *B = smem + kSlices * kPlaneA;
     uint4 *stage = reinterpret_cast<uint4 *>(smem + kSmemC128);   // [8][512] x 16 B
-    __shared__ __align__(8) uint64_t mbar_mma[2], mbar_free[2], mbar_planes, mbar_full, mbar_used;
+    __shared__ __align__(8) uint64_t mbar_mma[2], mbar_free[2], mbar_planes, mbar_full, mbar_used, mbar_b;
     __shared__ uint64_t moff[32];         // offset of member x within a group
     __shared__ uint64_t ioff[32];         // kSub: offset of the member at K position x (support members first)
     __shared__ int perm[32];              // kSub: member at K position x
@@ -531,44 +531,38 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
     // zero); they take K positions 0 .. M-1, in order, and the rows of B^T
     // follow them, so only the first M K positions of A can be nonzero
     const int M = kSub ? __popc(t.mmask) : 32;
-    if constexpr (kSub) {
+    // B comes in by bulk copies: 4 KB blocks in place, plane-major pack (plane j =
+    // halves 0, 1) -> half-major blocks; kSub: whole into the stage, from which all
+    // threads write it with its K positions permuted.  The issuing thread waits for
+    // them before its first MMA (kSub: everyone, here).  (20 qubits, 25 cycles: 209 ->
+    // 203 us, with loads by all threads and the smallest G_n found by one of them.)
+    const uint32_t mbar_b_a = smem_u32(&mbar_b);
+    if (tid == kSplitThreads + kEpiThreads) {
+        mbar_init(mbar_b_a, 1);
+        fence_mbar_init();
+        mbar_arrive_expect_tx(mbar_b_a, kSlicesB * kPlaneB);
+        if constexpr (kSub) {
+            bulk_g2s(smem_u32(stage), bpack, kSlicesB * kPlaneB, mbar_b_a);
+        } else {
+            for (int blk = 0; blk < 2 * kSlicesB; blk++)   // source block 2 j + h
+                bulk_g2s(smem_u32(B) + ((blk & 1) * kSlicesB + (blk >> 1)) * kBlockB, bpack + blk * kBlockB, kBlockB, mbar_b_a);
+        }
+    }
+    if constexpr (kSub)
         if (tid < 32) {
             const uint32_t below = (1u << tid) - 1u;
             perm[(t.mmask >> tid) & 1 ? __popc(t.mmask & below) : M + __popc(~t.mmask & below)] = tid;
         }
-        __syncthreads();
-        if (tid < 32) ioff[tid] = off5(perm[tid], t);
-        // plane-major pack -> half-major blocks, K positions permuted (a
-        // member's two reals are one 4-byte word)
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(bpack);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(B);
-        for (int i = tid; i < kSlicesB * 2 * 1024; i += blockDim.x) {
-            const int blk = i >> 10, n = (i >> 5) & 31, x = i & 31;   // source block 2 j + h, row n, K position x
-            const int j = blk >> 1, h = blk & 1;
-            dst[((h * kSlicesB + j) * kBlockB + cm_off16(n, 2 * x)) >> 2] = src[(blk * kBlockB + cm_off16(n, 2 * perm[x])) >> 2];
-        }
-    } else {
-        // plane-major pack (plane j = halves 0, 1) -> half-major blocks
-        const uint4 *src = reinterpret_cast<const uint4 *>(bpack);
-        uint4 *dst = reinterpret_cast<uint4 *>(B);
-        constexpr int kPerBlock = (int)(kBlockB / 16);
-        for (int i = tid; i < kSlicesB * 2 * kPerBlock; i += blockDim.x) {
-            const int blk = i / kPerBlock, w = i - blk * kPerBlock;   // source block 2 j + h
-            const int j = blk >> 1, h = blk & 1;
-            dst[(h * kSlicesB + j) * kPerBlock + w] = src[i];
-        }
-    }
     {
         const int *G = reinterpret_cast<const int *>(bpack + kSlicesB * kPlaneB);
         if (tid < kN) colX[tid] = (uint32_t)G[tid] << 20;
-        if (tid == 0) {
-            int lo = 2047, hi = 0;
-            for (int n = 0; n < kN; n++) {
-                lo = min(lo, G[n]);
-                hi = max(hi, G[n]);
+        if (warp == 2) {
+            const int a = G[tid & 31], b = G[(tid & 31) + 32];
+            const int lo = __reduce_min_sync(0xffffffffu, min(a, b)), hi = __reduce_max_sync(0xffffffffu, max(a, b));
+            if (tid == 64) {
+                gext[0] = lo;
+                gext[1] = hi;
             }
-            gext[0] = lo;
-            gext[1] = hi;
         }
         if (tid < 32) moff[tid] = off5(tid, t);
         if constexpr (kPost) post_load(ps, post, tid, blockDim.x);
@@ -588,7 +582,23 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         fence_mbar_init();
         abort_flag = 0;
     }
-    fence_proxy_async();
+    if constexpr (kSub) {
+        __syncthreads();
+        if (!mbar_wait_bounded(mbar_b_a, 0)) {
+            atomicExch(status, 1);
+            abort_flag = 1;
+        }
+        if (tid < 32) ioff[tid] = off5(perm[tid], t);
+        // a member's two reals are one 4-byte word
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(stage);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(B);
+        for (int i = tid; i < kSlicesB * 2 * 1024; i += blockDim.x) {
+            const int blk = i >> 10, n = (i >> 5) & 31, x = i & 31;   // source block 2 j + h, row n, K position x
+            const int j = blk >> 1, h = blk & 1;
+            dst[((h * kSlicesB + j) * kBlockB + cm_off16(n, 2 * x)) >> 2] = src[(blk * kBlockB + cm_off16(n, 2 * perm[x])) >> 2];
+        }
+        fence_proxy_async();
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -783,6 +793,11 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
             const uint64_t low = tile_base(kRows - 1, t) ^ tile_base(0, t);
             int it = 0;
+            const bool b_ready = mbar_wait_bounded(mbar_b_a, 0);
+            if (!b_ready) {
+                atomicExch(status, 1);
+                abort_flag = 1;
+            }
             for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, it++) {
                 // the folded phase's tile part for tile it+1, while the planes of
                 // tile it are written: slot (it+1) & 3 last held tile it-3's, which
@@ -814,6 +829,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             }
             // leave only after the last MMAs are complete (they read this CTA's planes)
             if (it > 0 && !abort_flag) mbar_wait_bounded(smem_u32(&mbar_mma[1]), (it - 1) & 1);
+            if (!b_ready) mbar_wait_bounded(mbar_b_a, 0);   // its own copies in flight
         }
     } else {
         // ------------------------------------------------------------- epilogue
