@@ -339,15 +339,15 @@ constexpr int kC128Threads = kSplitThreads + kEpiThreads + kIssueThreads;
 constexpr int kSplitParts = kSplitThreads / kRows;   // splitter threads per row
 constexpr int kMPT = 32 / kSplitParts;               // amplitudes per splitter thread
 
-__device__ __forceinline__ void bar_split() { asm volatile("bar.sync 1, %0;" ::"r"(kSplitThreads) : "memory"); }
-__device__ __forceinline__ bool bar_split_or(bool v)
+__device__ __forceinline__ void bar_split(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
+__device__ __forceinline__ bool bar_split_or(bool v, int n)
 {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, 1, %2, q;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}\n"
         : "=r"(r)
-        : "r"((uint32_t)v), "r"(kSplitThreads)
+        : "r"((uint32_t)v), "r"(n)
         : "memory");
     return r != 0;
 }
@@ -390,10 +390,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t parity
 //         writes D_i..D_6 of that half (24 MMAs per half, 48 per tile).
 // kSub (a sweep that widens the support: only M = 2^m of the 32 members of
 // a group can be nonzero): those members take K positions 0 .. M-1 (B's K
-// positions permuted to match when it is copied in), splitters whose K
-// positions all lie past M keep zero planes and only join the barriers, and
-// each half takes ceil(M / 8) K steps per A plane instead of 4.  Every
-// accumulator sum is an exact integer, so the order of K changes no bit.
+// positions permuted to match when it is copied in), splitters whose K positions
+// all lie past M have nothing to do, and each half takes ceil(M / 8) K steps per A
+// plane instead of 4.  Every accumulator sum is an exact integer, so the order of K
+// changes no bit.  kSub = 2: four members per splitter thread instead of eight, for
+// states of a tile per CTA at most, where a tile's latency is the sweep (16 qubits,
+// 25 cycles 142 -> 134 us; 30 qubits 0.7% slower).
 // kPost (a phase op folded into the sweep): the phase of a row splits into a
 // part of its tile, formed one tile ahead by the issuing thread while it
 // waits for the planes (four slots by tile index), and a part of its row,
@@ -500,7 +502,26 @@ __device__ __forceinline__ uint32_t post_rowpart(const PostSmem &ps, uint64_t l)
     return ((uint32_t)__popcll(l & ps.c1) & 3u) | q << 2 | f << 3;
 }
 
-template <bool kPost, bool kBulk, bool kSub>
+// The double of T = th:tl (rounded to nearest even) with `scale` added to its exponent
+// field, in integer operations; T = 0 gives +0.0.
+__device__ __forceinline__ void rebuild_int(uint32_t th, uint32_t tl, uint32_t scale, uint32_t &hw, uint32_t &lw)
+{
+    const uint32_t s = (uint32_t)((int)th >> 31);
+    uint32_t al, ah;
+    asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %4;" : "=r"(al), "=r"(ah) : "r"(tl ^ s), "r"(th ^ s), "r"(s));
+    const bool small = ah == 0;
+    const uint32_t h1 = small ? al : ah, l1 = small ? 0u : al;
+    const uint32_t n = (uint32_t)__clz((int)h1);
+    const uint32_t N = __funnelshift_l(l1, h1, n), L = l1 << (n & 31u);   // leading one at bit 63
+    const uint32_t ml = __funnelshift_r(L, N, 11);
+    const uint32_t up = ((L & 0x7FFu) + 0x3FFu + (ml & 1u)) >> 11;
+    const uint32_t e = scale - (((small ? 32u : 0u) + n) << 20) + (1085u << 20);
+    uint32_t h;
+    asm("add.cc.u32 %0, %2, %3;\n\taddc.u32 %1, %4, %5;" : "=r"(lw), "=r"(h) : "r"(ml), "r"(up), "r"(N >> 11), "r"(e));
+    hw = N == 0 ? 0u : h ^ (s & 0x80000000u);
+}
+
+template <bool kPost, bool kBulk, int kSub>
 __global__ void __launch_bounds__(kC128Threads, 1)
 k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const uint8_t *__restrict__ bpack,
                       const qs_post_phase *__restrict__ post, int *__restrict__ status)
@@ -531,6 +552,9 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
     // zero); they take K positions 0 .. M-1, in order, and the rows of B^T
     // follow them, so only the first M K positions of A can be nonzero
     const int M = kSub ? __popc(t.mmask) : 32;
+    // splitter threads, MPT members each
+    constexpr int MPT = kSub == 2 ? 4 : kMPT;
+    const int n_split = kSub ? kRows * ((M + MPT - 1) / MPT) : kSplitThreads;
     // B comes in by bulk copies: 4 KB blocks in place, plane-major pack (plane j =
     // halves 0, 1) -> half-major blocks; kSub: whole into the stage, from which all
     // threads write it with its K positions permuted.  The issuing thread waits for
@@ -589,6 +613,13 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             abort_flag = 1;
         }
         if (tid < 32) ioff[tid] = off5(perm[tid], t);
+        if (tid >= n_split && tid < kSplitThreads) {   // nothing to split: no exponent, zero planes
+            const int row = tid & (kRows - 1), part = tid >> 7;
+            rowexp[part][row] = 0;
+            for (int c = 0; c < MPT / 4; c++)
+                for (int sl = 0; sl < kSlices; sl++)
+                    *reinterpret_cast<uint4 *>(A + cm_off16(row, 2 * MPT * part + 8 * c) + sl * kPlaneA) = make_uint4(0u, 0u, 0u, 0u);
+        }
         // a member's two reals are one 4-byte word
         const uint32_t *src = reinterpret_cast<const uint32_t *>(stage);
         uint32_t *dst = reinterpret_cast<uint32_t *>(B);
@@ -614,21 +645,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
     }
     chain_wait();
 
-    if (kSub && tid < kSplitThreads && kMPT * (tid >> 7) >= M) {
-        // ------------------------------------------------- idle splitters (kSub)
-        // K positions kMPT part .. + kMPT-1 are past M: zero planes, written
-        // once; then only the splitters' barriers, tile by tile
-        const int row = tid & (kRows - 1), part = tid >> 7;
-        for (int c = 0; c < kMPT / 4; c++)
-            for (int sl = 0; sl < kSlices; sl++)
-                *reinterpret_cast<uint4 *>(A + cm_off16(row, 2 * kMPT * part + 8 * c) + sl * kPlaneA) = make_uint4(0u, 0u, 0u, 0u);
-        fence_proxy_async();
-        for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            rowexp[part][row] = 0;
-            bar_split();
-            if (bar_split_or(abort_flag)) break;
-        }
-    } else if (tid < kSplitThreads) {
+    if (tid < n_split) {
         // ------------------------------------------------------------ splitters
         // kBulk: the four threads of a row are lanes r, r+8, r+16, r+24 of one
         // warp (warp w: rows 8w .. 8w+7), so the row's exponent is two warp
@@ -638,17 +655,17 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
         const uint32_t one = *(volatile uint32_t *)&g_qs_one;
         const uint32_t stage_a = smem_u32(stage) + 16u * tid;
-        // this thread's kMPT amplitudes of tile tl into its own stage slots
+        // this thread's MPT amplitudes of tile tl into its own stage slots
         // (slot x at x * kSplitThreads + tid): asynchronous, a whole iteration ahead
         auto prefetch = [&](uint64_t tl) {
             const uint64_t g = tl * kRows + row;
             const bool val = tl < n_tiles && g < n_groups;
             const double2 *pp = psi + (val ? tile_base(g, t) : 0);
 #pragma unroll
-            for (int x = 0; x < kMPT; x++) {
+            for (int x = 0; x < MPT; x++) {
                 // kSub: K positions past M are members outside the support (zero)
-                const bool vx = val && (!kSub || kMPT * part + x < M);
-                cp_async16(stage_a + 16u * kSplitThreads * x, vx ? pp + (kSub ? ioff : moff)[kMPT * part + x] : psi, vx ? 16u : 0u);
+                const bool vx = val && (!kSub || MPT * part + x < M);
+                cp_async16(stage_a + 16u * kSplitThreads * x, vx ? pp + (kSub ? ioff : moff)[MPT * part + x] : psi, vx ? 16u : 0u);
             }
             cp_async_commit();
         };
@@ -682,15 +699,15 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             } else {
                 cp_async_wait_all();
             }
-            double2 v[kMPT];
+            double2 v[MPT];
 #pragma unroll
-            for (int x = 0; x < kMPT; x++) {
+            for (int x = 0; x < MPT; x++) {
                 const uint4 w = stage[kSplitThreads * x + (kBulk ? kRows * part + row : tid)];
                 v[x] = make_double2(__hiloint2double((int)w.y, (int)w.x), __hiloint2double((int)w.w, (int)w.z));
             }
             uint32_t emax = 0;
 #pragma unroll
-            for (int x = 0; x < kMPT; x++) {
+            for (int x = 0; x < MPT; x++) {
                 emax = max(emax, (uint32_t)__double2hiint(v[x].x) & 0x7FF00000u);
                 emax = max(emax, (uint32_t)__double2hiint(v[x].y) & 0x7FF00000u);
             }
@@ -713,7 +730,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             } else {
                 prefetch(tile + gridDim.x);
                 rowexp[part][row] = (int)(emax >> 20);
-                bar_split();
+                bar_split(n_split);
                 E = rowexp[0][row];
 #pragma unroll
                 for (int q = 1; q < kSplitParts; q++) E = max(E, rowexp[q][row]);
@@ -726,10 +743,10 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             E = max(E, 1074 - ((volatile int *)gext)[0]);
             if (part == 0 && E + ((volatile int *)gext)[1] > 3057) atomicOr(status, 2);
             const int E7f = E >= 25 ? E + 7 : 0x40000000;
-            uint32_t glo[2 * kMPT], ghi[2 * kMPT], sgn[kMPT];
+            uint32_t glo[2 * MPT], ghi[2 * MPT], sgn[MPT];
 #pragma unroll
-            for (int x = 0; x < kMPT; x++) {
-                if (bulk && x == kMPT / 2 && full_ok && tile + gridDim.x < n_tiles) {
+            for (int x = 0; x < MPT; x++) {
+                if (bulk && x == MPT / 2 && full_ok && tile + gridDim.x < n_tiles) {
                     // every splitter warp has read the stage (by now, as a rule):
                     // the next tile's runs
                     if ((tid & 31) == 0) {
@@ -753,8 +770,8 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             // tile it-2's scale, so slot it & 1 is free
             if (part == 0) rowX[it & 1][row] = (uint32_t)(E - 2096) << 20;
 #pragma unroll
-            for (int c = 0; c < kMPT / 4; c++) {
-                uint8_t *dst = A + cm_off16(row, 2 * kMPT * part + 8 * c);
+            for (int c = 0; c < MPT / 4; c++) {
+                uint8_t *dst = A + cm_off16(row, 2 * MPT * part + 8 * c);
                 uint32_t pl[6][4];                     // [plane][member of the chunk]
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
@@ -778,7 +795,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             fence_proxy_async();
             // every splitter has written its planes (and seen tile it-1's MMAs
             // finish, or the abort)
-            if (bar_split_or(!ok || abort_flag)) {
+            if (bar_split_or(!ok || abort_flag, n_split)) {
                 if (tid == 0) atomicExch(status, 1);
                 break;
             }
@@ -787,6 +804,8 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         cp_async_wait_all();
         // bulk copies still in flight land before the CTA leaves
         if (pending >= 0) mbar_wait_bounded(mfull, pending & 1);
+    } else if (kSub && tid < kSplitThreads) {
+        // nothing to split
     } else if (tid >= kSplitThreads + kEpiThreads) {
         // ---------------------------------------------------------------- issuer
         if (tid == kSplitThreads + kEpiThreads) {
@@ -836,6 +855,14 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         const int ew = warp - kSplitThreads / 32;                 // 0 .. 11
         const int row = 32 * (warp & 3) + (tid & 31), ej = ew >> 2;   // warp ej of its lane quarter
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        // The conversions to FP64 take 16 clocks of an SM's FP64 unit each for a warp, half
+        // of a tile's time in all; where a warp reads all its chunks first (and releases
+        // the half early) every warp reaches them at once.  kInTurn: chunk by chunk, so
+        // that some warps convert while others read, and one value in four (kSub: one in
+        // six) rebuilt in integer operations.  28 qubits, high targets (kBulk) 1.98 -> 1.94
+        // ms; widening 27 -> 28 qubits (kSub) 1.62 -> 1.59; with cp.async staging the
+        // splitters' copies are the longer part and it measured 2 to 4% slower.
+        constexpr bool kInTurn = kBulk || kSub != 0;
         int it = 0;
         bool failed = false;
         for (uint64_t tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x, it++) {
@@ -859,16 +886,13 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                 }
                 tc_fence_after();
                 const uint32_t Xr = rowX[it & 1][row];
-                // the half's accumulators reduced to the exact partial sums P, Q and
-                // the rounded low part, then the half is released to the next
-                // tile's MMAs before the FP64 rebuild and the stores
                 // this warp's chunks of the half: 3, 3, 2 (half 0) and 2, 3, 3 (half 1)
                 const int c0 = h == 0 ? 3 * ej : (ej == 0 ? 0 : 3 * ej - 1);
                 const int nc = h == 0 ? (ej < 2 ? 3 : 2) : (ej == 0 ? 2 : 3);
+                // a chunk's accumulators reduced to the exact partial sums P, Q and the
+                // rounded low part
                 int Pv[kEpiMaxChunks][4], Qv[kEpiMaxChunks][4], Rv[kEpiMaxChunks][4];
-#pragma unroll
-                for (int c = 0; c < kEpiMaxChunks; c++) {
-                    if (c >= nc) break;
+                auto read = [&](int c) {
                     const int col = 4 * (c0 + c);
                     float D[kDiags][4];
 #pragma unroll
@@ -889,12 +913,12 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                     for (int q = 0; q < 4; q++) {
                         Rv[c][q] = __float2int_rn(fmaf(D[4][q], 256.0f, fmaf(D[6][q], 0.00390625f, D[5][q])));
                     }
-                }
-                tc_fence_before();
-                mbar_arrive(smem_u32(&mbar_free[h]));   // the half's accumulators are read
-#pragma unroll
-                for (int c = 0; c < kEpiMaxChunks; c++) {
-                    if (c >= nc) break;
+                };
+                auto release = [&] {
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&mbar_free[h]));   // the half's accumulators are read
+                };
+                auto write = [&](int c) {
                     const int col = 4 * (c0 + c);              // column within the half
                     uint32_t hw[4], lw[4];
 #pragma unroll
@@ -907,11 +931,25 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                             : "=r"(tl), "=r"(th)
                             : "r"((uint32_t)Qt << 16), "r"((uint32_t)R), "r"((uint32_t)Pv[c][q] + (uint32_t)(Qt >> 16)),
                               "r"((uint32_t)(R >> 31) - 0x8B400000u));
-                        const double dv = __ll2double_rn((long long)((uint64_t)th << 32 | tl));
-                        const uint32_t hi = (uint32_t)__double2hiint(dv);
-                        // T = 0 gives +0.0 (hi = 0); otherwise add the scale to the exponent
-                        hw[q] = hi == 0 ? 0u : hi + Xr + colX[kHalfN * h + col + q];
-                        lw[q] = (uint32_t)__double2loint(dv);
+                        const long long T = (long long)((uint64_t)th << 32 | tl);
+                        if constexpr (kInTurn) {
+                            // (the exponent's terms before the conversion is waited for)
+                            const uint32_t scale = Xr + colX[kHalfN * h + col + q];
+                            if (q == 3 && (kBulk || c != 1)) {
+                                rebuild_int(th, tl, scale, hw[q], lw[q]);
+                            } else {
+                                const double dv = __ll2double_rn(T);
+                                const uint32_t hi = (uint32_t)__double2hiint(dv);
+                                hw[q] = hi == 0 ? 0u : hi + scale;
+                                lw[q] = (uint32_t)__double2loint(dv);
+                            }
+                        } else {
+                            const double dv = __ll2double_rn(T);
+                            const uint32_t hi = (uint32_t)__double2hiint(dv);
+                            // T = 0 gives +0.0 (hi = 0); otherwise add the scale to the exponent
+                            hw[q] = hi == 0 ? 0u : hi + Xr + colX[kHalfN * h + col + q];
+                            lw[q] = (uint32_t)__double2loint(dv);
+                        }
                     }
                     const int m0 = (kHalfN * h + col) >> 1;   // columns 2m, 2m+1: re, im of member m
                     if constexpr (kPost) {
@@ -923,6 +961,27 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                                                    __hiloint2double((int)hw[1], (int)lw[1]));
                         p[moff[m0 + 1]] = make_double2(__hiloint2double((int)hw[2], (int)lw[2]),
                                                        __hiloint2double((int)hw[3], (int)lw[3]));
+                    }
+                };
+                if constexpr (kInTurn) {
+#pragma unroll
+                    for (int c = 0; c < kEpiMaxChunks; c++) {
+                        if (c >= nc) break;
+                        read(c);
+                        if (c == nc - 1) release();
+                        write(c);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < kEpiMaxChunks; c++) {
+                        if (c >= nc) break;
+                        read(c);
+                    }
+                    release();
+#pragma unroll
+                    for (int c = 0; c < kEpiMaxChunks; c++) {
+                        if (c >= nc) break;
+                        write(c);
                     }
                 }
             }
@@ -948,7 +1007,7 @@ __global__ void k_wait_selftest(int *__restrict__ status, long polls)
 }
 
 bool g_attr_c64[2][2][64] = {};    // [folded phase][row pairs][device]
-bool g_attr_c128[2][3][64] = {};   // [folded phase][staging mode][device]
+bool g_attr_c128[2][4][64] = {};   // [folded phase][staging mode][device]
 using C64Kernel = void (*)(float2 *, uint64_t, TileLayout, const float *, const qs_post_phase *, int *);
 using C128Kernel = void (*)(double2 *, uint64_t, TileLayout, const uint8_t *, const qs_post_phase *, int *);
 
@@ -1101,15 +1160,16 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     // bit below bit 7), all members read: bulk copies of the stage
     const bool bulk = !c64 && (t.zmask & 0x7Full) == 0 && groups % kRows == 0 && t.mmask == 0xFFFFFFFFu;
     // complex128 staging: 0 cp.async (every member in the support), 1 bulk
-    // copies, 2 members outside the support (compacted, fewer K steps)
-    const int mode = bulk ? 1 : t.mmask != 0xFFFFFFFFu ? 2 : 0;
+    // copies, 2 members outside the support (compacted, fewer K steps), 3 the same
+    // with at most a tile per CTA
+    const int mode = bulk ? 1 : t.mmask == 0xFFFFFFFFu ? 0 : tiles <= (uint64_t)sms ? 3 : 2;
     C128Kernel c128 = nullptr;
     if (!c64) {
-        static const C128Kernel fns[2][3] = {
-            {k_dense5_tc_c128_pipe<false, false, false>, k_dense5_tc_c128_pipe<false, true, false>,
-             k_dense5_tc_c128_pipe<false, false, true>},
-            {k_dense5_tc_c128_pipe<true, false, false>, k_dense5_tc_c128_pipe<true, true, false>,
-             k_dense5_tc_c128_pipe<true, false, true>}};
+        static const C128Kernel fns[2][4] = {
+            {k_dense5_tc_c128_pipe<false, false, 0>, k_dense5_tc_c128_pipe<false, true, 0>,
+             k_dense5_tc_c128_pipe<false, false, 1>, k_dense5_tc_c128_pipe<false, false, 2>},
+            {k_dense5_tc_c128_pipe<true, false, 0>, k_dense5_tc_c128_pipe<true, true, 0>,
+             k_dense5_tc_c128_pipe<true, false, 1>, k_dense5_tc_c128_pipe<true, false, 2>}};
         c128 = fns[fold][mode];
         if (!g_attr_c128[fold][mode][dev]) {
             cudaError_t e = cudaFuncSetAttribute((const void *)c128, cudaFuncAttributeMaxDynamicSharedMemorySize,
