@@ -45,8 +45,11 @@ constexpr uint32_t kIdescTf32x2 = kIdescTf32 + ((uint32_t)(kN >> 3) << 17);   //
 // (t.join) the outputs leave in 16-byte stores too, two members exchanged between the
 // threads of neighbouring rows.  28 qubits: targets 1, 2, 11, 26, 27 1004 -> 838 us;
 // 1, 9, 15, 20, 22 776 -> 733; 1 to 5 1320 -> 1172.
-template <bool kPost, bool kTwo>
-__global__ void __launch_bounds__(128, 2)
+// NP = 2: two threads per row, 16 members each, for states of a tile per CTA at most,
+// where the loads and the split before the MMAs are a third of a sweep (16 qubits, 25
+// cycles 62 -> 59 us; 20 qubits 95 -> 91).
+template <bool kPost, bool kTwo, int NP>
+__global__ void __launch_bounds__(128 * NP, NP == 1 ? 2 : 1)
 k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const float *__restrict__ bpack,
                 const qs_post_phase *__restrict__ post, int *__restrict__ status)
 {
@@ -59,6 +62,9 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
     __shared__ PostSmem ps;
 
     const int tid = threadIdx.x, warp = tid >> 5;
+    constexpr int kMem = 32 / NP;   // members per thread
+    const int row = tid & (kRows - 1), part = NP == 1 ? 0 : tid >> 7;
+    const uint64_t part_off = part ? 1ULL << t.q[4] : 0;   // members 16 and up
     chain_start();
     {
         const float4 *src = reinterpret_cast<const float4 *>(bpack);
@@ -87,13 +93,13 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
     uint32_t parity = 0;
     // software pipeline: the next tile's amplitudes are loaded into registers
     // while the tensor cores work on the current one
-    float2 v[32];   // kTwo: v[2 x], v[2 x + 1]: member 16 h + x of the row written first and of the other
+    float2 v[kMem];   // kTwo: v[2 x], v[2 x + 1]: member 16 h + x of the row written first and of the other
     uint64_t tile = blockIdx.x;
     bool valid = false;
     float2 *p = psi;
     const int pi = tid & 63, ph = tid >> 6, second = (pi >> 2) & 1;   // kTwo
     auto load_tile = [&](uint64_t tl, float2 *vv, bool &val, float2 *&pp) {
-        const uint64_t g = tl * kRows + (kTwo ? 2 * pi : tid);
+        const uint64_t g = tl * kRows + (kTwo ? 2 * pi : row);
         val = tl < n_tiles && g < n_groups;
         pp = psi + (val ? tile_base(g, t) : 0);
         if constexpr (kTwo) {
@@ -108,15 +114,17 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
         } else if (t.pairs) {
             // members 2i and 2i+1 differ in qubit 0: one 16-byte load each
             // (a member outside the support is read but replaced by zero)
+            const uint32_t in = t.mmask >> (kMem * part);
 #pragma unroll
-            for (int x = 0; x < 32; x += 2) {
-                const float4 w = val ? *reinterpret_cast<const float4 *>(pp + off5(x, t)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                vv[x] = ((t.mmask >> x) & 1) ? make_float2(w.x, w.y) : make_float2(0.f, 0.f);
-                vv[x + 1] = ((t.mmask >> (x + 1)) & 1) ? make_float2(w.z, w.w) : make_float2(0.f, 0.f);
+            for (int x = 0; x < kMem; x += 2) {
+                const float4 w = val ? *reinterpret_cast<const float4 *>(pp + part_off + off5(x, t)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                vv[x] = ((in >> x) & 1) ? make_float2(w.x, w.y) : make_float2(0.f, 0.f);
+                vv[x + 1] = ((in >> (x + 1)) & 1) ? make_float2(w.z, w.w) : make_float2(0.f, 0.f);
             }
         } else {
+            const uint32_t in = t.mmask >> (kMem * part);
 #pragma unroll
-            for (int x = 0; x < 32; x++) vv[x] = val && ((t.mmask >> x) & 1) ? pp[off5(x, t)] : make_float2(0.f, 0.f);
+            for (int x = 0; x < kMem; x++) vv[x] = val && ((in >> x) & 1) ? pp[part_off + off5(x, t)] : make_float2(0.f, 0.f);
         }
     };
     auto split = [&](int row, int c, float2 v0, float2 v1) {
@@ -137,7 +145,7 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
             }
         } else {
 #pragma unroll
-            for (int c = 0; c < 16; c++) split(tid, c, v[2 * c], v[2 * c + 1]);
+            for (int c = 0; c < kMem / 2; c++) split(row, kMem / 2 * part + c, v[2 * c], v[2 * c + 1]);
         }
         fence_proxy_async();
         tc_fence_before();
@@ -179,17 +187,17 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
         }
         parity ^= 1;
         tc_fence_after();
-        const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
+        const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kN / NP * part;
         uint32_t pe = 0, pf = 0;
         if constexpr (kPost) post_row(ps, (uint64_t)(p_cur - psi), pe, pf);
         // output of member m: head + corrections, times the folded phase's factor
         auto out_of = [&](const float *r, const float *q, int l, int m) {
             float2 v = make_float2(r[2 * l] + q[2 * l], r[2 * l + 1] + q[2 * l + 1]);
-            if constexpr (kPost) v = rot_i(v, post_member(pe, pf, m));
+            if constexpr (kPost) v = rot_i(v, post_member(pe, pf, kMem * part + m));
             return v;
         };
 #pragma unroll
-        for (int c = 0; c < kN / 16; c++) {
+        for (int c = 0; c < kN / 16 / NP; c++) {
             float r[16], q[16];
             tmem_ld16(lane_addr + c * 16, r);
             tmem_ld16(lane_addr + kN + c * 16, q);
@@ -209,11 +217,11 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
 #pragma unroll
                 for (int l = 0; l < 8; l += 2) {
                     const float2 v0 = out_of(r, q, l, 8 * c + l), v1 = out_of(r, q, l + 1, 8 * c + l + 1);
-                    *reinterpret_cast<float4 *>(p_cur + off5(8 * c + l, t)) = make_float4(v0.x, v0.y, v1.x, v1.y);
+                    *reinterpret_cast<float4 *>(p_cur + part_off + off5(8 * c + l, t)) = make_float4(v0.x, v0.y, v1.x, v1.y);
                 }
             } else if (valid_cur) {
 #pragma unroll
-                for (int l = 0; l < 8; l++) p_cur[off5(8 * c + l, t)] = out_of(r, q, l, 8 * c + l);
+                for (int l = 0; l < 8; l++) p_cur[part_off + off5(8 * c + l, t)] = out_of(r, q, l, 8 * c + l);
             }
         }
         tc_fence_before();
@@ -1008,7 +1016,7 @@ __global__ void k_wait_selftest(int *__restrict__ status, long polls)
     if (!done) atomicExch(status, 1);
 }
 
-bool g_attr_c64[2][2][64] = {};    // [folded phase][row pairs][device]
+bool g_attr_c64[2][3][64] = {};    // [folded phase][form][device]
 bool g_attr_c128[2][4][64] = {};   // [folded phase][staging mode][device]
 using C64Kernel = void (*)(float2 *, uint64_t, TileLayout, const float *, const qs_post_phase *, int *);
 using C128Kernel = void (*)(double2 *, uint64_t, TileLayout, const uint8_t *, const qs_post_phase *, int *);
@@ -1150,13 +1158,15 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     // first MMA)
     const bool two = c64 && t.q[0] >= 1 && t.q[0] <= 4 && !(t.zmask & 1) && tiles >= 16 * (uint64_t)sms;
     t.join = two && t.q[0] <= 3;
-    static const C64Kernel c64s[2][2] = {{k_dense5_tc_c64<false, false>, k_dense5_tc_c64<false, true>},
-                                         {k_dense5_tc_c64<true, false>, k_dense5_tc_c64<true, true>}};
-    if (c64 && !g_attr_c64[fold][two][dev]) {
-        cudaError_t e = cudaFuncSetAttribute((const void *)c64s[fold][two], cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const int form = two ? 1 : tiles <= (uint64_t)sms ? 2 : 0;   // 256 threads on more tiles: 1 to 3% slower
+    static const C64Kernel c64s[2][3] = {
+        {k_dense5_tc_c64<false, false, 1>, k_dense5_tc_c64<false, true, 1>, k_dense5_tc_c64<false, false, 2>},
+        {k_dense5_tc_c64<true, false, 1>, k_dense5_tc_c64<true, true, 1>, k_dense5_tc_c64<true, false, 2>}};
+    if (c64 && !g_attr_c64[fold][form][dev]) {
+        cudaError_t e = cudaFuncSetAttribute((const void *)c64s[fold][form], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemF32);
         if (e != cudaSuccess) return qs_fail(QS_ECUDA, "tc smem attribute: %s", cudaGetErrorString(e));
-        g_attr_c64[fold][two][dev] = true;
+        g_attr_c64[fold][form][dev] = true;
     }
     // complex128 tiles of 128 consecutive amplitudes per member (no inserted
     // bit below bit 7), all members read: bulk copies of the stage
@@ -1187,7 +1197,7 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     cudaError_t e;
     if (c64) {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms * 2);
-        e = launch_sweep(s, c64s[fold][two], grid, kRows, kSmemF32, (float2 *)s->amp,
+        e = launch_sweep(s, c64s[fold][form], grid, form == 2 ? 2 * kRows : kRows, kSmemF32, (float2 *)s->amp,
                          groups, t, (const float *)dev_pack, post, status);
     } else {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms);
