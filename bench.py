@@ -409,7 +409,7 @@ def run_ours(args):
     # the spec form (learned schedule, complex64) on the 30- and 32-qubit
     # circuits, against the plain complex128 form and the oracle's amplitudes
     target = target_form(qs, stream, hbm_gbs) if extras and not args.no_target else None
-    # the batched workload: 512 circuits in one graph-replayed persistent launch
+    # the batched workload: 512 circuits in one graph launch
     batch = batch_section(qs, stream, 5, 3)[0] if extras and not args.no_batch else None
     if rank != 0:
         return None
@@ -441,7 +441,7 @@ def run_ours(args):
 
 def batch_section(qs, stream, steps, warmup, clock_index=None):
     """512 independent circuits (seeds 0..511; grids 4x4 / 4x5 / 3x7, depths
-    8..40), complex64, one persistent launch replayed from a CUDA graph, against
+    8..40), complex64, one launch per pass replayed from a CUDA graph, against
     a loop of single-circuit launches of the same schedules.  Returns the
     measured figures and the per-launch device time."""
     import torch
@@ -498,8 +498,8 @@ def batch_section(qs, stream, steps, warmup, clock_index=None):
     for sc in scheds:
         qs.qs_schedule_free(sc)
     per_launch = elapsed / steps
-    out = {"workload": "512 circuits (seeds 0..511), grids 4x4/4x5/3x7, 8..40 CZ cycles, c64, one persistent "
-                       "launch per step replayed from a CUDA graph",
+    out = {"workload": "512 circuits (seeds 0..511), grids 4x4/4x5/3x7, 8..40 CZ cycles, c64, one launch "
+                       "per pass, replayed from a CUDA graph",
            "autotuned": {"k_max": k_max, "cluster_ctas": C, "threads": T, "tune_ms": tune_ms,
                          "tune_wall_s": tune_s},
            "l2": "states total %.0f MB; inputs re-initialised every launch" % (

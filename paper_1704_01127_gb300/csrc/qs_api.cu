@@ -81,7 +81,7 @@ using qsd::prob;
 
 // p_i = |psi_i|^2 (first <= i < first + count), four steps in flight per thread; VEC = 2:
 // two neighbouring complex64 amplitudes per step (16-byte loads and stores).
-// 26 qubits: complex64 628 -> 261 us (HBM 159; one FP64 addition an amplitude, 116), complex128 412 -> 266 us
+// 26 qubits: complex64 628 -> 179 us (HBM 159; p is formed in integer operations), complex128 412 -> 266 us
 // (HBM 239; its three FP64 operations an amplitude took 348, the squares now run on the integer units).
 template <typename C, int VEC>
 __global__ void __launch_bounds__(256)
@@ -341,9 +341,10 @@ int ensure_fflog(cudaStream_t st)
 // ------------------------------------------------------------------ sampling
 constexpr uint32_t kFull = 0xffffffffu;
 
-// Pairwise sums over fixed power-of-two blocks: lane l of a warp reduces its
-// contiguous len/32 values as a perfect binary tree, then the 32 lane results
-// combine as the top five tree levels (lane pairs (0,1), (2,3), ... first).
+// Pairwise sums over fixed power-of-two blocks (blocks of 1024 amplitudes:
+// k_block_sums): lane l of a warp reduces its contiguous len/32 values as a perfect
+// binary tree, then the 32 lane results combine as the top five tree levels (lane
+// pairs (0,1), (2,3), ... first).
 
 template <typename C>
 __device__ double load_p(const C *psi, uint64_t i) { return prob(psi[i]); }
@@ -586,8 +587,9 @@ __device__ __forceinline__ double chain_add(double c, double p, double &half)
 // 31: all N at once while the sum stays in one binade without ties (the terms then
 // depend on c's exponent alone), else one group after another, addition by addition.
 // 2^e the start of c's binade: for p < 2^(e-20) a term is the low word of fl(2^e + p)
-// and a tie needs 20 zero bits at p's end.  Where some value has those or is larger,
-// the terms come from chain_term.
+// and a tie needs 20 zero bits at p's end.  Where some value has those (equal or
+// real-valued amplitudes) the bits that a term drops are looked at; where some is
+// larger, the terms come from chain_term.
 template <int N>
 __device__ __forceinline__ double chain_add_n(double c, const double *p, double *half, double *full)
 {
@@ -597,17 +599,28 @@ __device__ __forceinline__ double chain_add_n(double c, const double *p, double 
     const double c0 = __longlong_as_double((long long)(cb & 0x7FF0000000000000ULL));
     const uint32_t top = (uint32_t)max(E - 20, 0) << 20;
     uint32_t v[N], any = 0;
-    bool careful = E < 64;
+    bool large = E < 64, zeros = false;
 #pragma unroll
     for (int k = 0; k < N; k++) {
         const uint32_t h = (uint32_t)__double2hiint(p[k]), l = (uint32_t)__double2loint(p[k]);
         v[k] = (uint32_t)__double2loint(c0 + p[k]);
         any |= v[k];
-        careful = careful || h >= top || ((l & 0xFFFFFu) == 0 && (h | l) != 0);
+        large = large || h >= top;
+        zeros = zeros || ((l & 0xFFFFFu) == 0 && (h | l) != 0);
     }
     uint64_t at = cb, mid[N], end[N];
     bool slow = false;
-    if (!__any_sync(kFull, careful)) {
+    if (!__any_sync(kFull, large)) {
+        if (__any_sync(kFull, zeros)) {
+#pragma unroll
+            for (int k = 0; k < N; k++) {
+                const uint64_t b = (uint64_t)__double_as_longlong(p[k]);
+                const int sh = E - (int)(b >> 52);   // the term drops p's last sh bits, 21 of them or more
+                const uint64_t m = (b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
+                slow = slow || (sh < 54 && m << (64 - sh) == 1ULL << 63);
+            }
+            slow = __any_sync(kFull, slow);
+        }
         if (!__any_sync(kFull, any >> 27)) {   // 32 terms add up in 32 bits
 #pragma unroll
             for (int k = 0; k < N; k++) {
@@ -992,7 +1005,7 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
     const bool listed = m < 2 * (int64_t)nb, every = m >= 128 * (int64_t)nb;
     // a block is summed up to its largest draw where that saves more than the table
     // costs: some 16 draws per block at most (4: a fifth of the sums; 28 qubits
-    // complex128, 2^20 draws 4.38 -> 4.23 ms), and many blocks (21 qubits 3% slower)
+    // complex128, 2^20 draws: checkpoints 1.44 -> 1.31 ms), and many blocks (21 qubits 3% slower)
     const bool part_way = !every && nb >= (1u << 15) && m <= 16 * (int64_t)nb;
     const size_t n_work = listed ? (size_t)std::min<uint64_t>(nb, m_slots) : nb;
     const size_t n_sums = n_work * (every ? 1024 : kCks);

@@ -57,13 +57,13 @@ k_dense(typename cplx<R>::t *__restrict__ psi, uint64_t n_groups, Targets t,
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * G;
     for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x * G + threadIdx.x; g < n_groups; g += stride) {
         if constexpr (G == 1) {
-            qsd::dense_group<R, K, false>(psi + group_base<K>(g, t), t, Us);
+            qsd::dense_group<R, K>(psi + group_base<K>(g, t), t, Us);
         } else {
             C *p[G], v[G][D];
 #pragma unroll
             for (int i = 0; i < G; i++) {
                 p[i] = psi + group_base<K>(min(g + (uint64_t)i * blockDim.x, n_groups - 1), t);
-                qsd::dense_load<R, K, false>(p[i], t, v[i]);
+                qsd::dense_load<R, K>(p[i], t, v[i]);
             }
 #pragma unroll
             for (int i = 0; i < G; i++)

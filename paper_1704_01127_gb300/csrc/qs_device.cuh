@@ -1,5 +1,6 @@
-// Device building blocks shared by the single-state kernels (qs_apply.cu) and
-// the batched persistent kernel (qs_batch.cu), so both run the same arithmetic.
+// Device building blocks shared by the sweeps (qs_apply.cu), the passes
+// (qs_pass.cu), the statistics and the draws (qs_api.cu, qs_batch.cu), so that all
+// run the same arithmetic.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -40,24 +41,15 @@ __device__ __forceinline__ uint64_t member_offset(int x, const Targets &t)
     return o;
 }
 
-template <bool CG, typename C>
-__device__ __forceinline__ C ld(const C *p)
-{
-    if constexpr (CG) return __ldcg(p);
-    else return *p;
-}
-
 // One group of a dense k-qubit cluster (Sec. 3.2): the 2^K amplitudes at
 // strides 2^{q_j} are gathered into registers, v <- U v, and scattered back.
 // Each complex multiply-accumulate is the pair of real FMA updates of
 // Eqs. (2)-(3): acc += (v_R m_R, v_I m_R) then acc += (-v_I m_I, v_R m_I).
-// CG: loads bypass L1 (the batched kernel shares states between the CTAs of a
-// cluster).
-template <typename R, int K, bool CG>
+template <typename R, int K>
 __device__ __forceinline__ void dense_load(const typename cplx<R>::t *p, const Targets &t, typename cplx<R>::t *v)
 {
 #pragma unroll
-    for (int x = 0; x < (1 << K); x++) v[x] = ld<CG>(p + member_offset<K>(x, t));
+    for (int x = 0; x < (1 << K); x++) v[x] = p[member_offset<K>(x, t)];
 }
 
 template <typename R, int K>
@@ -86,12 +78,12 @@ __device__ __forceinline__ void dense_rows(typename cplx<R>::t *p, const Targets
     }
 }
 
-template <typename R, int K, bool CG>
+template <typename R, int K>
 __device__ __forceinline__ void dense_group(typename cplx<R>::t *p, const Targets &t,
                                             const typename cplx<R>::t *Us)
 {
     typename cplx<R>::t v[1 << K];
-    dense_load<R, K, CG>(p, t, v);
+    dense_load<R, K>(p, t, v);
     dense_rows<R, K>(p, t, Us, v);
 }
 
@@ -140,10 +132,8 @@ __device__ __forceinline__ C rotate8(C a, int m)
 
 // Phase products (Sec. 2, Sec. 3.5): amplitude i gets e^{i pi m(i)/4},
 // m(i) = sum_q c_q i_q + 4 sum_a i_a popc(i & P_a) mod 8, with P_a the CZ
-// partners b > a of qubit a.  With i = h | l (l: the low L bits) this is
-// m_lo(l) + m_hi(h) + 4 popc(l & M_h): m_lo is a table over the low bits,
-// m_hi and the mask M_h (low qubits whose partner set meets h an odd number of
-// times) are fixed for a chunk of 2^L amplitudes.
+// partners b > a of qubit a: the exponent of the bits x alone, both ends of a CZ
+// below bit L.
 __device__ __forceinline__ uint8_t phase_low(uint64_t x, const uint64_t *cm, const int *act,
                                              const uint64_t *part, int n_act, int L)
 {
@@ -155,33 +145,23 @@ __device__ __forceinline__ uint8_t phase_low(uint64_t x, const uint64_t *cm, con
     return (uint8_t)((m + 4 * (par & 1)) & 7);
 }
 
-__device__ __forceinline__ int phase_high(uint64_t h, const uint64_t *cm, const int *act, const uint64_t *part,
-                                          int n_act, int L, uint64_t &Mh)
-{
-    int mh = __popcll(h & cm[0]) + 2 * __popcll(h & cm[1]) + 4 * __popcll(h & cm[2]);
-    int parh = 0;
-    Mh = 0;
-    for (int t = 0; t < n_act; t++) {
-        const int a = act[t];
-        const int odd = __popcll(h & part[t]) & 1;
-        if (a >= L) parh ^= (int)((h >> a) & 1) & odd;
-        else Mh |= (uint64_t)odd << a;
-    }
-    return (mh + 4 * parh) & 7;
-}
-
 // fl(x^2) of a double, rounded to nearest even, from integer operations: the
 // FP64 unit gives two results a clock per SM, the integer units 64, so a pass
 // that also adds in FP64 runs the squares beside it.  x = m 2^(e - 1075), m the
 // 53-bit significand; m^2 has 105 or 106 bits (s = 0 or 1) and its top 53 are
 // kept: the round bit and the bits below it sit in x (bit 0 set when a dropped
 // word is not zero), whose carry out of 2^31 - 1 + lsb is the increment.  Squares
-// outside the normal range (and zeros, infinities, NaN) take the FP64 unit.
+// outside the normal range (and infinities, NaN) take the FP64 unit.
 __device__ __forceinline__ double sq_rn(double d)
 {
     const uint32_t hi = (uint32_t)__double2hiint(d) & 0x7FFFFFFFu, lo = (uint32_t)__double2loint(d);
     const uint32_t e = hi >> 20;
-    if (e - 513u > 1020u) return __dmul_rn(d, d);
+    if (e - 513u > 1020u) {
+        if ((hi | lo) == 0) return 0.0;   // real-valued states: not the FP64 unit for every zero
+        double sq;
+        asm volatile("mul.rn.f64 %0, %1, %1;" : "=d"(sq) : "d"(d));
+        return sq;
+    }
     const uint32_t mh = (hi & 0xFFFFFu) | 0x100000u;
     const uint64_t ll = (uint64_t)lo * lo, lh = (uint64_t)lo * mh, hh = (uint64_t)mh * mh;
     uint32_t L1, H0, H1;   // m^2 = H1:H0:L1:L0
@@ -227,19 +207,27 @@ __device__ __forceinline__ double sq_exact(float x)
     const uint64_t bexp = (uint64_t)(63 - lz + 2 * E + 1023);
     return __longlong_as_double((long long)((bexp << 52) | frac));
 }
-static __device__ __noinline__ double prob_rare(float2 v) { return __dadd_rn(sq_exact(v.x), sq_exact(v.y)); }
+static __device__ __noinline__ double prob_rare(float2 v)
+{
+    if (v.x == 0.f && v.y == 0.f) return 0.0;
+    return __dadd_rn(sq_exact(v.x), sq_exact(v.y));
+}
 // p = fl(x^2 + y^2) with exact squares: fl(fl(x^2) + fl(y^2)) in FP64, in integer
 // operations as well, so a pass that adds p in FP64 has that pipe to itself.  With
 // a >= b the magnitudes, significands shifted up by 7: A = ma^2 in [2^60, 2^62), and
 // mb^2 shifted down by twice the exponents' difference s, its dropped bits joined
 // into the lowest one (they lie below the rounding position).  The sum's leading one
 // is at bit 60, 61 or 62 and it is rounded to 53 bits, half to even, as in sq_rn.
-// Subnormal or zero b, infinities and NaN take the squares one by one.
+// Subnormal components, infinities and NaN take the squares one by one.  A zero b
+// beside a >= 2^-95 is shifted out altogether (s = 63), and the joined bit is below
+// half of a sum whose 14 lowest bits are zero otherwise: p = fl(a^2) without a branch
+// of its own.
 __device__ __forceinline__ double prob(float2 v)
 {
     const uint32_t bx = __float_as_uint(v.x) & 0x7fffffffu, by = __float_as_uint(v.y) & 0x7fffffffu;
     const uint32_t a = max(bx, by), b = min(bx, by);
-    if (b < 0x800000u || a >= 0x7f800000u) return prob_rare(v);
+    if (b < 0x800000u || a >= 0x7f800000u)
+        if (b != 0 || a < 0x10000000u || a >= 0x7f800000u) return prob_rare(v);
     const uint32_t ea = a >> 23, ma = (a << 7) & 0x3fffff80u | 0x40000000u, mb = (b << 7) & 0x3fffff80u | 0x40000000u;
     const uint64_t A = (uint64_t)ma * ma, B = (uint64_t)mb * mb;
     const uint32_t s = min(2u * (ea - (b >> 23)), 63u);
@@ -311,11 +299,6 @@ __device__ __forceinline__ ff ff_fast_two_sum(float a, float b)   // |a| >= |b| 
 {
     const float s = __fadd_rn(a, b);
     return ff{s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ ff ff_add_f(ff a, float b)
-{
-    ff s = ff_two_sum(a.hi, b);
-    return ff_fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
 }
 // x^2 exactly as hi + lo (the FMA gives the rounding error of the product)
 __device__ __forceinline__ ff ff_sqr_f(float x)
