@@ -769,7 +769,7 @@ def run_kernel(args):
         qs.qs_mlp_train(net, X, Y, args.reps)
         per = (time.perf_counter() - t) / args.reps * 1e3
         qs.qs_mlp_free(net)
-        print(json.dumps({"kernel": "mlp training epoch (k_mlp_fwd, k_mlp_delta, k_mlp_grad, k_adam)",
+        print(json.dumps({"kernel": "mlp training epoch (k_mlp_tile, k_mlp_adam)",
                           "batch": args.batch, "epochs": args.reps, "ms_per_epoch": per}))
         return None
     h = qs.qs_alloc(n, dtype, stream)

@@ -475,12 +475,15 @@ constexpr size_t kSmemC128Pipe = kSmemC128 + kStageC128;
 // MMA-issuing thread, the row's part once per CTA for each of its 128 rows;
 // X_H is kept as its bits at the `low` positions (bit k: the k-th lowest), so
 // parity(l & X_H) = parity(r & X) for row r of the tile.
-__device__ __forceinline__ void post_tile(const PostSmem &ps, uint64_t H, uint64_t low, uint32_t &X, uint32_t &C)
+// A warp forms a tile's part, a term per lane (one thread took 15 terms to 3 to 4 thousand
+// cycles a tile, as long as the split that it ran beside).  pos: the position of the
+// lane-th lowest bit of `low` (lanes 0 to 6).
+__device__ __forceinline__ void post_tile(const PostSmem &ps, uint64_t H, uint64_t low, int pos, int lane, uint32_t &X, uint32_t &C)
 {
-    uint32_t q = (uint32_t)__popcll(H & ps.c2) & 1u;
+    uint32_t q = 0;
     uint64_t x = 0;
 #pragma unroll 1
-    for (int i = 0; i < ps.n; i++) {
+    for (int i = lane; i < ps.n; i += 32) {
         const uint64_t P = ps.part[i];
         const int a = ps.a[i];
         const uint32_t hp = (uint32_t)__popcll(H & P) & 1u;
@@ -491,14 +494,21 @@ __device__ __forceinline__ void post_tile(const PostSmem &ps, uint64_t H, uint64
             x ^= 1ULL << a;
         }
     }
-    uint32_t f = 0;
-#pragma unroll
-    for (int j = 0; j < 5; j++) f |= ((uint32_t)__popcll(H & ps.tp[j]) & 1u) << j;
-    uint32_t xc = 0;
-    int k = 0;
-    for (uint64_t w = low; w; w &= w - 1, k++) xc |= (uint32_t)((x >> (__ffsll((long long)w) - 1)) & 1) << k;
-    X = xc;
-    C = ((uint32_t)__popcll(H & ps.c1) & 3u) | q << 2 | f << 3;
+    __syncwarp();
+    q = __reduce_xor_sync(0xffffffffu, q) ^ ((uint32_t)__popcll(H & ps.c2) & 1u);
+    x = (uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(x >> 32)) << 32 | __reduce_xor_sync(0xffffffffu, (uint32_t)x);
+    const uint32_t f = __ballot_sync(0xffffffffu, lane < 5 && (__popcll(H & ps.tp[lane < 5 ? lane : 0]) & 1));
+    const uint32_t xc = __ballot_sync(0xffffffffu, lane < 7 && ((x >> pos) & 1));
+    if (lane == 0) {
+        X = xc;
+        C = ((uint32_t)__popcll(H & ps.c1) & 3u) | q << 2 | f << 3;
+    }
+}
+// position of the k-th lowest set bit of w (0 where w has no more than k)
+__device__ __forceinline__ int nth_bit(uint64_t w, int k)
+{
+    for (int i = 0; i < k; i++) w &= w - 1;
+    return w ? __ffsll((long long)w) - 1 : 0;
 }
 __device__ __forceinline__ uint32_t post_rowpart(const PostSmem &ps, uint64_t l)
 {
@@ -649,8 +659,10 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         // the folded phase's row part, row by row (the same in every tile), and
         // the tile part of this CTA's first tile
         if (tid < kRows) postR[tid] = (uint8_t)post_rowpart(ps, tile_base(tid, t) ^ tile_base(0, t));
-        if (tid == kRows && blockIdx.x < n_tiles)
-            post_tile(ps, tile_base((uint64_t)blockIdx.x * kRows, t), tile_base(kRows - 1, t) ^ tile_base(0, t), postX[0], postC[0]);
+        if (warp == kRows / 32 && blockIdx.x < n_tiles) {
+            const uint64_t low = tile_base(kRows - 1, t) ^ tile_base(0, t);
+            post_tile(ps, tile_base((uint64_t)blockIdx.x * kRows, t), low, nth_bit(low, min(tid & 31, 7)), tid & 31, postX[0], postC[0]);
+        }
         __syncthreads();
     }
     chain_wait();
@@ -818,14 +830,20 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         // nothing to split
     } else if (tid >= kSplitThreads + kEpiThreads) {
         // ---------------------------------------------------------------- issuer
-        if (tid == kSplitThreads + kEpiThreads) {
+        // (one lane; with a folded phase the warp, whose lanes form the tile parts)
+        const int lane = tid & 31;
+        if (kPost || lane == 0) {
             const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
-            const uint64_t low = tile_base(kRows - 1, t) ^ tile_base(0, t);
+            const uint64_t low = kPost ? tile_base(kRows - 1, t) ^ tile_base(0, t) : 0;
+            const int pos = kPost ? nth_bit(low, min(lane, 7)) : 0;
             int it = 0;
-            const bool b_ready = mbar_wait_bounded(mbar_b_a, 0);
-            if (!b_ready) {
-                atomicExch(status, 1);
-                abort_flag = 1;
+            bool b_ready = true;
+            if (lane == 0) {
+                b_ready = mbar_wait_bounded(mbar_b_a, 0);
+                if (!b_ready) {
+                    atomicExch(status, 1);
+                    abort_flag = 1;
+                }
             }
             for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, it++) {
                 // the folded phase's tile part for tile it+1, while the planes of
@@ -834,31 +852,36 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                 // by tile it-1's MMAs); it reads tile it+1's after the last MMAs of
                 // tile it complete (committed after this write)
                 if (kPost && tile + gridDim.x < n_tiles)
-                    post_tile(ps, tile_base((tile + gridDim.x) * kRows, t), low, postX[(it + 1) & 3], postC[(it + 1) & 3]);
-                if (!mbar_wait_bounded(smem_u32(&mbar_planes), it & 1) || abort_flag) {
-                    atomicExch(status, 1);
-                    abort_flag = 1;
-                    break;
-                }
-                tc_fence_after();
-                // half h of tile it-1 must have been read out before half h of tile it
+                    post_tile(ps, tile_base((tile + gridDim.x) * kRows, t), low, pos, lane, postX[(it + 1) & 3], postC[(it + 1) & 3]);
                 bool ok = true;
-                for (int h = 0; h < 2 && ok; h++) {
-                    if (it > 0 && !mbar_wait_bounded(smem_u32(&mbar_free[h]), (it - 1) & 1)) {
+                if (lane == 0) {
+                    if (!mbar_wait_bounded(smem_u32(&mbar_planes), it & 1) || abort_flag) {
                         atomicExch(status, 1);
                         abort_flag = 1;
                         ok = false;
-                        break;
                     }
                     tc_fence_after();
-                    issue_c128_half(tmem, a0, b0, h, (M + 7) >> 3);
-                    mma_commit(smem_u32(&mbar_mma[h]));
+                    // half h of tile it-1 must have been read out before half h of tile it
+                    for (int h = 0; h < 2 && ok; h++) {
+                        if (it > 0 && !mbar_wait_bounded(smem_u32(&mbar_free[h]), (it - 1) & 1)) {
+                            atomicExch(status, 1);
+                            abort_flag = 1;
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        issue_c128_half(tmem, a0, b0, h, (M + 7) >> 3);
+                        mma_commit(smem_u32(&mbar_mma[h]));
+                    }
                 }
+                if constexpr (kPost) ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
                 if (!ok) break;
             }
-            // leave only after the last MMAs are complete (they read this CTA's planes)
-            if (it > 0 && !abort_flag) mbar_wait_bounded(smem_u32(&mbar_mma[1]), (it - 1) & 1);
-            if (!b_ready) mbar_wait_bounded(mbar_b_a, 0);   // its own copies in flight
+            if (lane == 0) {
+                // leave only after the last MMAs are complete (they read this CTA's planes)
+                if (it > 0 && !abort_flag) mbar_wait_bounded(smem_u32(&mbar_mma[1]), (it - 1) & 1);
+                if (!b_ready) mbar_wait_bounded(mbar_b_a, 0);   // its own copies in flight
+            }
         }
     } else {
         // ------------------------------------------------------------- epilogue
@@ -879,13 +902,17 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             const uint64_t g = tile * kRows + row;
             const bool valid = g < n_groups;
             double2 *p = psi + (valid ? tile_base(g, t) : 0);
-            uint32_t pe = 0, pf = 0;
+            uint32_t podd = 0, psign = 0;
             if constexpr (kPost) {
-                // i^pe (-1)^popc(m & pf) for member m of this row
+                // i^pe (-1)^popc(m & pf) for member m of this row: a swap where pe is odd;
+                // bit m of psign: the sign of the imaginary part (of the real part where
+                // pe is even, else its opposite)
                 const uint32_t X = postX[it & 3], C = postC[it & 3], Crow = postR[row];
                 const uint32_t sq = ((C ^ Crow) >> 2) ^ (uint32_t)__popc((uint32_t)row & X);
-                pe = ((C & 3u) + (Crow & 3u) + 2u * (sq & 1u)) & 3u;
-                pf = ((C ^ Crow) >> 3) & 31u;
+                const uint32_t pe = (C & 3u) + (Crow & 3u) + 2u * (sq & 1u), pf = (C ^ Crow) >> 3;
+                podd = pe << 31;
+                psign = (pe & 2u ? 0xFFFFFFFFu : 0u) ^ (pf & 1u ? 0xAAAAAAAAu : 0u) ^ (pf & 2u ? 0xCCCCCCCCu : 0u) ^
+                        (pf & 4u ? 0xF0F0F0F0u : 0u) ^ (pf & 8u ? 0xFF00FF00u : 0u) ^ (pf & 16u ? 0xFFFF0000u : 0u);
             }
             for (int h = 0; h < 2; h++) {
                 if (!mbar_wait_bounded(smem_u32(&mbar_mma[h]), it & 1) || abort_flag) {
@@ -963,8 +990,8 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                     }
                     const int m0 = (kHalfN * h + col) >> 1;   // columns 2m, 2m+1: re, im of member m
                     if constexpr (kPost) {
-                        rot_i_words(hw[0], lw[0], hw[1], lw[1], post_member(pe, pf, m0));
-                        rot_i_words(hw[2], lw[2], hw[3], lw[3], post_member(pe, pf, m0 + 1));
+                        rot_i_words(hw[0], lw[0], hw[1], lw[1], podd, psign << (31 - m0));
+                        rot_i_words(hw[2], lw[2], hw[3], lw[3], podd, psign << (30 - m0));
                     }
                     if (valid) {
                         p[moff[m0]] = make_double2(__hiloint2double((int)hw[0], (int)lw[0]),

@@ -248,18 +248,15 @@ __device__ __forceinline__ float2 rot_i(float2 v, uint32_t r)
     return make_float2(((r + 1u) & 2u) ? -a : a, (r & 2u) ? -b : b);
 }
 
-// the same on the two words of each FP64 value: a swap and sign-bit flips
-__device__ __forceinline__ void rot_i_words(uint32_t &h0, uint32_t &l0, uint32_t &h1, uint32_t &l1, uint32_t r)
+// the same on the two words of each FP64 value: a swap (odd: bit 31) and sign-bit flips
+// (sign: bit 31 for the imaginary part, its opposite for the real part of a swap)
+__device__ __forceinline__ void rot_i_words(uint32_t &h0, uint32_t &l0, uint32_t &h1, uint32_t &l1, uint32_t odd, uint32_t sign)
 {
-    if (r & 1u) {
-        const uint32_t th = h0, tl = l0;
-        h0 = h1;
-        l0 = l1;
-        h1 = th;
-        l1 = tl;
-    }
-    h0 ^= ((r + 1u) & 2u) ? 0x80000000u : 0u;
-    h1 ^= (r & 2u) ? 0x80000000u : 0u;
+    const uint32_t a = odd ? h1 : h0, al = odd ? l1 : l0, b = odd ? h0 : h1, bl = odd ? l0 : l1;
+    h0 = a ^ ((sign ^ odd) & 0x80000000u);
+    l0 = al;
+    h1 = b ^ (sign & 0x80000000u);
+    l1 = bl;
 }
 
 }  // namespace

@@ -225,3 +225,21 @@ def test_fold_of_the_identity_phase(dtype):
     alone, _ = lib_run(N, dtype, ops[:1], psi=psi)
     assert ms[1] == -1
     assert np.array_equal(got, alone)
+
+
+@pytest.mark.parametrize("targets", [(16, 17, 18, 19, 20), (0, 1, 2, 3, 4), (3, 8, 12, 13, 19)])
+def test_fold_over_several_tiles_per_block(targets):
+    """More tiles than blocks, so that tile parts are formed ahead of their tile: every
+    other qubit carries a term (even coefficients, CZ pairs in a ring and across it), and
+    the folded run equals the unfolded one bit for bit."""
+    n = 21
+    off = [q for q in range(n) if q not in targets]
+    coeff = np.zeros(n, dtype=np.int64)
+    coeff[off] = 2 * rng(50).integers(0, 4, len(off))
+    pairs = list(zip(off, off[1:] + off[:1])) + list(zip(off[:5], off[7:12])) + list(zip(targets, off[3:8]))
+    ops = [(qs.QS_OP_DENSE, targets, random_unitary(5, 51)), (qs.QS_OP_PHASE, pairs, coeff)]
+    psi = random_state(n, 52)
+    got, ms = lib_run(n, qs.QS_C128, ops, psi=psi)
+    plain, _ = lib_run(n, qs.QS_C128, ops, psi=psi, fold=False)
+    assert ms[1] == -1
+    assert np.array_equal(got, plain)
