@@ -134,6 +134,16 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
         *reinterpret_cast<float4 *>(A_h + cm_off(row, 4 * c)) = h;
         *reinterpret_cast<float4 *>(A_t + cm_off(row, 4 * c)) = tl;
     };
+    uint64_t low = 0;
+    uint32_t prow = 0;
+    int pos = 0;
+    bool quarter = false;
+    if constexpr (kPost) {
+        low = tile_base(kRows - 1, t) ^ tile_base(0, t);
+        pos = nth_bit(low, min(tid & 31, 7));
+        prow = post_rowpart(ps, tile_base(row, t) ^ tile_base(0, t));
+        quarter = ps.c1 != 0;
+    }
     load_tile(tile, v, valid, p);
     for (; tile < n_tiles; tile += gridDim.x) {
         // split: members 2c and 2c+1 fill K columns 4c..4c+3
@@ -169,6 +179,13 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
         float2 *const p_cur = kTwo ? psi + tile_base(tile * kRows + tid, t) : p;   // this thread's row
         const bool valid_cur = valid;
         load_tile(tile + gridDim.x, v, valid, p);
+        uint32_t podd = 0, psign = 0;
+        if constexpr (kPost) {
+            uint32_t X, C;
+            post_tile(ps, tile_base(tile * kRows, t), low, pos, tid & 31, X, C);
+            post_signs(X, C, prow, (uint32_t)row, podd, psign);
+            psign >>= kMem * part;
+        }
         bool ok = false;
         for (long it = 0; it < kWaitLimit; it++)
             if (mbar_try_wait(mbar_a, parity)) {
@@ -188,12 +205,15 @@ k_dense5_tc_c64(float2 *__restrict__ psi, uint64_t n_groups, TileLayout t, const
         parity ^= 1;
         tc_fence_after();
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kN / NP * part;
-        uint32_t pe = 0, pf = 0;
-        if constexpr (kPost) post_row(ps, (uint64_t)(p_cur - psi), pe, pf);
         // output of member m: head + corrections, times the folded phase's factor
         auto out_of = [&](const float *r, const float *q, int l, int m) {
             float2 v = make_float2(r[2 * l] + q[2 * l], r[2 * l + 1] + q[2 * l + 1]);
-            if constexpr (kPost) v = rot_i(v, post_member(pe, pf, kMem * part + m));
+            if constexpr (kPost) {
+                if (quarter) v = podd ? make_float2(v.y, v.x) : v;   // (CZ pairs alone never make pe odd)
+                const uint32_t s = psign << (31 - m);
+                v.x = __uint_as_float(__float_as_uint(v.x) ^ ((s ^ podd) & 0x80000000u));
+                v.y = __uint_as_float(__float_as_uint(v.y) ^ (s & 0x80000000u));
+            }
             return v;
         };
 #pragma unroll
@@ -407,7 +427,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t parity
 // states of a tile per CTA at most, where a tile's latency is the sweep (16 qubits,
 // 25 cycles 142 -> 134 us; 30 qubits 0.7% slower).
 // kPost (a phase op folded into the sweep): the phase of a row splits into a
-// part of its tile, formed one tile ahead by the issuing thread while it
+// part of its tile, formed one tile ahead by the issuing warp while it
 // waits for the planes (four slots by tile index), and a part of its row,
 // formed once per CTA (a table of 128); the epilogue combines the two.
 // Hand-offs per tile: mbar_planes (splitter thread 0 after the planes are
@@ -461,66 +481,6 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 constexpr size_t kStageC128 = (size_t)kSplitThreads * kMPT * 16;   // raw next tile: 64 KB
 constexpr size_t kSmemC128Pipe = kSmemC128 + kStageC128;
-
-// The folded phase of a row (kPost) split into the part of its tile and the
-// part of its row.  A row's base is b = H | l: H the base of the tile's first
-// group, l the row's bits among the 7 lowest group positions (`low`).  Then
-//   e(b) = popc(H & c1) + popc(l & c1) + 2 (q_H ^ q_l ^ parity(l & X_H))  (mod 4),
-//   flip(b) = flip(H) ^ flip(l),
-// where q_H, X_H depend on the tile alone (a term whose qubit a is set in H
-// adds parity(H & partners) to q_H and its partners to X_H; a term whose qubit
-// lies in `low` and whose partners meet H an odd number of times adds bit a to
-// X_H) and q_l on the row alone (parity(l & c2) and the terms with both ends
-// in the row's bits).  The tile's part is formed once per tile by the
-// MMA-issuing thread, the row's part once per CTA for each of its 128 rows;
-// X_H is kept as its bits at the `low` positions (bit k: the k-th lowest), so
-// parity(l & X_H) = parity(r & X) for row r of the tile.
-// A warp forms a tile's part, a term per lane (one thread took 15 terms to 3 to 4 thousand
-// cycles a tile, as long as the split that it ran beside).  pos: the position of the
-// lane-th lowest bit of `low` (lanes 0 to 6).
-__device__ __forceinline__ void post_tile(const PostSmem &ps, uint64_t H, uint64_t low, int pos, int lane, uint32_t &X, uint32_t &C)
-{
-    uint32_t q = 0;
-    uint64_t x = 0;
-#pragma unroll 1
-    for (int i = lane; i < ps.n; i += 32) {
-        const uint64_t P = ps.part[i];
-        const int a = ps.a[i];
-        const uint32_t hp = (uint32_t)__popcll(H & P) & 1u;
-        if ((H >> a) & 1) {
-            q ^= hp;
-            x ^= P;
-        } else if (((low >> a) & 1) && hp) {
-            x ^= 1ULL << a;
-        }
-    }
-    __syncwarp();
-    q = __reduce_xor_sync(0xffffffffu, q) ^ ((uint32_t)__popcll(H & ps.c2) & 1u);
-    x = (uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(x >> 32)) << 32 | __reduce_xor_sync(0xffffffffu, (uint32_t)x);
-    const uint32_t f = __ballot_sync(0xffffffffu, lane < 5 && (__popcll(H & ps.tp[lane < 5 ? lane : 0]) & 1));
-    const uint32_t xc = __ballot_sync(0xffffffffu, lane < 7 && ((x >> pos) & 1));
-    if (lane == 0) {
-        X = xc;
-        C = ((uint32_t)__popcll(H & ps.c1) & 3u) | q << 2 | f << 3;
-    }
-}
-// position of the k-th lowest set bit of w (0 where w has no more than k)
-__device__ __forceinline__ int nth_bit(uint64_t w, int k)
-{
-    for (int i = 0; i < k; i++) w &= w - 1;
-    return w ? __ffsll((long long)w) - 1 : 0;
-}
-__device__ __forceinline__ uint32_t post_rowpart(const PostSmem &ps, uint64_t l)
-{
-    uint32_t q = (uint32_t)__popcll(l & ps.c2) & 1u;
-#pragma unroll 1
-    for (int i = 0; i < ps.n; i++)
-        if ((l >> ps.a[i]) & 1) q ^= (uint32_t)__popcll(l & ps.part[i]) & 1u;
-    uint32_t f = 0;
-#pragma unroll
-    for (int j = 0; j < 5; j++) f |= ((uint32_t)__popcll(l & ps.tp[j]) & 1u) << j;
-    return ((uint32_t)__popcll(l & ps.c1) & 3u) | q << 2 | f << 3;
-}
 
 // The double of T = th:tl (rounded to nearest even) with `scale` added to its exponent
 // field, in integer operations; T = 0 gives +0.0.
@@ -661,7 +621,9 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         if (tid < kRows) postR[tid] = (uint8_t)post_rowpart(ps, tile_base(tid, t) ^ tile_base(0, t));
         if (warp == kRows / 32 && blockIdx.x < n_tiles) {
             const uint64_t low = tile_base(kRows - 1, t) ^ tile_base(0, t);
-            post_tile(ps, tile_base((uint64_t)blockIdx.x * kRows, t), low, nth_bit(low, min(tid & 31, 7)), tid & 31, postX[0], postC[0]);
+            uint32_t X, C;
+            post_tile(ps, tile_base((uint64_t)blockIdx.x * kRows, t), low, nth_bit(low, min(tid & 31, 7)), tid & 31, X, C);
+            if ((tid & 31) == 0) postX[0] = X, postC[0] = C;
         }
         __syncthreads();
     }
@@ -851,8 +813,11 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                 // the epilogue read before releasing tile it-2's half 0 (waited for
                 // by tile it-1's MMAs); it reads tile it+1's after the last MMAs of
                 // tile it complete (committed after this write)
-                if (kPost && tile + gridDim.x < n_tiles)
-                    post_tile(ps, tile_base((tile + gridDim.x) * kRows, t), low, pos, lane, postX[(it + 1) & 3], postC[(it + 1) & 3]);
+                if (kPost && tile + gridDim.x < n_tiles) {
+                    uint32_t X, C;
+                    post_tile(ps, tile_base((tile + gridDim.x) * kRows, t), low, pos, lane, X, C);
+                    if (lane == 0) postX[(it + 1) & 3] = X, postC[(it + 1) & 3] = C;
+                }
                 bool ok = true;
                 if (lane == 0) {
                     if (!mbar_wait_bounded(smem_u32(&mbar_planes), it & 1) || abort_flag) {
@@ -894,8 +859,10 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
         // that some warps convert while others read, and one value in four (kSub: one in
         // six) rebuilt in integer operations.  28 qubits, high targets (kBulk) 1.98 -> 1.94
         // ms; widening 27 -> 28 qubits (kSub) 1.62 -> 1.59; with cp.async staging the
-        // splitters' copies are the longer part and it measured 2 to 4% slower.
-        constexpr bool kInTurn = kBulk || kSub != 0;
+        // splitters' copies are the longer part and it measured 2 to 4% slower (1.5% faster
+        // with a folded phase, which needs the registers: 30 qubits 8.79 -> 8.65 ms).
+        constexpr bool kInTurn = kBulk || kSub != 0 || kPost;
+        const bool quarter = kPost && ps.c1 != 0;
         int it = 0;
         bool failed = false;
         for (uint64_t tile = blockIdx.x; tile < n_tiles && !failed; tile += gridDim.x, it++) {
@@ -904,15 +871,7 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
             double2 *p = psi + (valid ? tile_base(g, t) : 0);
             uint32_t podd = 0, psign = 0;
             if constexpr (kPost) {
-                // i^pe (-1)^popc(m & pf) for member m of this row: a swap where pe is odd;
-                // bit m of psign: the sign of the imaginary part (of the real part where
-                // pe is even, else its opposite)
-                const uint32_t X = postX[it & 3], C = postC[it & 3], Crow = postR[row];
-                const uint32_t sq = ((C ^ Crow) >> 2) ^ (uint32_t)__popc((uint32_t)row & X);
-                const uint32_t pe = (C & 3u) + (Crow & 3u) + 2u * (sq & 1u), pf = (C ^ Crow) >> 3;
-                podd = pe << 31;
-                psign = (pe & 2u ? 0xFFFFFFFFu : 0u) ^ (pf & 1u ? 0xAAAAAAAAu : 0u) ^ (pf & 2u ? 0xCCCCCCCCu : 0u) ^
-                        (pf & 4u ? 0xF0F0F0F0u : 0u) ^ (pf & 8u ? 0xFF00FF00u : 0u) ^ (pf & 16u ? 0xFFFF0000u : 0u);
+                post_signs(postX[it & 3], postC[it & 3], postR[row], (uint32_t)row, podd, psign);
             }
             for (int h = 0; h < 2; h++) {
                 if (!mbar_wait_bounded(smem_u32(&mbar_mma[h]), it & 1) || abort_flag) {
@@ -990,8 +949,15 @@ k_dense5_tc_c128_pipe(double2 *__restrict__ psi, uint64_t n_groups, TileLayout t
                     }
                     const int m0 = (kHalfN * h + col) >> 1;   // columns 2m, 2m+1: re, im of member m
                     if constexpr (kPost) {
-                        rot_i_words(hw[0], lw[0], hw[1], lw[1], podd, psign << (31 - m0));
-                        rot_i_words(hw[2], lw[2], hw[3], lw[3], podd, psign << (30 - m0));
+                        if (quarter) {   // (CZ pairs alone never make pe odd)
+                            swap_if(podd, hw[0], lw[0], hw[1], lw[1]);
+                            swap_if(podd, hw[2], lw[2], hw[3], lw[3]);
+                        }
+                        const uint32_t s0 = psign << (31 - m0), s1 = psign << (30 - m0);
+                        hw[0] ^= (s0 ^ podd) & 0x80000000u;
+                        hw[1] ^= s0 & 0x80000000u;
+                        hw[2] ^= (s1 ^ podd) & 0x80000000u;
+                        hw[3] ^= s1 & 0x80000000u;
                     }
                     if (valid) {
                         p[moff[m0]] = make_double2(__hiloint2double((int)hw[0], (int)lw[0]),

@@ -248,14 +248,85 @@ __device__ __forceinline__ float2 rot_i(float2 v, uint32_t r)
     return make_float2(((r + 1u) & 2u) ? -a : a, (r & 2u) ? -b : b);
 }
 
-// the same on the two words of each FP64 value: a swap (odd: bit 31) and sign-bit flips
-// (sign: bit 31 for the imaginary part, its opposite for the real part of a swap)
-__device__ __forceinline__ void rot_i_words(uint32_t &h0, uint32_t &l0, uint32_t &h1, uint32_t &l1, uint32_t odd, uint32_t sign)
+// The folded phase of a row (kPost) split into the part of its tile and the
+// part of its row.  A row's base is b = H | l: H the base of the tile's first
+// group, l the row's bits among the 7 lowest group positions (`low`).  Then
+//   e(b) = popc(H & c1) + popc(l & c1) + 2 (q_H ^ q_l ^ parity(l & X_H))  (mod 4),
+//   flip(b) = flip(H) ^ flip(l),
+// where q_H, X_H depend on the tile alone (a term whose qubit a is set in H
+// adds parity(H & partners) to q_H and its partners to X_H; a term whose qubit
+// lies in `low` and whose partners meet H an odd number of times adds bit a to
+// X_H) and q_l on the row alone (parity(l & c2) and the terms with both ends
+// in the row's bits).  The tile's part is formed once per tile by a warp, the
+// row's part once per CTA for each of its 128 rows;
+// X_H is kept as its bits at the `low` positions (bit k: the k-th lowest), so
+// parity(l & X_H) = parity(r & X) for row r of the tile.
+// A term per lane: complex128, 30 qubits, 9.37 ms where one thread went through the terms,
+// as long as the split that it ran beside, 8.43 ms so (8.06 with the row's signs in one
+// word and no swaps for CZ pairs; 7.43 without a phase); complex64, 28 qubits, 719 us where
+// every row's thread did, 704 so (682 without a phase).  pos: the position of the
+// lane-th lowest bit of `low` (lanes 0 to 6).  Every lane gets the result.
+__device__ __forceinline__ void post_tile(const PostSmem &ps, uint64_t H, uint64_t low, int pos, int lane, uint32_t &X, uint32_t &C)
+{
+    uint32_t q = 0;
+    uint64_t x = 0;
+#pragma unroll 1
+    for (int i = lane; i < ps.n; i += 32) {
+        const uint64_t P = ps.part[i];
+        const int a = ps.a[i];
+        const uint32_t hp = (uint32_t)__popcll(H & P) & 1u;
+        if ((H >> a) & 1) {
+            q ^= hp;
+            x ^= P;
+        } else if (((low >> a) & 1) && hp) {
+            x ^= 1ULL << a;
+        }
+    }
+    __syncwarp();
+    q = __reduce_xor_sync(0xffffffffu, q) ^ ((uint32_t)__popcll(H & ps.c2) & 1u);
+    x = (uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(x >> 32)) << 32 | __reduce_xor_sync(0xffffffffu, (uint32_t)x);
+    const uint32_t f = __ballot_sync(0xffffffffu, lane < 5 && (__popcll(H & ps.tp[lane < 5 ? lane : 0]) & 1));
+    const uint32_t xc = __ballot_sync(0xffffffffu, lane < 7 && ((x >> pos) & 1));
+    X = xc;
+    C = ((uint32_t)__popcll(H & ps.c1) & 3u) | q << 2 | f << 3;
+}
+// position of the k-th lowest set bit of w (0 where w has no more than k)
+__device__ __forceinline__ int nth_bit(uint64_t w, int k)
+{
+    for (int i = 0; i < k; i++) w &= w - 1;
+    return w ? __ffsll((long long)w) - 1 : 0;
+}
+__device__ __forceinline__ uint32_t post_rowpart(const PostSmem &ps, uint64_t l)
+{
+    uint32_t q = (uint32_t)__popcll(l & ps.c2) & 1u;
+#pragma unroll 1
+    for (int i = 0; i < ps.n; i++)
+        if ((l >> ps.a[i]) & 1) q ^= (uint32_t)__popcll(l & ps.part[i]) & 1u;
+    uint32_t f = 0;
+#pragma unroll
+    for (int j = 0; j < 5; j++) f |= ((uint32_t)__popcll(l & ps.tp[j]) & 1u) << j;
+    return ((uint32_t)__popcll(l & ps.c1) & 3u) | q << 2 | f << 3;
+}
+
+// i^pe (-1)^popc(m & pf) for member m of a row: a swap of real and imaginary part where
+// pe is odd (bit 31 of `odd`), and bit m of `sign`: the sign of the imaginary part (of the
+// real part where pe is even, else its opposite)
+__device__ __forceinline__ void post_signs(uint32_t X, uint32_t C, uint32_t Crow, uint32_t row, uint32_t &odd, uint32_t &sign)
+{
+    const uint32_t sq = ((C ^ Crow) >> 2) ^ (uint32_t)__popc(row & X);
+    const uint32_t pe = (C & 3u) + (Crow & 3u) + 2u * (sq & 1u), pf = (C ^ Crow) >> 3;
+    odd = pe << 31;
+    sign = (pe & 2u ? 0xFFFFFFFFu : 0u) ^ (pf & 1u ? 0xAAAAAAAAu : 0u) ^ (pf & 2u ? 0xCCCCCCCCu : 0u) ^
+           (pf & 4u ? 0xF0F0F0F0u : 0u) ^ (pf & 8u ? 0xFF00FF00u : 0u) ^ (pf & 16u ? 0xFFFF0000u : 0u);
+}
+
+// two FP64 values, as words, change places where `odd` is not 0
+__device__ __forceinline__ void swap_if(uint32_t odd, uint32_t &h0, uint32_t &l0, uint32_t &h1, uint32_t &l1)
 {
     const uint32_t a = odd ? h1 : h0, al = odd ? l1 : l0, b = odd ? h0 : h1, bl = odd ? l0 : l1;
-    h0 = a ^ ((sign ^ odd) & 0x80000000u);
+    h0 = a;
     l0 = al;
-    h1 = b ^ (sign & 0x80000000u);
+    h1 = b;
     l1 = bl;
 }
 
