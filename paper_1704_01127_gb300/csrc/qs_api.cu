@@ -586,9 +586,11 @@ __device__ __forceinline__ double chain_add(double c, double p, double &half)
 // The same for N groups of 32 values, half[k] and full[k] after group k's lanes 15 and
 // 31: all N at once while the sum stays in one binade without ties (the terms then
 // depend on c's exponent alone), else one group after another, addition by addition.
-// 2^e the start of c's binade: for p < 2^(e-20) a term is the low word of fl(2^e + p)
-// and a tie needs 20 zero bits at p's end.  Where some value has those (equal or
-// real-valued amplitudes) the bits that a term drops are looked at; where some is
+// 2^e the start of c's binade, u = 2^(e-52): for p < 2^(e-20) - 2^(e-41) a term is the
+// low word of fl(2^e + p) (it rounds to at most 2^32 - 2^11 units; the p up to 2^(e-20)
+// left out, one value of the high word, can round to 2^32 units, which that word does
+// not hold) and a tie needs 20 zero bits at p's end.  Where some value has those (equal
+// or real-valued amplitudes) the bits that a term drops are looked at; where some is
 // larger, the terms come from chain_term.
 template <int N>
 __device__ __forceinline__ double chain_add_n(double c, const double *p, double *half, double *full)
@@ -597,7 +599,7 @@ __device__ __forceinline__ double chain_add_n(double c, const double *p, double 
     const int E = (int)(cb >> 52);
     const bool low = (threadIdx.x & 31) < 16;
     const double c0 = __longlong_as_double((long long)(cb & 0x7FF0000000000000ULL));
-    const uint32_t top = (uint32_t)max(E - 20, 0) << 20;
+    const uint32_t top = ((uint32_t)max(E - 20, 1) << 20) - 1u;
     uint32_t v[N], any = 0;
     bool large = E < 64, zeros = false;
 #pragma unroll
