@@ -118,6 +118,7 @@ k_probs(const C *__restrict__ psi, uint64_t first, uint64_t count, double *__res
 using qsd::ff;
 using qsd::ff_abs_double;
 using qsd::ff_accumulate;
+using qsd::ff_add;
 using qsd::ff_p_ln_p;
 using qsd::ff_fast_two_sum;
 using qsd::ff_sqr_loose;
@@ -131,20 +132,6 @@ __device__ __align__(16) FFLogTable g_fflog;
 
 __global__ void k_fflog_init() { ff_log_table_init(g_fflog); }
 
-// Per-block FP64 partial sums of (p, -p ln p, p, p^2); NSTAT = 1 or 4.  The
-// mean of N p equals the sum of p, and the mean of (N p)^2 is N sum p^2, so
-// the moments cost one product per amplitude; the host applies the factor N.
-// Everything runs in float-float on the FP32 pipe (GB300's FP64 pipe runs at
-// 1/64 of its rate): complex128 amplitudes are split into float-float by bit
-// manipulation (48 of their 53 bits), complex64 ones give p exactly (x^2 and
-// y^2 with their FMA rounding errors).  p, p^2 and p ln p (table-driven log,
-// ff_p_ln_p) are summed per thread in float-float; the rounding errors of
-// those sums are random, about 2^-48 of the partial sum per step, so the
-// total norm of a 30-qubit state carries an error near 1e-15.  p below 2^-79
-// (where the low half of p's float-float form would leave the normal float
-// range) takes p ln p from the FP64 math library, and complex128 amplitudes of
-// 2^30 or more (unnormalised input) are summed in FP64 throughout; p below the
-// normal double range contributes less than 1e-305 and is left out.
 // p ln p by the FP64 math library, out of the way of the common cases' code
 __device__ __noinline__ double p_ln_p_rare(double p) { return p * log(p); }
 
@@ -152,7 +139,22 @@ __device__ __noinline__ double p_ln_p_rare(double p) { return p * log(p); }
 // reduces the block (every thread of the block calls it).
 struct StatsAcc {
     double d0 = 0, d3 = 0, dent = 0;
-    ff f0{0.f, 0.f}, f3{0.f, 0.f}, fent{0.f, 0.f};
+    ff f0{0.f, 0.f}, f3{0.f, 0.f}, fent{0.f, 0.f};   // of the terms since the last fold()
+    ff g0{0.f, 0.f}, g3{0.f, 0.f}, gent{0.f, 0.f};   // of those before
+
+    // After every kTerms amplitudes: their sums into the normalised ones.
+    static constexpr int kTerms = 16;
+    template <int NSTAT>
+    __device__ __forceinline__ void fold()
+    {
+        g0 = ff_add(g0, f0);
+        f0 = ff{0.f, 0.f};
+        if (NSTAT == 4) {
+            g3 = ff_add(g3, f3);
+            gent = ff_add(gent, fent);
+            f3 = fent = ff{0.f, 0.f};
+        }
+    }
 
     template <int NSTAT>
     __device__ __forceinline__ void add(const double2 a, const FFLogTable &lt)
@@ -211,14 +213,15 @@ struct StatsAcc {
 
     // part[blockIdx.x * NSTAT + j]: the block's sums of (p, -p ln p, p, p^2)
     template <int NSTAT>
-    __device__ void partials(double *__restrict__ part) const
+    __device__ void partials(double *__restrict__ part)
     {
+        fold<NSTAT>();
         double acc[NSTAT];
-        acc[0] = d0 + ((double)f0.hi + (double)f0.lo);
+        acc[0] = d0 + ((double)g0.hi + (double)g0.lo);
         if (NSTAT == 4) {
-            acc[NSTAT > 1 ? 1 : 0] = -(dent + ((double)fent.hi + (double)fent.lo));
+            acc[NSTAT > 1 ? 1 : 0] = -(dent + ((double)gent.hi + (double)gent.lo));
             acc[NSTAT > 2 ? 2 : 0] = acc[0];
-            acc[NSTAT > 3 ? 3 : 0] = d3 + ((double)f3.hi + (double)f3.lo);
+            acc[NSTAT > 3 ? 3 : 0] = d3 + ((double)g3.hi + (double)g3.lo);
         }
         __shared__ double red[NSTAT][32];
 #pragma unroll
@@ -257,11 +260,13 @@ __device__ __forceinline__ void load_fflog(FFLogTable &lt)
 // the moments cost one product per amplitude; the host applies the factor N.
 // Everything runs in float-float on the FP32 pipe (GB300's FP64 pipe runs at
 // 1/64 of its rate): complex128 amplitudes are split into float-float by bit
-// manipulation (48 of their 53 bits), complex64 ones give p exactly (x^2 and
-// y^2 with their FMA rounding errors).  p, p^2 and p ln p (table-driven log,
-// ff_p_ln_p) are summed per thread in float-float; the rounding errors of
-// those sums are random, about 2^-48 of the partial sum per step, so the
-// total norm of a 30-qubit state carries an error near 1e-15.  p below 2^-79
+// manipulation (the lowest 29 of their 53 bits rounded to 24), complex64 ones give
+// p rounded to 32 bits.  p, p^2 and p ln p (table-driven log, ff_p_ln_p) are summed
+// per thread in float-float, in sums of 16 terms that go into normalised ones.
+// Errors against exact sums at 28 qubits, relative: random amplitudes 3e-15 (p), 2e-15
+// (entropy), 6e-15 (p^2); equal amplitudes, whose rounding errors add up, up to 3e-14
+// (1.7e-11 without the sums of 16; 1.4e-13 with each term added to a normalised sum).
+// The sums of 16 cost 1% of the pass (complex64: 2%).  p below 2^-79
 // (where the low half of p's float-float form would leave the normal float
 // range) takes p ln p from the FP64 math library, and complex128 amplitudes of
 // 2^30 or more (unnormalised input) are summed in FP64 throughout; p below the
@@ -276,7 +281,9 @@ __global__ void k_stats_partial(const C *__restrict__ psi, uint64_t N, double *_
     // each thread loads kAhead amplitudes (block-strided, so every load of a
     // warp is contiguous) before it adds them up: more loads in flight
     constexpr int kAhead = c128 ? 4 : 8;
+    constexpr uint32_t kBatches = StatsAcc::kTerms / kAhead;
     const uint64_t span = (uint64_t)blockDim.x * kAhead;
+    uint32_t batch = 0;
     for (uint64_t base = (uint64_t)blockIdx.x * span; base < N; base += (uint64_t)gridDim.x * span) {
         C av[kAhead];
 #pragma unroll
@@ -286,6 +293,7 @@ __global__ void k_stats_partial(const C *__restrict__ psi, uint64_t N, double *_
         }
 #pragma unroll
         for (int k = 0; k < kAhead; k++) acc.add<NSTAT>(av[k], lt);
+        if (++batch % kBatches == 0) acc.fold<NSTAT>();
     }
     acc.partials<NSTAT>(part);
 }
@@ -461,8 +469,8 @@ __device__ __forceinline__ double piece_sum(const double2 *__restrict__ p, F see
 // (One piece after another: unrolled altogether, with the statistics, the code leaves
 // the instruction cache.)  With the statistics, 29 qubits complex64: 3.33 ms as one
 // 32-value run per lane, 1.71 ms.
-template <typename C, typename F>
-__device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen)
+template <typename C, typename F, typename G>
+__device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen, G piece_seen)
 {
     using V = std::conditional_t<sizeof(C) == 8, float4, double2>;
     constexpr int kPieces = sizeof(C) == 8 ? 2 : 4;
@@ -475,6 +483,7 @@ __device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen)
 #pragma unroll
         for (int j = 0; j + 1 < kPieces; j++) v[j] = v[j + 1];
         v[kPieces - 1] = piece_sum(p + 256 * i, seen);
+        piece_seen();
     }
     halve<kPieces>(v, 8);
     if constexpr (kPieces == 4) halve<2>(v, 16);
@@ -493,7 +502,7 @@ k_block_sums(const C *__restrict__ psi, uint64_t nb, double *__restrict__ out)
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t b = warp; b < nb; b += nwarps) {
-        const double v = block_sum(psi + b * 1024, [](const C &) {});
+        const double v = block_sum(psi + b * 1024, [](const C &) {}, [] {});
         if ((threadIdx.x & 31) == 0) out[b] = v;
     }
 }
@@ -512,7 +521,8 @@ k_block_sums_stats(const C *__restrict__ psi, uint64_t nb, double *__restrict__ 
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t b = warp; b < nb; b += nwarps) {
-        const double v = block_sum(psi + b * 1024, [&](const C &a) { acc.add<4>(a, lt); });
+        const double v = block_sum(
+            psi + b * 1024, [&](const C &a) { acc.add<4>(a, lt); }, [&] { acc.fold<4>(); });   // 16 amplitudes a piece
         if ((threadIdx.x & 31) == 0) out[b] = v;
     }
     acc.partials<4>(part);

@@ -314,8 +314,10 @@ __device__ __forceinline__ ff ff_sqr_loose(ff x)
     return ff{p, fmaf(__fadd_rn(x.hi, x.hi), x.lo, fmaf(x.hi, x.hi, -p))};
 }
 // s += a, the error of the high parts' sum and a's low part collected in s.lo and
-// never folded back (Ogita, Rump and Oishi's Sum2, SIAM J. Sci. Comput. 26,
-// 2005): the sum's error is that of adding the low parts in FP32
+// not folded back (Ogita, Rump and Oishi's Sum2, SIAM J. Sci. Comput. 26, 2005): s.lo
+// grows with the number of terms, and its roundings with it (of k equal terms they all
+// go one way, some k^2 2^-50 of the sum), so a sum takes a few terms and goes into
+// another one by ff_add
 __device__ __forceinline__ void ff_accumulate(ff &s, ff a)
 {
     const ff t = ff_two_sum(s.hi, a.hi);
@@ -327,6 +329,12 @@ __device__ __forceinline__ void ff_accumulate(ff &s, float a)
     const ff t = ff_two_sum(s.hi, a);
     s.hi = t.hi;
     s.lo = __fadd_rn(s.lo, t.lo);
+}
+// a + b, normalised
+__device__ __forceinline__ ff ff_add(ff a, ff b)
+{
+    const ff s = ff_two_sum(a.hi, b.hi);
+    return ff_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
 // |d| of a double with |d| in [2^-60, 2^30), its high word h without the sign:
 // hi = its top 24 significant bits (the exponent rebased by flipping one bit),
