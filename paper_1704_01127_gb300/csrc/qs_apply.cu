@@ -172,7 +172,10 @@ k_diag(typename cplx<R>::t *__restrict__ psi, int n, int L, int k, const int *__
 // coefficients' bits have odd parity; two rows are therefore paired so that
 // exactly one of a thread's two amplitudes is odd (the second row's column with
 // its lowest odd bit flipped when the rows' parities agree), and one rotation
-// serves both: 2 FP64 operations per amplitude, below the HBM time.
+// serves both: 2 FP64 operations per amplitude, below the HBM time.  Without an odd
+// coefficient on the lanes' bits, rows that differ in an odd row bit are paired, or
+// else all lanes and rows of a step are alike and the odd steps alone reach the FP64
+// pipe (27 qubits, one T gate on qubits 5 to 12 or 26: 1020 to 1070 -> 560 to 610 us).
 // 27 qubits complex128, T-type and CZ terms: 1139 -> 680 us (94% of the HBM copy
 // rate); 28 qubits complex64: 996 -> 680 us; a phase op on 14 qubits: 53 -> 4 us
 // (chunks used to be 2^14 amplitudes with a table entry each, built by every
@@ -216,7 +219,9 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
     const int m02 = odd ? qsd::phase_low(e2, cm, act, part, n_act, rb) : 0;
     const bool in = e < (1u << rb);
     const bool any_odd = cm[0] != 0;
-    const bool pairs = odd != 0 && rows > 1 && rb == RB;
+    // (no such bit, but one of the two lowest row bits: rows that differ in it are paired as they are)
+    const uint32_t odd_row = VEC == 1 && odd == 0 ? (uint32_t)(cm[0] >> rb) & (uint32_t)(rows - 1) & 3u : 0u;
+    const bool pairs = (odd | odd_row) != 0 && rows > 1 && rb == RB, two_apart = odd_row == 2u;
     __syncthreads();
     chain_wait();
     const uint64_t n_chunks = 1ULL << (n - L);
@@ -241,7 +246,7 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
             C *p[kAhead];
 #pragma unroll
             for (int j = 0; j < kAhead; j++) {
-                const int rj = r + j;
+                const int rj = r + (two_apart ? (j & 1) << 1 | j >> 1 : j);
                 const bool ok = rj < rows;
                 const int mr = ok ? row_m[rj] + mh + 4 * __popc((uint32_t)rj & Mr) : 0;
                 const uint32_t X = ok ? row_x[rj] ^ Me : 0u;
@@ -276,11 +281,20 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
                     else v[j + 1][0] = t;
                 }
             } else if (any_odd) {
+                // one branch around all rows: the compiler turns a branch around one row's four
+                // FP64 instructions into predicates, and the FP64 pipe takes those too
+                int o = VEC == 2;
 #pragma unroll
                 for (int j = 0; j < kAhead; j++)
 #pragma unroll
-                    for (int k = 0; k < VEC; k++)
-                        if (m[j][k] & 1) v[j][k] = qsd::eighth_turn(v[j][k]);
+                    for (int k = 0; k < VEC; k++) o |= m[j][k];
+                if (o & 1) {
+#pragma unroll
+                    for (int j = 0; j < kAhead; j++)
+#pragma unroll
+                        for (int k = 0; k < VEC; k++)
+                            if (m[j][k] & 1) v[j][k] = qsd::eighth_turn(v[j][k]);
+                }
             }
 #pragma unroll
             for (int j = 0; j < kAhead; j++) {

@@ -45,6 +45,27 @@ def test_phase_rows_and_chunks(dtype, odd, n):
     assert np.all(np.abs(out - ref) <= bound * np.abs(psi))
 
 
+@pytest.mark.parametrize("bits", [(8,), (9,), (8, 9), (9, 12), (10,), (6, 8)])
+@pytest.mark.parametrize("n", [9, 10, 13, 18, 19, 21])
+def test_phase_odd_rows(n, bits):
+    """Odd coefficients on row bits, none on the lanes' bits: rows next to one another or
+    two apart make a pair."""
+    coeff, edges = random_phase_poly(n, n, n)
+    coeff = np.asarray(coeff) // 2 * 2
+    coeff[[b for b in bits if b < n]] += 1
+    psi = random_state(n, n)
+    ref = psi.copy()
+    sim.apply_phase(ref, coeff, edges)
+    h = qs.qs_alloc(n, qs.QS_C128)
+    try:
+        qs.qs_set_amplitudes(h, psi)
+        qs.qs_apply_phase(h, coeff, edges)
+        out = qs.qs_get_amplitudes(h)
+    finally:
+        qs.qs_free(h)
+    assert np.all(np.abs(out - ref) <= 8 * EPS[qs.QS_C128] * np.abs(psi))
+
+
 @pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
 @pytest.mark.parametrize("n,k", [(1, 1), (2, 2), (8, 3), (9, 9), (10, 1), (14, 12), (19, 6), (20, 12), (23, 5)])
 def test_table_rows_and_chunks(dtype, n, k):
@@ -61,3 +82,36 @@ def test_table_rows_and_chunks(dtype, n, k):
         qs.qs_free(h)
     # the table's rounding, one rounded product and one rounded sum per component
     assert np.all(np.abs(out - ref) <= 8 * EPS[dtype] * np.abs(psi))
+
+
+def device_ms(calls, reps=20):
+    torch = pytest.importorskip("torch")
+    out = []
+    for call in calls:
+        best = float("inf")
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(reps):
+                call()
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) / reps)
+        out.append(best)
+    return out
+
+
+@pytest.mark.parametrize("q", [5, 8, 9, 12, 24])
+def test_one_t_gate_costs_no_more_than_the_whole_state(q):
+    """complex128: a T gate off the lanes' bits turns half of the amplitudes, so it takes no
+    longer than one on bit 0, which reads and writes every sector (it took 1.6 to 1.8
+    times as long where the FP64 pipe was given the other half as well)."""
+    n = 25
+    h = qs.qs_alloc(n, qs.QS_C128)
+    try:
+        qs.qs_init_uniform(h)
+        t = [np.eye(n, dtype=int)[b] for b in (0, q)]
+        all_of_it, half = device_ms([lambda c=c: qs.qs_apply_phase(h, c, []) for c in t])
+    finally:
+        qs.qs_free(h)
+    assert half <= 1.25 * all_of_it
