@@ -175,7 +175,7 @@ k_diag(typename cplx<R>::t *__restrict__ psi, int n, int L, int k, const int *__
 // serves both: 2 FP64 operations per amplitude, below the HBM time.  Without an odd
 // coefficient on the lanes' bits, rows that differ in an odd row bit are paired, or
 // else all lanes and rows of a step are alike and the odd steps alone reach the FP64
-// pipe (27 qubits, one T gate on qubits 5 to 12 or 26: 1020 to 1070 -> 560 to 610 us).
+// pipe (27 qubits, one T gate on qubits 5 to 12 or 26: 1020 to 1070 -> 550 to 580 us).
 // 27 qubits complex128, T-type and CZ terms: 1139 -> 680 us (94% of the HBM copy
 // rate); 28 qubits complex64: 996 -> 680 us; a phase op on 14 qubits: 53 -> 4 us
 // (chunks used to be 2^14 amplitudes with a table entry each, built by every
@@ -225,6 +225,13 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
     __syncthreads();
     chain_wait();
     const uint64_t n_chunks = 1ULL << (n - L);
+    // no factor on a chunk's own bits alone: chunks that none of the others reach are passed over
+    // (complex128, 27 qubits, T on qubit 26 608 -> 555 us, CZ on 25 and 26 307 -> 184)
+    const uint64_t own = (1ULL << L) - 1ULL;
+    uint64_t low = (cm[0] | cm[1] | cm[2]) & own;
+    for (int t = lane; t < n_act; t += 32)
+        if (act[t] < L) low |= part[t] & own;
+    const bool flat = !__any_sync(0xffffffffu, low != 0);
     constexpr int kAhead = kDiagAhead;
     for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
         const uint64_t h = ch << L;
@@ -239,7 +246,7 @@ k_phase(typename cplx<R>::t *__restrict__ psi, int n, int L, const qs_phase_dev 
         parh = __reduce_xor_sync(0xffffffffu, parh & 1u);
         const int mh = __popcll(h & cm[0]) + 2 * __popcll(h & cm[1]) + 4 * (__popcll(h & cm[2]) + (int)parh);
         const uint32_t Me = Mh & ((1u << rb) - 1u), Mr = Mh >> rb;
-        if (!in) continue;
+        if (!in || (flat && Mh == 0 && (mh & 7) == 0)) continue;
         for (int r = 0; r < rows; r += kAhead) {
             int m[kAhead][VEC];
             C v[kAhead][VEC];
@@ -371,16 +378,21 @@ int qs_launch_dense(qs_state *s, const int *sorted_qubits, int k, const void *de
                                : launch_dense_r<float>(s, sorted_qubits, k, dev_matrix);
 }
 
-// Chunk bits of a diagonal sweep: up to 32 rows, fewer where the chunks would
-// not fill the GPU; *grid: its blocks.
+// Chunk bits of a diagonal sweep: up to 32 rows, fewer (4 at least) where a block would
+// get less than four chunks, and fewer still where the chunks would not fill the GPU
+// (complex128 table, 23 qubits: 79 us with 1.7 chunks a block, 72 so).
+// *grid: its blocks.  Their number is odd where blocks take several chunks: a block's
+// chunks then differ in every bit of their number.  (With an even one the blocks split
+// by the lowest bit, and one T gate or CZ on that qubit left half of them without
+// work: complex128, 27 qubits, T on qubit 13 1080 us, 567 so.)
 template <typename R>
 static int diag_chunk(int n, int *grid)
 {
     const int rb = std::min(n, kDiagRowBits<R>);
     const uint64_t cap = (uint64_t)sm_count() * 4;
     int L = std::min(n, rb + 5);
-    while (L > rb && (1ULL << (n - L)) < cap) L--;
-    *grid = (int)std::min<uint64_t>(1ULL << (n - L), cap);
+    while (L > rb && (1ULL << (n - L)) < (L > rb + 2 ? 4 * cap : cap)) L--;
+    *grid = (int)std::min<uint64_t>(1ULL << (n - L), (cap - 1) | 1);
     return L;
 }
 

@@ -67,6 +67,26 @@ def test_phase_odd_rows(n, bits):
 
 
 @pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
+@pytest.mark.parametrize("n", [16, 20, 22])
+def test_phase_of_single_factors(n, dtype):
+    """Factors on a chunk's own bits, above them and across: chunks that none reaches stay as they are."""
+    psi = rounded(random_state(n, n), dtype)
+    h = qs.qs_alloc(n, dtype)
+    try:
+        for bits in [(0,), (9,), (10,), (13,), (n - 1,), (1, 3), (2, n - 1), (9, n - 2), (13, n - 1), (n - 2, n - 1)]:
+            coeff, edges = np.zeros(n, dtype=np.int64), [bits] if len(bits) == 2 else []
+            coeff[bits[0]] = 0 if edges else 3
+            ref = psi.copy()
+            sim.apply_phase(ref, coeff, edges)
+            qs.qs_set_amplitudes(h, psi)
+            qs.qs_apply_phase(h, coeff, edges)
+            out = qs.qs_get_amplitudes(h)
+            assert np.all(np.abs(out - ref) <= 8 * EPS[dtype] * np.abs(psi)), bits
+    finally:
+        qs.qs_free(h)
+
+
+@pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
 @pytest.mark.parametrize("n,k", [(1, 1), (2, 2), (8, 3), (9, 9), (10, 1), (14, 12), (19, 6), (20, 12), (23, 5)])
 def test_table_rows_and_chunks(dtype, n, k):
     qubits, d = random_qubits(n, k, 5 * n + k), random_diag(k, k)
@@ -101,11 +121,12 @@ def device_ms(calls, reps=20):
     return out
 
 
-@pytest.mark.parametrize("q", [5, 8, 9, 12, 24])
+@pytest.mark.parametrize("q", [5, 8, 9, 12, 13, 24])
 def test_one_t_gate_costs_no_more_than_the_whole_state(q):
     """complex128: a T gate off the lanes' bits turns half of the amplitudes, so it takes no
     longer than one on bit 0, which reads and writes every sector (it took 1.6 to 1.8
-    times as long where the FP64 pipe was given the other half as well)."""
+    times as long where the FP64 pipe was given the other half as well, or where half of
+    the blocks had no chunk with work)."""
     n = 25
     h = qs.qs_alloc(n, qs.QS_C128)
     try:
