@@ -22,14 +22,16 @@
 // pipe; one cluster of CTAs per circuit before): 26.3 -> 6.0 ms, two thirds of the
 // issue slots used, two thirds of them by FMAs.  What the kernel holds across an op
 // has to stay out of the registers (spills inside the rows: 6.9 ms).  A plain circuit
-// of 83 gates on 16 qubits, complex128: 320 -> 98 us (a sweep per gate before); there
+// of 83 gates on 16 qubits, complex128: 320 -> 90 us (a sweep per gate before); there
 // a chunk has 512 amplitudes and the instructions' latency shows, so gates that are one
-// factor of a phase product visit just the amplitudes they turn (115 us with an exponent
-// for every amplitude).
+// factor of a phase product visit just the amplitudes they turn (17 us more with an
+// exponent for every amplitude), and even turns have loops without the FP64 pipe (97 us
+// without those; 24 qubits, a CZ of a pass 37 -> 11 us, an S gate 70 -> 15).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "qs_device.cuh"
@@ -297,11 +299,17 @@ __device__ __forceinline__ void phase_chunk(typename cplx<R>::t *sm, int W, cons
         }
         return;
     }
-    for (int r = 0; r < rows; r++) {
-        const int m = (mc + row_m[r] + 4 * __popcll(xc & row_M[r])) & 7;
-        C *p = sm + place<R>(((uint32_t)r << cb) | col);
-        if (m && in) *p = qsd::rotate8<C, R>(*p, m);
-    }
+    auto each_row = [&](auto odd) {
+        for (int r = 0; r < rows; r++) {
+            const int m = (mc + row_m[r] + 4 * __popcll(xc & row_M[r])) & 7;
+            C *p = sm + place<R>(((uint32_t)r << cb) | col);
+            if (m && in) *p = decltype(odd)::value ? qsd::rotate8<C, R>(*p, m) : qsd::quarter_turns<C>(*p, m >> 1);
+        }
+    };
+    // (complex128: a loop of their own for even exponents; a branch around an eighth turn alone
+    // is made into predicates, and the FP64 pipe takes those instructions too)
+    if (sizeof(R) == 4 || c0) each_row(std::true_type{});
+    else each_row(std::false_type{});
 }
 
 // One factor of a phase op by itself (a T-type gate on one qubit, a CZ): the
@@ -315,13 +323,17 @@ __device__ __forceinline__ void turn_chunk(typename cplx<R>::t *sm, int W, int k
         const uint32_t lo = l & ((1u << q) - 1u);
         return ((l ^ lo) << 1) | lo | 1u << q;
     };
-    for (uint32_t h = threadIdx.x; h < (1u << (W - k)); h += T) {
-        uint32_t l = h;
-        if (k > 0) l = with_bit(l, q0);
-        if (k > 1) l = with_bit(l, q1);
-        C *p = sm + place<R>(l);
-        *p = qsd::rotate8<C, R>(*p, c);
-    }
+    auto each = [&](auto odd) {
+        for (uint32_t h = threadIdx.x; h < (1u << (W - k)); h += T) {
+            uint32_t l = h;
+            if (k > 0) l = with_bit(l, q0);
+            if (k > 1) l = with_bit(l, q1);
+            C *p = sm + place<R>(l);
+            *p = decltype(odd)::value ? qsd::rotate8<C, R>(*p, c) : qsd::quarter_turns<C>(*p, c >> 1);
+        }
+    };
+    if (sizeof(R) == 4 || (c & 1)) each(std::true_type{});   // two loops as in phase_chunk
+    else each(std::false_type{});
 }
 
 __device__ __forceinline__ void copy16(uint32_t dst, const void *src)

@@ -76,3 +76,43 @@ def test_batches_from_zero_equal_sweeps(dtype, sizes):
         qs.qs_batch_free(b)
         for sc in scheds:
             qs.qs_schedule_free(sc)
+
+
+def run_ms(h, n, ops, timed=False, reps=10):
+    """Best time of qs_run_circuit on these ops; timed: of the ops as one sweep each."""
+    torch = pytest.importorskip("torch")
+    sched = qs.qs_schedule_from_ops(n, ops)
+    best = float("inf")
+    try:
+        for _ in range(5):
+            if timed:
+                ms = np.sum(np.maximum(qs.qs_run_circuit_timed(h, sched), 0))
+            else:
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                a.record()
+                for _ in range(reps):
+                    qs.qs_run_circuit(h, sched)
+                b.record()
+                b.synchronize()
+                ms = a.elapsed_time(b) / reps
+            best = min(best, ms)
+    finally:
+        qs.qs_schedule_free(sched)
+    return best
+
+
+def turn(n, q, eighths):
+    return (qs.QS_OP_PHASE, [], eighths * np.eye(n, dtype=np.int64)[q])
+
+
+def test_even_turns_leave_the_fp64_pipe_alone():
+    """complex128: an S gate in a pass swaps and negates, a T gate is four FP64 operations an
+    amplitude; a pass of S gates took as long as one of T gates where both went to that pipe."""
+    n = 23
+    h = qs.qs_alloc(n, qs.QS_C128)
+    try:
+        qs.qs_init_uniform(h)
+        s, t = [run_ms(h, n, [turn(n, q, e) for q in range(20)]) for e in (2, 1)]
+    finally:
+        qs.qs_free(h)
+    assert s <= 0.75 * t
