@@ -336,8 +336,14 @@ int launch_dense_t(qs_state *s, const int *q, const void *U)
     uint64_t groups = 1ULL << (s->n - K);
     const int block = 128;
     int grid = grid_for(groups, block, 8);
-    const cudaError_t e = launch_sweep(s, k_dense<R, K>, grid, block, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), groups,
-                                       t, reinterpret_cast<const R *>(U));
+    // An SM holds up to 16 of these blocks.  Started early they pile up on the SMs that are
+    // free first, which costs more than the start gains unless the sweep is little more
+    // than a launch.  Three table diagonals and three clusters in turn, us, early start and
+    // not: complex128 k = 3, 14 qubits 39, 45; 16 qubits 201, 45; 27 qubits k = 1 13.9,
+    // 8.6 ms.  complex64 k = 1, 20 qubits 22, 29; k = 4, 16 qubits 20, 24, 18 qubits 38, 27.
+    const bool chain = s->chain && s->n <= (sizeof(R) == 8 ? 14 : K <= 2 ? 20 : 16);
+    const cudaError_t e = launch_sweep(s, chain, k_dense<R, K>, grid, block, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp),
+                                       groups, t, reinterpret_cast<const R *>(U));
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_dense launch: %s", cudaGetErrorString(e));
 }
 
@@ -401,7 +407,7 @@ static cudaError_t launch_diag_r(qs_state *s, const int *dev_qubits, int k, cons
 {
     int grid;
     const int L = diag_chunk<R>(s->n, &grid);
-    return launch_sweep(s, k_diag<R>, grid, kDiagThreads, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, k,
+    return launch_sweep(s, s->chain, k_diag<R>, grid, kDiagThreads, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L, k,
                         dev_qubits, reinterpret_cast<const R *>(dev_table));
 }
 
@@ -410,7 +416,9 @@ static cudaError_t launch_phase_r(qs_state *s, const void *dev_phase, int n_act)
 {
     int grid;
     const int L = diag_chunk<R>(s->n, &grid);
-    return launch_sweep(s, k_phase<R>, grid, kDiagThreads, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L,
+    // (complex128 states beyond L2 lose by an early start after a tensor-core sweep: 27 qubits,
+    // three of each in turn, 5.47 ms, without 5.18)
+    return launch_sweep(s, s->chain && (sizeof(R) == 4 || s->n <= 23), k_phase<R>, grid, kDiagThreads, 0, reinterpret_cast<typename cplx<R>::t *>(s->amp), s->n, L,
                         (const qs_phase_dev *)dev_phase, n_act);
 }
 

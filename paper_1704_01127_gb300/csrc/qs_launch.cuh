@@ -20,8 +20,13 @@ namespace {
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// chain: s->chain, or false for a kernel that must not start early.  The blocks that do
+// start go to the SMs that are free first, as many as fit there, and stay: a kernel
+// with a fixed number of blocks for the whole GPU is spread evenly only if no SM can
+// hold more than its share of them (the tensor-core sweeps' shared memory, the phase
+// sweep's registers), or if it has no work to speak of.
 template <typename... P, typename... A>
-cudaError_t launch_sweep(const qs_state *s, void (*kernel)(P...), int grid, int block, size_t smem, A... args)
+cudaError_t launch_sweep(const qs_state *s, bool chain, void (*kernel)(P...), int grid, int block, size_t smem, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -32,7 +37,7 @@ cudaError_t launch_sweep(const qs_state *s, void (*kernel)(P...), int grid, int 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = s->chain ? 1 : 0;
+    cfg.numAttrs = chain ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

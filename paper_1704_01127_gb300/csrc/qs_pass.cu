@@ -512,7 +512,7 @@ int launch_pass_r(qs_state *s, const qs_pass &ps)
 {
     static bool ready[64] = {};
     if (int rc = allow_smem(k_pass<R>, pass_smem<R>(kPassBits<R>), ready)) return rc;
-    const cudaError_t e = launch_sweep(s, k_pass<R>, 1 << (s->n - ps.W), kOneThreads<R>, pass_smem<R>(ps.W), ps,
+    const cudaError_t e = launch_sweep(s, s->chain, k_pass<R>, 1 << (s->n - ps.W), kOneThreads<R>, pass_smem<R>(ps.W), ps,
                                        reinterpret_cast<typename cplx<R>::t *>(s->amp));
     return e == cudaSuccess ? QS_OK : qs_fail(QS_ECUDA, "k_pass launch: %s", cudaGetErrorString(e));
 }

@@ -1190,11 +1190,11 @@ int qs_launch_dense5_tc(qs_state *s, const int *sorted_qubits, const void *dev_p
     cudaError_t e;
     if (c64) {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms * 2);
-        e = launch_sweep(s, c64s[fold][form], grid, form == 2 ? 2 * kRows : kRows, kSmemF32, (float2 *)s->amp,
+        e = launch_sweep(s, s->chain, c64s[fold][form], grid, form == 2 ? 2 * kRows : kRows, kSmemF32, (float2 *)s->amp,
                          groups, t, (const float *)dev_pack, post, status);
     } else {
         int grid = (int)std::min<uint64_t>(tiles, (uint64_t)sms);
-        e = launch_sweep(s, c128, grid, kC128Threads, kSmemC128Pipe, (double2 *)s->amp, groups, t,
+        e = launch_sweep(s, s->chain, c128, grid, kC128Threads, kSmemC128Pipe, (double2 *)s->amp, groups, t,
                          (const uint8_t *)dev_pack, post, status);
     }
     // amplitudes on the padding targets of an embedded cluster keep their

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import paper_1704_01127_gb300.qs as qs
-from inputs import random_phase_poly, random_qubits, random_state, random_unitary
+from inputs import random_diag, random_phase_poly, random_qubits, random_state, random_unitary
 
 pytestmark = pytest.mark.gpu
 
@@ -116,3 +116,19 @@ def test_even_turns_leave_the_fp64_pipe_alone():
     finally:
         qs.qs_free(h)
     assert s <= 0.75 * t
+
+
+@pytest.mark.parametrize("dtype,n,k", [(qs.QS_C128, 16, 3), (qs.QS_C128, 16, 4), (qs.QS_C128, 20, 1), (qs.QS_C128, 24, 1),
+                                       (qs.QS_C64, 23, 2)])
+def test_sweeps_in_turn_cost_no_more_than_one_by_one(dtype, n, k):
+    """Table diagonals and clusters in turn: blocks of a sweep that starts early pile up on a few SMs
+    (2 to 4 times the time in complex128, 1.3 in complex64)."""
+    ops = [(qs.QS_OP_DIAG, [0, 3, n - 1], random_diag(3, 1)), (qs.QS_OP_DENSE, [2, 5, 8, 7, n - 1][-k:], random_unitary(k, k))] * 3
+    h = qs.qs_alloc(n, dtype)
+    try:
+        qs.qs_set_path(h, qs.QS_PATH_CUDA_CORES)
+        qs.qs_init_uniform(h)
+        together, apart = run_ms(h, n, ops), run_ms(h, n, ops, timed=True)
+    finally:
+        qs.qs_free(h)
+    assert together <= 1.1 * apart
