@@ -777,11 +777,49 @@ int launch_op_dense(qs_state *s, const qs_dev_sched &d, size_t i, const qs_op_ho
     return qs_launch_dense(s, op.qubits, op.k, data, nullptr);
 }
 
+// Whether a pass is faster than its ops as one sweep each.  Up to 4 MB of state always (every
+// sweep is a launch there).  Above, a pass pays for its own read and write of the state
+// and its row tables, and saves per op, in microseconds with M = 2^20 amplitudes (fitted to
+// runs of 2, 3 and 4 equal ops, complex64 20 to 28 and complex128 19 to 27 qubits):
+//   complex64   pass 5 + 3.4 M; a dense op saves 3 + 1.6 M, one factor of a phase op
+//               2.2 + (2.2 f - 0.1) M, a longer phase op 2 - M
+//   complex128  pass 3 + 10.4 M; a dense op saves 1 (it is bound by the FP64 pipe either
+//               way), a T gate 3 + 0.3 M, another factor 3.5 + (4.5 f - 0.6) M, a longer
+//               phase op 2 - 2.5 M
+// where f is the part of the state that the factor's sweep touches (bits below a 64-byte
+// piece save nothing), and a state in L2 has sweeps of half the traffic's time.  24 qubits
+// complex128: two phase ops of 24 terms 183 us as sweeps, 462 as a pass, two CZs on high
+// qubits 37 and 194; 27 qubits complex64: four CZs on low qubits 1366 and 640, two phase
+// ops 686 and 1275.  Circuits gate by gate are passes at every size.
+bool pass_pays(const qs_state *s, const qs_pass &p)
+{
+    const bool c64 = s->dtype == QS_C64;
+    const double bytes = (c64 ? 8.0 : 16.0) * std::ldexp(1.0, s->n), M = std::ldexp(1.0, s->n - 20);
+    if (bytes <= (4 << 20)) return true;
+    const double l2 = bytes <= (96 << 20) ? 0.5 : 1.0;
+    double gain = 0;
+    for (int i = 0; i < p.n_ops; i++) {
+        const qs_pass_op &op = p.op[i];
+        if (op.kind == QS_OP_DENSE) {
+            gain += c64 ? 3 + 1.6 * l2 * M : 1;
+        } else if (op.kind == QS_OP_PHASE) {
+            gain += c64 ? 2 - M : 2 - 2.5 * M;
+        } else {
+            // the factor's index bits: op.data outside the chunk, op.q among its local bits
+            double f = std::ldexp(1.0, -__builtin_popcountll(op.data));
+            for (int j = 0; j < op.k; j++)
+                if (op.q[j] >= (c64 ? 3 : 2)) f /= 2;   // (the lowest local bits are the lowest index bits)
+            gain += c64 ? 2.2 + (2.2 * f - 0.1) * l2 * M : op.n_act & 1 ? 3 + 0.3 * M : 3.5 + (4.5 * f - 0.6) * l2 * M;
+        }
+    }
+    return gain > (c64 ? 5 + 3.4 * M : 3 + 10.4 * M);
+}
+
 // Ops i, i + 1, ... that run on the CUDA cores as passes (qs_pass.cu), *done of
-// them: two or more ops per read and write of the state, a pass of one op as its
-// own sweep.  A chunk has 2^(n-7) amplitudes, within the kernel's 2^8 .. 2^13
-// (complex64) or 2^12: 128 chunks at least, a CTA each, so a small state still
-// fills the GPU.
+// them: two or more ops per read and write of the state, a pass of one op, or one
+// that does not pay, as sweeps.  A chunk has 2^(n-7) amplitudes, within the kernel's
+// 2^8 .. 2^13 (complex64) or 2^12: 128 chunks at least, a CTA each, so a small state
+// still fills the GPU.
 int run_passes(qs_state *s, const qs_schedule *sc, const qs_dev_sched &d, size_t i, size_t *done)
 {
     *done = 0;
@@ -798,16 +836,19 @@ int run_passes(qs_state *s, const qs_schedule *sc, const qs_dev_sched &d, size_t
     if (in.size() < 2) return QS_OK;
     const int wmax = std::max(8, std::min(qs_pass_bits(s->dtype), s->n - 7));
     for (const qs_pass &p : qs_plan_passes(s->n, s->dtype, wmax, in, false)) {
-        int rc;
-        if (p.n_ops > 1) {
-            rc = qs_launch_pass(s, p);
-        } else {
-            const qs_pass_in &op = in[p.first_op];
-            const void *data = (const void *)(uintptr_t)op.data;
-            rc = op.kind == QS_OP_DENSE ? qs_launch_dense(s, op.qubits, op.k, data, nullptr) : qs_launch_phase(s, data, op.n_act);
+        if (p.n_ops > 1 && pass_pays(s, p)) {
+            if (int rc = qs_launch_pass(s, p)) return rc;
+            s->chain = !s->pair_sweeps;
+            continue;
         }
-        if (rc) return rc;
-        s->chain = !s->pair_sweeps;
+        for (int j = p.first_op; j < p.first_op + p.n_ops; j++) {
+            const qs_pass_in &op = in[j];
+            const void *data = (const void *)(uintptr_t)op.data;
+            if (int rc = op.kind == QS_OP_DENSE ? qs_launch_dense(s, op.qubits, op.k, data, nullptr)
+                                                : qs_launch_phase(s, data, op.n_act))
+                return rc;
+            s->chain = !s->pair_sweeps;
+        }
     }
     *done = in.size();
     return QS_OK;

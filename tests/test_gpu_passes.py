@@ -132,3 +132,25 @@ def test_sweeps_in_turn_cost_no_more_than_one_by_one(dtype, n, k):
     finally:
         qs.qs_free(h)
     assert together <= 1.1 * apart
+
+
+def few(kind, n):
+    if kind == "phases":
+        return [(qs.QS_OP_PHASE, *reversed(random_phase_poly(n, n, i))) for i in (1, 2)]
+    if kind == "clusters and a phase":
+        return few("phases", n)[:1] + [(qs.QS_OP_DENSE, [n - 1], random_unitary(1, 1))]
+    return [(qs.QS_OP_PHASE, [pair], np.zeros(n, dtype=np.int64)) for pair in ((n - 2, n - 1), (n - 4, n - 3))]
+
+
+@pytest.mark.parametrize("kind", ["phases", "pairs", "clusters and a phase"])
+@pytest.mark.parametrize("dtype,n", [(qs.QS_C128, 21), (qs.QS_C128, 24), (qs.QS_C64, 24), (qs.QS_C64, 27)])
+def test_few_ops_cost_no_more_than_their_sweeps(dtype, n, kind):
+    """Two ops that a pass would not pay for (1.4 to 5 times the time of their sweeps)."""
+    h = qs.qs_alloc(n, dtype)
+    try:
+        qs.qs_set_path(h, qs.QS_PATH_CUDA_CORES)
+        qs.qs_init_uniform(h)
+        together, apart = run_ms(h, n, few(kind, n)), run_ms(h, n, few(kind, n), timed=True)
+    finally:
+        qs.qs_free(h)
+    assert together <= 1.1 * apart
