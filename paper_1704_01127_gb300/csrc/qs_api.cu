@@ -1123,9 +1123,11 @@ int gather_impl(qs_state *s, const uint64_t *idx, int64_t count, double *out)
     cudaStream_t st = (cudaStream_t)s->stream;
     const bool moved = !qs_loc_identity(s);
     void *scr = nullptr;
-    if (count > 0 && qs_state_scratch(s, sizeof(double2) * (size_t)std::min(count, kGatherChunk), &scr)) {
-        // no room on the device: one copy per index
-        cudaGetLastError();
+    // one copy per index: for one (15 us, a launch and a copy take 21), for up to four on a state
+    // that has no scratch yet (60 us, its allocation alone takes 90), and without room for it
+    const bool copies = count <= (s->scratch ? 1 : 4);
+    if (copies || qs_state_scratch(s, sizeof(double2) * (size_t)std::min(count, kGatherChunk), &scr)) {
+        if (!copies) cudaGetLastError();
         for (int64_t j = 0; j < count; j++) {
             C a;
             QS_CUDA(cudaMemcpyAsync(&a, (const C *)s->amp + (moved ? qs_loc_index(s, idx[j]) : idx[j]), sizeof(C),

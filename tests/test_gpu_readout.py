@@ -1,6 +1,8 @@
 """Results read out: amplitudes by index (more and fewer indices than one launch
 takes, none, one out of range, qubits moved to other bits) and complex128
 probabilities over the whole range of doubles."""
+import time
+
 import numpy as np
 import pytest
 
@@ -11,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("dtype", [qs.QS_C128, qs.QS_C64])
-@pytest.mark.parametrize("count", [0, 1, 31, 480, 481, 65536, 65536 + 481])
+@pytest.mark.parametrize("count", [0, 1, 4, 5, 31, 480, 481, 65536, 65536 + 481])
 def test_gather(dtype, count):
     n = 12
     psi = random_state(n, 3).astype(np.complex64).astype(np.complex128)
@@ -19,11 +21,32 @@ def test_gather(dtype, count):
     try:
         qs.qs_set_amplitudes(h, psi)
         idx = rng(count).integers(0, 1 << n, count)
-        assert np.array_equal(qs.qs_get_amplitudes_at(h, idx), psi[idx])
+        for _ in range(2):   # before and after the state has its scratch
+            assert np.array_equal(qs.qs_get_amplitudes_at(h, idx), psi[idx])
+            qs.qs_norm(h)
         with pytest.raises(qs.QSError):
             qs.qs_get_amplitudes_at(h, np.append(idx, 1 << n))
     finally:
         qs.qs_free(h)
+
+
+def test_one_index_costs_less_than_a_gather():
+    """One amplitude is one copy; a launch and a copy took 1.4 times as long."""
+    h = qs.qs_alloc(12, qs.QS_C128)
+    try:
+        qs.qs_init_uniform(h)
+        qs.qs_norm(h)
+        best = []
+        for count in (1, 8):
+            idx, took = np.arange(count), []
+            for _ in range(200):
+                t = time.perf_counter()
+                qs.qs_get_amplitudes_at(h, idx)
+                took.append(time.perf_counter() - t)
+            best.append(np.median(took))
+    finally:
+        qs.qs_free(h)
+    assert best[0] <= 0.85 * best[1]
 
 
 def test_gather_after_remapped_circuit():
