@@ -142,7 +142,7 @@ struct StatsAcc {
     ff f0{0.f, 0.f}, f3{0.f, 0.f}, fent{0.f, 0.f};   // of the terms since the last fold()
     ff g0{0.f, 0.f}, g3{0.f, 0.f}, gent{0.f, 0.f};   // of those before
 
-    // After every kTerms amplitudes: their sums into the normalised ones.
+    // After every kTerms amplitudes or so: their sums into the normalised ones.
     static constexpr int kTerms = 16;
     template <int NSTAT>
     __device__ __forceinline__ void fold()
@@ -266,21 +266,23 @@ __device__ __forceinline__ void load_fflog(FFLogTable &lt)
 // Errors against exact sums at 28 qubits, relative: random amplitudes 3e-15 (p), 2e-15
 // (entropy), 6e-15 (p^2); equal amplitudes, whose rounding errors add up, up to 3e-14
 // (1.7e-11 without the sums of 16; 1.4e-13 with each term added to a normalised sum).
-// The sums of 16 cost 1% of the pass (complex64: 2%).  p below 2^-79
+// The sums of 16 cost 0.2% of the pass (complex64 beside the block sums, sums of 32: 0.7%),
+// within 48 registers: at 54, one block less per SM, 1%.  p below 2^-79
 // (where the low half of p's float-float form would leave the normal float
 // range) takes p ln p from the FP64 math library, and complex128 amplitudes of
 // 2^30 or more (unnormalised input) are summed in FP64 throughout; p below the
 // normal double range contributes less than 1e-305 and is left out.
+template <typename C> constexpr int kStatsAhead = sizeof(C) == 16 ? 4 : 8;   // loads in flight per thread
+
 template <typename C, int NSTAT>
-__global__ void k_stats_partial(const C *__restrict__ psi, uint64_t N, double *__restrict__ part)
+__global__ void __launch_bounds__(256, NSTAT == 4 ? 5 : 8) k_stats_partial(const C *__restrict__ psi, uint64_t N, double *__restrict__ part)
 {
-    constexpr bool c128 = sizeof(C) == 16;
     __shared__ __align__(16) FFLogTable lt;
     load_fflog<C, NSTAT>(lt);
     StatsAcc acc;
     // each thread loads kAhead amplitudes (block-strided, so every load of a
     // warp is contiguous) before it adds them up: more loads in flight
-    constexpr int kAhead = c128 ? 4 : 8;
+    constexpr int kAhead = kStatsAhead<C>;
     constexpr uint32_t kBatches = StatsAcc::kTerms / kAhead;
     const uint64_t span = (uint64_t)blockDim.x * kAhead;
     uint32_t batch = 0;
@@ -469,8 +471,8 @@ __device__ __forceinline__ double piece_sum(const double2 *__restrict__ p, F see
 // (One piece after another: unrolled altogether, with the statistics, the code leaves
 // the instruction cache.)  With the statistics, 29 qubits complex64: 3.33 ms as one
 // 32-value run per lane, 1.71 ms.
-template <typename C, typename F, typename G>
-__device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen, G piece_seen)
+template <typename C, typename F>
+__device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen)
 {
     using V = std::conditional_t<sizeof(C) == 8, float4, double2>;
     constexpr int kPieces = sizeof(C) == 8 ? 2 : 4;
@@ -483,7 +485,6 @@ __device__ __forceinline__ double block_sum(const C *__restrict__ psi, F seen, G
 #pragma unroll
         for (int j = 0; j + 1 < kPieces; j++) v[j] = v[j + 1];
         v[kPieces - 1] = piece_sum(p + 256 * i, seen);
-        piece_seen();
     }
     halve<kPieces>(v, 8);
     if constexpr (kPieces == 4) halve<2>(v, 16);
@@ -502,7 +503,7 @@ k_block_sums(const C *__restrict__ psi, uint64_t nb, double *__restrict__ out)
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t b = warp; b < nb; b += nwarps) {
-        const double v = block_sum(psi + b * 1024, [](const C &) {}, [] {});
+        const double v = block_sum(psi + b * 1024, [](const C &) {});
         if ((threadIdx.x & 31) == 0) out[b] = v;
     }
 }
@@ -521,8 +522,8 @@ k_block_sums_stats(const C *__restrict__ psi, uint64_t nb, double *__restrict__ 
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t b = warp; b < nb; b += nwarps) {
-        const double v = block_sum(
-            psi + b * 1024, [&](const C &a) { acc.add<4>(a, lt); }, [&] { acc.fold<4>(); });   // 16 amplitudes a piece
+        const double v = block_sum(psi + b * 1024, [&](const C &a) { acc.add<4>(a, lt); });
+        acc.fold<4>();   // 32 terms: without low parts of their own they round half as much as complex128's
         if ((threadIdx.x & 31) == 0) out[b] = v;
     }
     acc.partials<4>(part);
@@ -926,16 +927,24 @@ __global__ void k_draw_run(const C *__restrict__ psi, const double *__restrict__
     }
 }
 
+// 16 blocks of 256 per SM: the float-float work is latency-bound at lower occupancy
+// (30 qubits: 7.35 ms with 4 per SM, 6.64 ms with 16).  No block without an amplitude: its
+// closing sums are FP64 work all the same (19 qubits: complex64 54 -> 31 us a call, complex128
+// 56 -> 43).
 constexpr int kStatsBlocksPerSM = 16;
+
+template <typename C>
+int stats_grid(uint64_t N, int per_sm)
+{
+    constexpr uint64_t span = 256 * kStatsAhead<C>;
+    return (int)std::min<uint64_t>((N + span - 1) / span, (uint64_t)sm_count_dev() * per_sm);
+}
 
 template <typename C>
 int stats_impl(qs_state *s, double *out, int nstat)
 {
     uint64_t N = 1ULL << s->n;
-    const int block = 256;
-    // 16 blocks of 256 per SM: the float-float work is latency-bound at lower
-    // occupancy (30 qubits: 7.35 ms with 4 per SM, 6.64 ms with 16)
-    int grid = (int)std::min<uint64_t>((N + block - 1) / block, (uint64_t)sm_count_dev() * kStatsBlocksPerSM);
+    const int block = 256, grid = stats_grid<C>(N, kStatsBlocksPerSM);
     void *scr = nullptr;
     int rc = qs_state_scratch(s, sizeof(double) * (size_t)(grid + 1) * 4, &scr);
     if (rc) return rc;
@@ -1005,7 +1014,7 @@ int sample_impl(qs_state *s, uint64_t seed, int64_t m, uint64_t *out, double *st
         if (int rc = ensure_fflog(st)) return rc;
     if (beside)
         if (int rc = side_stream(s, &ss)) return rc;
-    const int sgrid = (int)std::min<uint64_t>((N + 255) / 256, (uint64_t)sms * kStatsBlocksPerSM);   // stats_impl's grid
+    const int sgrid = stats_grid<C>(N, kStatsBlocksPerSM);   // stats_impl's
     const size_t stats_bytes = beside ? sizeof(double) * ((size_t)sgrid + 1) * 4 : 0;
     const size_t m_slots = (size_t)std::max<int64_t>(m, 1);
     size_t bytes = sizeof(double) * (2 * nb + 2 * ns) + sizeof(uint64_t) * m_slots;
@@ -1615,8 +1624,7 @@ int stats_static_impl(const void *amp, int n, void *stream, double *out)
     if (rc) return rc;
     const uint64_t N = 1ULL << n;
     const int block = 256;
-    int grid = (int)std::min<uint64_t>((N + block - 1) / block, (uint64_t)sm_count_dev() * 4);
-    grid = std::min(grid, kStaticStatsBlocks);
+    const int grid = std::min(stats_grid<C>(N, 4), kStaticStatsBlocks);
     double *part = scr, *res = scr + 4 * kStaticStatsBlocks;
     cudaStream_t st = (cudaStream_t)stream;
     if ((rc = ensure_fflog(st))) return rc;
