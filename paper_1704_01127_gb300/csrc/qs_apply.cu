@@ -384,9 +384,11 @@ int qs_launch_dense(qs_state *s, const int *sorted_qubits, int k, const void *de
                                : launch_dense_r<float>(s, sorted_qubits, k, dev_matrix);
 }
 
-// Chunk bits of a diagonal sweep: up to 32 rows, fewer (4 at least) where a block would
-// get less than four chunks, and fewer still where the chunks would not fill the GPU
-// (complex128 table, 23 qubits: 79 us with 1.7 chunks a block, 72 so).
+// Chunk bits of a diagonal sweep: up to 32 rows, fewer (8) where a block would get less
+// than four chunks, 4 where less than two, and fewer still where the chunks would not
+// fill the GPU (complex128 table, 23 qubits: 79 us with 1.7 chunks a block, 72 so; a
+// chunk of few rows costs a phase op its terms: complex64, 23 qubits, 25.3 us with 4 rows,
+// 22.8 with 8).
 // *grid: its blocks.  Their number is odd where blocks take several chunks: a block's
 // chunks then differ in every bit of their number.  (With an even one the blocks split
 // by the lowest bit, and one T gate or CZ on that qubit left half of them without
@@ -397,7 +399,7 @@ static int diag_chunk(int n, int *grid)
     const int rb = std::min(n, kDiagRowBits<R>);
     const uint64_t cap = (uint64_t)sm_count() * 4;
     int L = std::min(n, rb + 5);
-    while (L > rb && (1ULL << (n - L)) < (L > rb + 2 ? 4 * cap : cap)) L--;
+    while (L > rb && (1ULL << (n - L)) < (L > rb + 3 ? 4 : L > rb + 2 ? 2 : 1) * cap) L--;
     *grid = (int)std::min<uint64_t>(1ULL << (n - L), (cap - 1) | 1);
     return L;
 }
