@@ -445,16 +445,23 @@ typedef struct {
 int qs_schedule_op(const qs_schedule *sc, int i, qs_op_info *info, double *matrix,
                    int32_t *gate_idx, int32_t *coeff, int32_t *edges);
 
-/* Apply every op of a schedule, in order, to the state (one HBM sweep per op). */
+/* Apply every op of a schedule, in order, to the state: one HBM sweep per op,
+ * except that a phase op may run inside the tensor-core sweep before it
+ * (qs_set_phase_fold), two clusters may share one (qs_set_pair_sweeps), and
+ * consecutive CUDA-core ops share one read and write of the state (a pass)
+ * where that is faster, with the same bits.  A sweep may start while the one
+ * before it finishes. */
 int qs_run_circuit(qs_state *s, const qs_schedule *sc);
 
-/* As qs_run_circuit, recording a CUDA event before and after every op on the
- * state's stream; waits for the stream and writes op i's device time in
- * milliseconds to op_ms[i] (host, qs_schedule_num_ops entries).  An op that
- * runs inside the sweep before it launches nothing and gets op_ms[i] = -1:
- * a phase op folded into a tensor-core sweep (qs_set_phase_fold) or the
- * second cluster of a pair sweep (qs_set_pair_sweeps); its time is part of
- * the previous op's. */
+/* The same result, bit for bit, with every op run by itself as its own sweep
+ * (no passes, no early starts): records a CUDA event before and after every op
+ * on the state's stream, waits for the stream and writes op i's device time in
+ * milliseconds to op_ms[i] (host, qs_schedule_num_ops entries).  Where
+ * qs_run_circuit joins ops into passes or overlaps sweeps it takes less than
+ * the sum.  An op that runs inside the sweep before it launches nothing and
+ * gets op_ms[i] = -1: a phase op folded into a tensor-core sweep
+ * (qs_set_phase_fold) or the second cluster of a pair sweep
+ * (qs_set_pair_sweeps); its time is part of the previous op's. */
 int qs_run_circuit_timed(qs_state *s, const qs_schedule *sc, float *op_ms);
 
 /* ------------------------------------------------------------------------

@@ -1,4 +1,4 @@
-"""Batched persistent kernel: bit-exact against single-state CUDA-core runs of
+"""Batches (one launch per pass): bit-exact against single-state CUDA-core runs of
 the same schedules, within tolerance of the oracle, for every launch
 configuration and through CUDA-graph replay."""
 import numpy as np
@@ -123,8 +123,8 @@ def test_batch_rejects_bad_config(torch_stream):
 
 
 def test_batch_512_circuits_autotuned_graph(torch_stream):
-    """Config 4 at its stated size: all 512 circuits (seeds 0..511) in one
-    persistent launch replayed from a CUDA graph with the autotuner's choice;
+    """Config 4 at its stated size: all 512 circuits (seeds 0..511), one
+    launch per pass, replayed from a CUDA graph with the autotuner's choice;
     every circuit's norm within 1e-5, and 23 circuits spread over the seeds
     (every grid) against the oracle within 2e-6."""
     circs = batch_circuits(range(512))
