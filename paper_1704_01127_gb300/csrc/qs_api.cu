@@ -135,6 +135,10 @@ __global__ void k_fflog_init() { ff_log_table_init(g_fflog); }
 // p ln p by the FP64 math library, out of the way of the common cases' code
 __device__ __noinline__ double p_ln_p_rare(double p) { return p * log(p); }
 
+// Terms of a sum before it goes into the normalised one.  complex64's have no low parts of
+// their own and round half as much (32 qubits: 6.06 ms without, 6.15 with 16, 6.04 with 32).
+template <typename C> constexpr int kStatsTerms = sizeof(C) == 16 ? 16 : 32;
+
 // Per-thread sums of the statistics; add() takes one amplitude, partials()
 // reduces the block (every thread of the block calls it).
 struct StatsAcc {
@@ -142,8 +146,7 @@ struct StatsAcc {
     ff f0{0.f, 0.f}, f3{0.f, 0.f}, fent{0.f, 0.f};   // of the terms since the last fold()
     ff g0{0.f, 0.f}, g3{0.f, 0.f}, gent{0.f, 0.f};   // of those before
 
-    // After every kTerms amplitudes or so: their sums into the normalised ones.
-    static constexpr int kTerms = 16;
+    // After every kStatsTerms amplitudes: their sums into the normalised ones.
     template <int NSTAT>
     __device__ __forceinline__ void fold()
     {
@@ -262,12 +265,12 @@ __device__ __forceinline__ void load_fflog(FFLogTable &lt)
 // 1/64 of its rate): complex128 amplitudes are split into float-float by bit
 // manipulation (the lowest 29 of their 53 bits rounded to 24), complex64 ones give
 // p rounded to 32 bits.  p, p^2 and p ln p (table-driven log, ff_p_ln_p) are summed
-// per thread in float-float, in sums of 16 terms that go into normalised ones.
+// per thread in float-float, in sums of 16 or 32 terms that go into normalised ones.
 // Errors against exact sums at 28 qubits, relative: random amplitudes 3e-15 (p), 2e-15
 // (entropy), 6e-15 (p^2); equal amplitudes, whose rounding errors add up, up to 3e-14
 // (1.7e-11 without the sums of 16; 1.4e-13 with each term added to a normalised sum).
-// The sums of 16 cost 0.2% of the pass (complex64 beside the block sums, sums of 32: 0.7%),
-// within 48 registers: at 54, one block less per SM, 1%.  p below 2^-79
+// The sums of 16 (complex64: 32) cost at most 0.7% of a pass, within 48 registers: at 54,
+// one block less per SM, 1%.  p below 2^-79
 // (where the low half of p's float-float form would leave the normal float
 // range) takes p ln p from the FP64 math library, and complex128 amplitudes of
 // 2^30 or more (unnormalised input) are summed in FP64 throughout; p below the
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(256, NSTAT == 4 ? 5 : 8) k_stats_partial(const
     // each thread loads kAhead amplitudes (block-strided, so every load of a
     // warp is contiguous) before it adds them up: more loads in flight
     constexpr int kAhead = kStatsAhead<C>;
-    constexpr uint32_t kBatches = StatsAcc::kTerms / kAhead;
+    constexpr uint32_t kBatches = kStatsTerms<C> / kAhead;
     const uint64_t span = (uint64_t)blockDim.x * kAhead;
     uint32_t batch = 0;
     for (uint64_t base = (uint64_t)blockIdx.x * span; base < N; base += (uint64_t)gridDim.x * span) {
@@ -523,7 +526,7 @@ k_block_sums_stats(const C *__restrict__ psi, uint64_t nb, double *__restrict__ 
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t b = warp; b < nb; b += nwarps) {
         const double v = block_sum(psi + b * 1024, [&](const C &a) { acc.add<4>(a, lt); });
-        acc.fold<4>();   // 32 terms: without low parts of their own they round half as much as complex128's
+        acc.fold<4>();   // 32 terms
         if ((threadIdx.x & 31) == 0) out[b] = v;
     }
     acc.partials<4>(part);

@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 # is at most k 2^-24 of the sum, so its 16 roundings come to 94 2^-48 of the sum at most
 # (the sum of k^2 / 16); a term itself errs by 4 2^-48, p^2 and p ln p by about 8 2^-48; and
 # the total of T such sums by T 2^-48.  1725 terms a thread (28 qubits, 608 blocks):
-# (94 + 8 + 108) 2^-48 = 7.5e-13.  (complex64 beside the draws' block sums: 32 terms, without
-# low parts of their own, so half of 358 2^-48.)
+# (94 + 8 + 108) 2^-48 = 7.5e-13.  complex64: 32 terms without low parts of their own, so half
+# of 358 2^-48 in the place of 94 2^-48: 8.4e-13 with 862 terms.
 BOUND = 1e-12
 
 
